@@ -15,120 +15,185 @@ __device__ __forceinline__ uint32_t combine(uint32_t x, uint32_t y) {
   return x + y;  // wraps modulo 2^32
 }
 
+template <int OP>
+__device__ __forceinline__ uint32_t combine3(uint32_t x, uint32_t y, uint32_t z) {
+  if constexpr (OP == 0) return __vimin3_u32(x, y, z);
+  return x + y + z;
+}
+
+// Barrier over the threads that compute cells (`count`, a multiple of 32).
+__device__ __forceinline__ void bar_step(int count) { asm volatile("bar.sync 1, %0;" ::"r"(count) : "memory"); }
+
+__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ void sts_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
 // RING = 0: read the table in global memory (window too large for shared memory).
 // RING = 1: a ring of R = 2^ring_log2 words indexed modulo R.
 // RING = 2: the same ring stored twice (word x at x and at x + R), so that the
 //           read of ST[i - a_j] is ring[(i mod R) + R - a_j] with no wrap:
 //           an add, a load and the operator per offset.
-// KREG: offsets held in registers (k <= kSdpMaxKRegs); KFULL: k == kSdpMaxKRegs
-// (no per-offset predicate).
-template <int OP, int RING, bool KREG, bool KFULL>
-__global__ void __launch_bounds__(1024) sdp_kernel(const SdpLaunchArgs args) {
+// KP: offsets held in registers (k <= KP); 0: offsets read from shared memory
+//     (k > kSdpMaxKRegs).  G: loads in flight together.  FULL: k == KP (no
+//     per-offset predicate).
+//
+// What bounds a step of W cells.  With many warps, shared-memory wavefronts:
+// k W / 32 of reads and W / 16 of the two stores, one per clock (k = 32, W =
+// 1024: 1088 of the 1290 clocks a step takes, data pipe 84 % busy, no bank
+// conflicts).  With few, the latency of loads, combination, store and
+// barrier.  Ring positions and displacements are byte addresses, so that a
+// read is an add and a load: as word indices, which the compiler scales again
+// at every read, a step took 1470 clocks.  Fewer loads in flight (G = 8
+// against 16 or 32) drain more evenly when the pipe is the limit, more of them
+// hide latency when it is not: k = 32, W = 64: 339, 296 and 280 clocks a step.
+// Reading the next step's far offsets (a_j >= 2 W) before the barrier was
+// slower at every size (W = 1024: 1750 clocks, W = 64: 385 against 225).
+template <int OP, int RING, int KP, int G, bool FULL>
+__global__ void __launch_bounds__(1024) sdp_kernel(const __grid_constant__ SdpLaunchArgs args) {
   extern __shared__ __align__(16) uint32_t sm[];
-  const int b = blockIdx.x;
-  SdpInstDev in = args.insts ? args.insts[b] : args.one;
-  uint32_t* st = args.st_off ? args.st_all + args.st_off[b] : in.st;
+  constexpr uint32_t kIdentity = OP == 0 ? 0xFFFFFFFFu : 0u;
+  const int tid = threadIdx.x;
+
+  SdpInstDev in = args.insts ? args.insts[blockIdx.x] : args.one;
+  uint32_t* st = args.st_off ? args.st_all + args.st_off[blockIdx.x] : in.st;
   const int64_t n = in.n;
   const int k = in.k;
-  const int tid = threadIdx.x;
   const int ring_log2 = args.ring_log2;
   const uint32_t R = RING ? (1u << ring_log2) : 0u;
   const uint32_t mask = R - 1u;
   uint32_t* ring = sm;
-  int32_t* offs = reinterpret_cast<int32_t*>(sm + (RING == 2 ? 2 * R : R));
-
-  for (int j = tid; j < k; j += blockDim.x) offs[j] = args.insts ? in.a[j] : args.one_offs[j];
-  __syncthreads();
-  const int32_t a1 = offs[0];
-  const int32_t ak = offs[k - 1];
+  const int32_t* a = args.insts ? in.a : args.one_offs;
+  const int32_t a1 = a[0];
+  const int32_t ak = a[k - 1];
   if (n <= a1) return;
-  // per-offset read displacement: -a_j (table), R - a_j (mirrored ring)
-  int32_t ro[kSdpMaxKRegs];
-  if constexpr (KREG) {
-#pragma unroll
-    for (int j = 0; j < kSdpMaxKRegs; ++j) {
-      const int32_t a = j < k ? offs[j] : offs[0];
-      ro[j] = RING == 2 ? (int32_t)R - a : a;
-    }
-  }
+  const int W = ak < (int)blockDim.x ? ak : (int)blockDim.x;
+  const int nstep = (W + 31) & ~31;  // threads that take part in the steps (blockDim is a multiple of 32)
+  // per-offset read displacement: -a_j words (table), -4 a_j bytes (masked
+  // ring), 4 (R - a_j) bytes + the ring's address (mirrored ring)
+  const uint32_t rb = smem_u32(ring), maskb = 4 * R - 1u;
+  int32_t* disp = reinterpret_cast<int32_t*>(sm + (RING == 2 ? 2 * R : R));
+  for (int j = tid; j < k; j += blockDim.x) disp[j] = RING == 2 ? 4 * ((int32_t)R - a[j]) + (int32_t)rb : (RING == 1 ? -4 * a[j] : -a[j]);
   if constexpr (RING != 0) {
     for (int x = tid; x < a1; x += blockDim.x) {
       const uint32_t v = st[x];
       ring[(uint32_t)x & mask] = v;
       if constexpr (RING == 2) ring[((uint32_t)x & mask) + R] = v;
     }
-    __syncthreads();
   }
-  const int W = ak < (int)blockDim.x ? ak : (int)blockDim.x;
-  uint32_t pos = ((uint32_t)a1 + (uint32_t)tid) & mask;  // (i mod R) for the ring modes
-  for (int64_t base = a1; base < n; base += W) {
-    const int64_t i = base + tid;
-    if (tid < W && i < n) {
-      uint32_t v;
-      if constexpr (RING == 2) {
-        const uint32_t* rp = ring + pos;
-        if constexpr (KREG) {
-          v = rp[ro[0]];
+  __syncthreads();
+  if (tid < nstep) {
+    constexpr int NR = KP > 0 ? KP : 1;
+    int32_t ro[NR];
+    if constexpr (KP > 0) {
 #pragma unroll
-          for (int j = 1; j < kSdpMaxKRegs; ++j)
-            if (KFULL || j < k) v = combine<OP>(v, rp[ro[j]]);
-        } else {
-          v = rp[(int32_t)R - offs[0]];
-          for (int j = 1; j < k; ++j) v = combine<OP>(v, rp[(int32_t)R - offs[j]]);
-        }
-        ring[pos] = v;
-        ring[pos + R] = v;
-      } else if constexpr (RING == 1) {
-        if constexpr (KREG) {
-          v = ring[(pos - (uint32_t)ro[0]) & mask];
-#pragma unroll
-          for (int j = 1; j < kSdpMaxKRegs; ++j)
-            if (KFULL || j < k) v = combine<OP>(v, ring[(pos - (uint32_t)ro[j]) & mask]);
-        } else {
-          v = ring[(pos - (uint32_t)offs[0]) & mask];
-          for (int j = 1; j < k; ++j) v = combine<OP>(v, ring[(pos - (uint32_t)offs[j]) & mask]);
-        }
-        ring[pos] = v;
-      } else {
-        if constexpr (KREG) {
-          v = st[i - ro[0]];
-#pragma unroll
-          for (int j = 1; j < kSdpMaxKRegs; ++j)
-            if (KFULL || j < k) v = combine<OP>(v, st[i - ro[j]]);
-        } else {
-          v = st[i - offs[0]];
-          for (int j = 1; j < k; ++j) v = combine<OP>(v, st[i - offs[j]]);
-        }
-      }
-      st[i] = v;
+      for (int j = 0; j < KP; ++j) ro[j] = disp[j < k ? j : 0];  // (min: reading a_1's term again changes nothing)
     }
-    pos = (pos + (uint32_t)W) & mask;
-    __syncthreads();
+    uint32_t pos = RING ? 4 * (((uint32_t)a1 + (uint32_t)tid) & mask) : 0u;  // 4 (i mod R) of the cell being computed
+    uint32_t* cur = st + a1 + tid;                                           // its place in the table
+    auto rd = [&](int32_t d) -> uint32_t {
+      if constexpr (RING == 2) return lds_u32(pos + (uint32_t)d);
+      if constexpr (RING == 1) return lds_u32(rb + ((pos + (uint32_t)d) & maskb));
+      return cur[d];
+    };
+    auto cell = [&]() -> uint32_t {
+      uint32_t v = kIdentity;
+      if constexpr (KP > 0) {
+#pragma unroll
+        for (int q = 0; q < KP; q += G) {
+          if (FULL || q < k) {
+            uint32_t x[G];
+#pragma unroll
+            for (int i = 0; i < G; ++i) x[i] = (FULL || OP == 0 || q + i < k) ? rd(ro[q + i]) : kIdentity;
+#pragma unroll
+            for (int i = 0; i < G; i += 2) v = combine3<OP>(x[i], x[i + 1], v);
+          }
+        }
+      } else {
+        int j = 0;
+        for (; j + G <= k; j += G) {
+          uint32_t x[G];
+#pragma unroll
+          for (int i = 0; i < G; i += 4) {
+            const int4 d = *reinterpret_cast<const int4*>(disp + j + i);
+            x[i] = rd(d.x), x[i + 1] = rd(d.y), x[i + 2] = rd(d.z), x[i + 3] = rd(d.w);
+          }
+#pragma unroll
+          for (int i = 0; i < G; i += 2) v = combine3<OP>(x[i], x[i + 1], v);
+        }
+        for (; j < k; ++j) v = combine<OP>(v, rd(disp[j]));
+      }
+      return v;
+    };
+    auto put = [&](uint32_t v) {
+      if constexpr (RING != 0) {
+        sts_u32(rb + pos, v);
+        if constexpr (RING == 2) sts_u32(rb + 4 * R + pos, v);
+      }
+      *cur = v;
+    };
+    // Whole steps: threads from W up read with the others (their reads stay
+    // inside the ring; off the ring they are kept from the table) and write
+    // nothing.
+    const bool active = tid < W;
+    const bool all = nstep == (int)blockDim.x;
+    const int64_t whole = (n - a1) / W;
+    for (int64_t s = 0; s < whole; ++s) {
+      if (RING != 0 || active) {
+        const uint32_t v = cell();
+        if (active) put(v);
+      }
+      pos = (pos + 4 * (uint32_t)W) & maskb;
+      cur += W;
+      if (all) __syncthreads();
+      else bar_step(nstep);
+    }
+    if (tid < n - a1 - whole * W) put(cell());
   }
 }
 
-template <int OP, int RING, bool KREG, bool KFULL>
+template <int OP, int RING, int KP, int G, bool FULL>
 cudaError_t launch_variant(const SdpLaunchArgs& a, size_t smem, cudaStream_t stream) {
-  auto kern = sdp_kernel<OP, RING, KREG, KFULL>;
+  auto kern = sdp_kernel<OP, RING, KP, G, FULL>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   kern<<<a.ninst, a.threads, smem, stream>>>(a);
   return cudaGetLastError();
 }
 
+// The smallest register-resident variant that holds kmax offsets: in one of
+// twice the size half the reads are predicated off but still issued (k = 16,
+// W = 600: 1106 clocks a step in the 32-offset variant, 522 in its own).
 template <int OP, int RING>
-cudaError_t launch_k(const SdpLaunchArgs& a, int kmax, bool all_full, size_t smem, cudaStream_t stream) {
-  if (kmax > kSdpMaxKRegs) return launch_variant<OP, RING, false, false>(a, smem, stream);
-  if (all_full) return launch_variant<OP, RING, true, true>(a, smem, stream);
-  return launch_variant<OP, RING, true, false>(a, smem, stream);
+cudaError_t launch_k(const SdpLaunchArgs& a, int kmax, bool same_k, size_t smem, cudaStream_t stream) {
+  // off the ring a read waits for L2, and 64-bit addresses leave no registers
+  // for more offsets
+  if (kmax > (RING == 0 ? 8 : kSdpMaxKRegs)) return launch_variant<OP, RING, 0, 8, false>(a, smem, stream);
+  if constexpr (RING != 0) {
+    if (kmax > 16) {
+      if (!same_k || kmax < 32) return launch_variant<OP, RING, 32, 8, false>(a, smem, stream);
+      // up to 8 warps the latency of the loads counts, above the pipe does
+      return a.threads <= 256 ? launch_variant<OP, RING, 32, 32, true>(a, smem, stream)
+                              : launch_variant<OP, RING, 32, 8, true>(a, smem, stream);
+    }
+    if (kmax > 8)
+      return same_k && kmax == 16 ? launch_variant<OP, RING, 16, 8, true>(a, smem, stream)
+                                  : launch_variant<OP, RING, 16, 8, false>(a, smem, stream);
+  }
+  if (kmax > 4) return launch_variant<OP, RING, 8, 8, false>(a, smem, stream);
+  return launch_variant<OP, RING, 4, 4, false>(a, smem, stream);
 }
 
 template <int OP>
-cudaError_t launch_op(const SdpLaunchArgs& a, int kmax, bool all_full, size_t smem, cudaStream_t stream) {
+cudaError_t launch_op(const SdpLaunchArgs& a, int kmax, bool same_k, size_t smem, cudaStream_t stream) {
   const int mode = sdp_ring_mode(a.ring_log2);
-  if (mode == 2) return launch_k<OP, 2>(a, kmax, all_full, smem, stream);
-  if (mode == 1) return launch_k<OP, 1>(a, kmax, all_full, smem, stream);
-  return launch_k<OP, 0>(a, kmax, all_full, smem, stream);
+  if (mode == 2) return launch_k<OP, 2>(a, kmax, same_k, smem, stream);
+  if (mode == 1) return launch_k<OP, 1>(a, kmax, same_k, smem, stream);
+  return launch_k<OP, 0>(a, kmax, same_k, smem, stream);
 }
 
 }  // namespace
@@ -141,18 +206,18 @@ int sdp_ring_mode(int ring_log2) {
 size_t sdp_smem_bytes(int ring_log2, int kmax) {
   const int mode = sdp_ring_mode(ring_log2);
   const size_t ring = mode == 0 ? 0 : ((size_t)1 << ring_log2) * 4 * (mode == 2 ? 2 : 1);
-  return ring + (size_t)kmax * 4;
+  return ring + ((size_t)kmax * 4 + 31) / 32 * 32;
 }
 
 cudaError_t launch_sdp(const SdpLaunchArgs& a, cudaStream_t stream) {
   if (a.ninst <= 0) return cudaSuccess;
   // kmax: largest k in the launch (the host passes it through one.k for both
-  // paths); kfull: every instance has exactly kSdpMaxKRegs offsets
+  // paths); same_k: every instance has that many offsets
   const int kmax = a.one.k;
-  const bool kfull = a.kfull != 0;
+  const bool same_k = a.same_k != 0;
   const size_t smem = sdp_smem_bytes(a.ring_log2, kmax);
-  if (a.op == 0) return launch_op<0>(a, kmax, kfull, smem, stream);
-  return launch_op<1>(a, kmax, kfull, smem, stream);
+  if (a.op == 0) return launch_op<0>(a, kmax, same_k, smem, stream);
+  return launch_op<1>(a, kmax, same_k, smem, stream);
 }
 
 }  // namespace dpk

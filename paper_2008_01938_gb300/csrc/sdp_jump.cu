@@ -421,7 +421,7 @@ dp_status launch_records(const dpk::SdpInstDev* insts, int count, int32_t k, int
   dpk::SdpLaunchArgs args{};
   args.insts = insts;
   args.one.k = k;
-  args.kfull = k == dpk::kSdpMaxKRegs;
+  args.same_k = 1;
   args.ninst = count;
   args.op = DP_OP_ADD_MOD32;
   args.threads = threads;

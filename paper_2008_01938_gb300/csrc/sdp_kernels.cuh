@@ -41,7 +41,7 @@ struct SdpLaunchArgs {
   int32_t op;                // 0 = min, 1 = add mod 2^32
   int32_t ring_log2;         // 0: no ring (read the table in global memory)
   int32_t threads;
-  int32_t kfull;             // 1: every instance has exactly kSdpMaxKRegs offsets
+  int32_t same_k;            // 1: every instance has exactly one.k offsets
   int32_t pad_;
   uint32_t* st_all;          // batched tables
   const int64_t* st_off;

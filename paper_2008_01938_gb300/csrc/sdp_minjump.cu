@@ -450,7 +450,7 @@ dp_status mj_launch_records(const dpk::SdpInstDev* insts, int count, int32_t k, 
   dpk::SdpLaunchArgs args{};
   args.insts = insts;
   args.one.k = k;
-  args.kfull = k == dpk::kSdpMaxKRegs;
+  args.same_k = 1;
   args.ninst = count;
   args.op = DP_OP_MIN;
   args.threads = threads;

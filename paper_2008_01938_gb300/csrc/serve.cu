@@ -234,7 +234,7 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
                                   : sdp_jump_chunks(r->n, r->offs.data(), k, ds->sms);
     if (chunks[b] < 2) bat.push_back(b);
   }
-  bool ring_ok = true, kfull = !bat.empty();
+  bool ring_ok = true, same_k = true;
   std::vector<int64_t> st_off(reqs.size());
   int64_t cells = 0, noffs = 0;
   for (size_t b = 0; b < reqs.size(); ++b) {
@@ -246,7 +246,7 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
   for (size_t b : bat) {
     const Req* r = reqs[b];
     kmax = std::max(kmax, (int)r->offs.size());
-    kfull = kfull && (int)r->offs.size() == dpk::kSdpMaxKRegs;
+    same_k = same_k && r->offs.size() == reqs[bat[0]]->offs.size();
     int th, lg;
     sdp_shape(r->offs[0], r->offs.back(), &th, &lg);
     threads = std::max(threads, th);
@@ -318,7 +318,7 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
     dpk::SdpLaunchArgs args{};
     args.insts = reinterpret_cast<const dpk::SdpInstDev*>(ws + o_insts);
     args.one.k = kmax;
-    args.kfull = kfull;
+    args.same_k = same_k;
     args.ninst = (int32_t)bat.size();
     args.op = op;
     args.threads = threads;
