@@ -260,7 +260,12 @@ dp_status mcm_plan_destroy(void *plan);
  * window obtained by products modulo the recurrence's characteristic
  * polynomial.  That path enqueues a few dozen launches and takes a
  * workspace of a few MB from the stream-ordered allocator (released on the
- * same stream).  Its result is bit-identical. */
+ * same stream).  Its result is bit-identical.
+ * With DP_OP_MIN every cell from some position on is the minimum of its
+ * residue class of the preset, modulo the gcd of the offsets.  Where the
+ * offsets (read on the host) say that this position is near enough, one
+ * launch computes the cells before it and writes the others; otherwise long
+ * tables are cut into chunks as above. */
 dp_status sdp_solve(uint32_t *ST, int64_t n, const int32_t *a, int32_t k, dp_op op,
                     int32_t *status_dev, void *stream);
 

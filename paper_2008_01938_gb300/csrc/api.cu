@@ -12,6 +12,7 @@
 #include <list>
 #include <map>
 #include <mutex>
+#include <numeric>
 #include <string>
 #include <tuple>
 
@@ -361,6 +362,97 @@ void sdp_shape(int32_t a1, int32_t ak, int* threads, int* ring_log2) {
   *ring_log2 = lg <= dpk::kSdpRingMaxLog2 ? std::max(lg, 1) : 0;
 }
 
+int64_t sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g_out) {
+  int32_t g = a[0], gap = a[k - 1];
+  for (int j = 1; j < k; ++j) {
+    g = std::gcd(g, a[j]);
+    gap = std::max(gap, a[j - 1] - a[j]);
+  }
+  // The sums of offsets / g as a bitset, 64 at a time, until offsets[k-1] / g
+  // consecutive ones: from the first of those (c) on, every number is a sum.
+  // The search stops at the table's end, and after kTailOps word operations
+  // (a word costs about k + 8; 40 us of host time in all), which offsets that
+  // fill in slowly reach first.
+  constexpr int64_t kTailOps = 1 << 15;
+  const int64_t room = n - ((int64_t)a[0] + gap + g);  // largest useful g c
+  if (room < 0) return 0;
+  const int64_t words = std::min<int64_t>(kTailOps / (k + 8), room / g / 64 + 1);
+  std::vector<uint64_t> sum((size_t)words + 1, 0);
+  const int64_t need = a[k - 1] / g;
+  int64_t run = 0, c = -1;
+  for (int64_t w = 0; w < words && c < 0; ++w) {
+    uint64_t x = w == 0 ? 1u : 0u;
+    for (int j = 0; j < k; ++j) {
+      const int64_t at = 64 * w - a[j] / g;  // sums at .. at + 63, of which those in earlier words are known
+      if (at <= -64) continue;
+      const int64_t q = at >> 6;
+      const int r = (int)(at & 63);
+      const uint64_t lo = q >= 0 ? sum[(size_t)q] : 0u, hi = q + 1 >= 0 && q + 1 < w ? sum[(size_t)q + 1] : 0u;
+      x |= r == 0 ? lo : (lo >> r) | (hi << (64 - r));
+    }
+    for (int j = k - 1; j >= 0 && a[j] / g < 64; --j)  // offsets that add up inside the word
+      for (int64_t d = a[j] / g; d < 64; d *= 2) x |= x << d;
+    sum[(size_t)w] = x;
+    if (x == ~(uint64_t)0) {
+      run += 64;
+      if (run >= need) c = 64 * w + 64 - run;
+    } else {
+      const int low = __builtin_ctzll(~x);  // ones that continue the run from the word below
+      if (run + low >= need) c = 64 * w - run;
+      for (int b = low, r = 0; need < 64 && b < 64 && c < 0; ++b) {  // runs inside the word
+        r = (x >> b) & 1u ? r + 1 : 0;
+        if (r >= need) c = 64 * w + b + 1 - r;
+      }
+      run = __builtin_clzll(~x);  // ones at the top start the next run
+    }
+  }
+  if (c < 0) return 0;
+  // every s < a_1 has an offset a_j with a_1 <= s + a_j < a_1 + gap, so from
+  // N0 = g c + a_1 - 1 + gap on every s congruent to N reaches N
+  const int64_t n0 = g * c + a[0] - 1 + gap;
+  if (n0 + g >= n) return 0;
+  *g_out = g;
+  return n0 + g;  // the last g cells below hold the classes' minima
+}
+
+SdpRoute sdp_route(int64_t n, const int32_t* a, int32_t k, int op, int sms) {
+  SdpRoute r;
+  if (op == DP_OP_ADD_MOD32) {
+    r.chunks = sdp_jump_chunks(n, a, k, sms);
+    return r;
+  }
+  r.tail_from = sdp_min_tail(n, a, k, &r.g);
+  int threads = 0, ring_log2 = 0;
+  sdp_shape(a[0], a[k - 1], &threads, &ring_log2);
+  if (ring_log2 <= 0) r.tail_from = 0;  // the fill keeps the class minima where the ring would be
+  r.chunks = sdp_min_jump_chunks(n, a, k, sms, r.tail_from);
+  if (r.chunks >= 2) r.tail_from = 0;
+  return r;
+}
+
+void sdp_single_args(dpk::SdpLaunchArgs* args, uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int op,
+                     const SdpRoute& route, int sms, int32_t* status) {
+  *args = dpk::SdpLaunchArgs{};
+  args->one.st = ST;
+  args->one.n = n;
+  args->one.k = k;
+  args->same_k = 1;
+  args->ninst = 1;
+  args->op = op;
+  sdp_shape(a[0], a[k - 1], &args->threads, &args->ring_log2);
+  if (route.tail_from > 0) {
+    // one block computes, the others fill: a block per 16384 cells keeps a
+    // short tail from reading the preset more often than it writes, and one
+    // per SM (1024 threads storing 16 bytes each) saturates the memory
+    args->one.tail_from = route.tail_from;
+    args->one.g = route.g;
+    args->threads = 1024;
+    args->fill_blocks = (int32_t)std::max<int64_t>(1, std::min<int64_t>(sms - 1, (n - route.tail_from) / 16384));
+  }
+  args->status = status;
+  for (int j = 0; j < k; ++j) args->one_offs[j] = a[j];
+}
+
 }  // namespace dph
 
 using namespace dph;
@@ -637,7 +729,16 @@ int32_t dp_test_sdp_jump_chunks(int64_t n, const int32_t* a, int32_t k) {
 int32_t dp_test_sdp_min_jump_chunks(int64_t n, const int32_t* a, int32_t k) {
   DevState* ds = nullptr;
   if (!a || k < 1 || current_dev(&ds) != DP_OK) return -1;
-  return sdp_min_jump_chunks(n, a, k, ds->sms);
+  return sdp_min_jump_chunks(n, a, k, ds->sms, 0);
+}
+
+// Test hook without a device: where the periodic tail of a min table starts
+// (0: none found below n); *g gets its period.
+int64_t dp_test_sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g) {
+  if (!a || !g || k < 1 || k > dpk::kSdpMaxK) return -1;
+  for (int j = 0; j < k; ++j)
+    if (a[j] < 1 || (j > 0 && a[j] >= a[j - 1])) return -1;
+  return n > a[0] ? sdp_min_tail(n, a, k, g) : 0;
 }
 
 // Test hook without a device: the min jump plan sdp_solve would take for
@@ -822,31 +923,16 @@ dp_status sdp_solve(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, dp_op 
   if (n <= a[0]) return DP_OK;
   DevState* ds = nullptr;
   if ((rc = current_dev(&ds)) != DP_OK) return rc;
-  if (op == DP_OP_ADD_MOD32) {
-    // long tables: chunks from jumped windows, side by side (sdp_jump.cu)
-    const int chunks = sdp_jump_chunks(n, a, k, ds->sms);
-    if (chunks >= 2)
-      return sdp_add_jump(ST, n, a, k, chunks, status_dev ? status_dev : ds->status,
-                          static_cast<cudaStream_t>(stream));
-  } else {
-    // the same for min, with Boolean products (sdp_minjump.cu)
-    const int chunks = sdp_min_jump_chunks(n, a, k, ds->sms);
-    if (chunks >= 2)
-      return sdp_min_jump(ST, n, a, k, chunks, status_dev ? status_dev : ds->status,
-                          static_cast<cudaStream_t>(stream));
-  }
-  dpk::SdpLaunchArgs args{};
-  args.insts = nullptr;
-  args.one.st = ST;
-  args.one.n = n;
-  args.one.a = nullptr;
-  args.one.k = k;
-  args.same_k = 1;
-  args.ninst = 1;
-  args.op = (int32_t)op;
-  sdp_shape(a[0], a[k - 1], &args.threads, &args.ring_log2);
-  args.status = status_dev ? status_dev : ds->status;
-  for (int j = 0; j < k; ++j) args.one_offs[j] = a[j];
+  // long tables: chunks from jumped windows, side by side (sdp_jump.cu for +,
+  // sdp_minjump.cu for min), or for min the cells before the periodic tail
+  // beside its fill; the cost models decide
+  const SdpRoute route = sdp_route(n, a, k, op, ds->sms);
+  int32_t* status = status_dev ? status_dev : ds->status;
+  if (route.chunks >= 2)
+    return op == DP_OP_ADD_MOD32 ? sdp_add_jump(ST, n, a, k, route.chunks, status, static_cast<cudaStream_t>(stream))
+                                 : sdp_min_jump(ST, n, a, k, route.chunks, status, static_cast<cudaStream_t>(stream));
+  dpk::SdpLaunchArgs args;
+  sdp_single_args(&args, ST, n, a, k, op, route, ds->sms, status);
   const bool prof = profiling();
   if (prof) profile_mark(1, static_cast<cudaStream_t>(stream), false);
   cudaError_t e = dpk::launch_sdp(args, static_cast<cudaStream_t>(stream));
@@ -922,6 +1008,10 @@ dp_status sdp_plan_create(int32_t batch, const int64_t* n_host, const int32_t* k
     if (lg > dpk::kSdpRingMaxLog2) ring_ok = false;
     ring_log2 = std::max(ring_log2, lg);
   }
+  // min: each block fills its own periodic tail (the class values need the ring's room)
+  if (op == DP_OP_MIN && ring_ok)
+    for (int b = 0; b < batch; ++b)
+      insts[b].tail_from = sdp_min_tail(insts[b].n, a_host + insts[b].a_off, insts[b].k, &insts[b].g);
   auto* pl = new SdpPlan();
   pl->device = ds->device;
   pl->batch = batch;

@@ -79,6 +79,21 @@ dp_status mcm_enqueue(const McmStatic& sp, const McmLayout& L, void* ws, const i
 // ---------------------------------------------------------------------------
 dp_status sdp_validate(int64_t n, const int32_t* a, int32_t k, int op);
 void sdp_shape(int32_t a1, int32_t ak, int* threads, int* ring_log2);
+// (x) = min: the first cell from which the table repeats its last g cells, g
+// the gcd of the offsets (host arithmetic on the offsets only; see
+// sdp_kernels.cuh).  0: not below n, or not found within a bounded search.
+int64_t sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g);
+// How one table is solved: in `chunks` >= 2 chunks from jumped windows, or by
+// the step kernel, with tail_from > 0 up to there and the rest filled.
+struct SdpRoute {
+  int chunks = 0;
+  int64_t tail_from = 0;
+  int32_t g = 0;
+};
+SdpRoute sdp_route(int64_t n, const int32_t* a, int32_t k, int op, int sms);
+// Fills the arguments of the step kernel's launch for one table (not for chunks >= 2).
+void sdp_single_args(dpk::SdpLaunchArgs* args, uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int op,
+                     const SdpRoute& route, int sms, int32_t* status);
 // (x) = + on one instance, by chunks that start from jumped windows
 // (sdp_jump.cu): the number of chunks the cost model picks (0: solve step by
 // step), and the solve with a given number of chunks.
@@ -91,10 +106,10 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
 // (x) = min on one instance, by chunks whose windows come from Boolean
 // products modulo the characteristic polynomial (sdp_minjump.cu): whether the
 // path applies (a_k >= 32, a_1 <= 8192, a long enough table, the window on
-// chip), the number of chunks the cost model picks (0: solve step by step),
-// and the solve with a given number of chunks.
+// chip), the number of chunks the cost model picks (0: solve step by step, up
+// to tail_from when that is not 0), and the solve with a given number of chunks.
 bool sdp_min_jump_eligible(int64_t n, const int32_t* a, int32_t k);
-int sdp_min_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms);
+int sdp_min_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms, int64_t tail_from);
 // The plan behind it (host arithmetic only): P, L, L0, squarings, chunks asked.
 int sdp_min_jump_plan(int64_t n, const int32_t* a, int32_t k, int sms, int64_t out[5]);
 dp_status sdp_min_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int chunks, int32_t* status,

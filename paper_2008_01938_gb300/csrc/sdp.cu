@@ -24,6 +24,48 @@ __device__ __forceinline__ uint32_t combine3(uint32_t x, uint32_t y, uint32_t z)
 // Barrier over the threads that compute cells (`count`, a multiple of 32).
 __device__ __forceinline__ void bar_step(int count) { asm volatile("bar.sync 1, %0;" ::"r"(count) : "memory"); }
 
+// Writes st[lo .. hi) with the values cls[x mod g] of the residue classes,
+// as the part-th of nparts blocks.  Stores are 16 bytes wide where the table
+// allows (lo and hi need no alignment).  Bound by the memory's write rate: a
+// table of 2^26 cells (268 MB) takes 49 us in all, 5.5 TB/s, with the cells
+// before the tail computed beside the fill (in 152 chunks it took 404 us);
+// 200 tables of 4096 to 65536 cells in one launch 19 us (325 us step by step).
+__device__ void fill_classes(uint32_t* st, int64_t lo, int64_t hi, const uint32_t* cls, int g, int part, int nparts) {
+  const int64_t mis = (int64_t)((reinterpret_cast<uintptr_t>(st) >> 2) & 3);  // words past a 16-byte boundary
+  int64_t v0 = (lo + mis + 3) >> 2, v1 = (hi + mis) >> 2;                     // whole vectors: words 4v - mis ..
+  if (v1 < v0) v1 = v0;
+  const int64_t head = v0 * 4 - mis < hi ? v0 * 4 - mis : hi;
+  if (part == 0) {
+    for (int64_t x = lo + threadIdx.x; x < head; x += blockDim.x) st[x] = cls[x % g];
+    for (int64_t x = (v1 * 4 - mis > head ? v1 * 4 - mis : head) + threadIdx.x; x < hi; x += blockDim.x)
+      st[x] = cls[x % g];
+  }
+  const int64_t stride = (int64_t)nparts * blockDim.x;
+  int64_t v = v0 + (int64_t)part * blockDim.x + threadIdx.x;
+  uint4* out = reinterpret_cast<uint4*>(st - mis);
+  if (g == 1) {
+    const uint32_t c = cls[0];
+    const uint4 q = make_uint4(c, c, c, c);
+#pragma unroll 4
+    for (; v < v1; v += stride) out[v] = q;
+    return;
+  }
+  const int adv = (int)((4 * stride) % g);
+  int r = v < v1 ? (int)((4 * v - mis) % g) : 0;
+  for (; v < v1; v += stride) {
+    uint32_t c[4];
+    int x = r;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      c[i] = cls[x];
+      if (++x == g) x = 0;
+    }
+    out[v] = make_uint4(c[0], c[1], c[2], c[3]);
+    r += adv;
+    if (r >= g) r -= g;
+  }
+}
+
 __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
   uint32_t v;
   asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
@@ -59,9 +101,37 @@ __global__ void __launch_bounds__(1024) sdp_kernel(const __grid_constant__ SdpLa
   constexpr uint32_t kIdentity = OP == 0 ? 0xFFFFFFFFu : 0u;
   const int tid = threadIdx.x;
 
+  if ((int)blockIdx.x >= args.ninst) {
+    // single table whose cells from one.tail_from - g on depend on their
+    // residue class modulo g alone: this block fills its share of them with
+    // the minima of the preset's classes while block 0 computes the rest
+    const SdpInstDev in = args.one;
+    const int g = in.g, A = args.one_offs[0];
+    for (int c = tid; c < g; c += blockDim.x) sm[c] = 0xFFFFFFFFu;
+    __syncthreads();
+    if (g == 1) {
+      uint32_t v = 0xFFFFFFFFu;
+      for (int s = tid; s < A; s += blockDim.x) v = min(v, in.st[s]);
+      v = __reduce_min_sync(0xFFFFFFFFu, v);
+      if ((tid & 31) == 0) atomicMin(sm, v);
+    } else {  // a stride that is a multiple of g where one fits: a thread stays in one class
+      const int stride = g < (int)blockDim.x ? (int)blockDim.x / g * g : (int)blockDim.x;
+      if (g <= (int)blockDim.x) {
+        uint32_t v = 0xFFFFFFFFu;
+        for (int s = tid; tid < stride && s < A; s += stride) v = min(v, in.st[s]);
+        if (tid < stride) atomicMin(sm + tid % g, v);
+      } else {
+        for (int s = tid; s < A; s += stride) atomicMin(sm + s % g, in.st[s]);
+      }
+    }
+    __syncthreads();
+    fill_classes(in.st, in.tail_from, in.n, sm, g, (int)blockIdx.x - args.ninst, (int)gridDim.x - args.ninst);
+    return;
+  }
+
   SdpInstDev in = args.insts ? args.insts[blockIdx.x] : args.one;
   uint32_t* st = args.st_off ? args.st_all + args.st_off[blockIdx.x] : in.st;
-  const int64_t n = in.n;
+  const int64_t n = in.tail_from > 0 ? in.tail_from : in.n;  // cells computed by the recurrence
   const int k = in.k;
   const int ring_log2 = args.ring_log2;
   const uint32_t R = RING ? (1u << ring_log2) : 0u;
@@ -70,7 +140,7 @@ __global__ void __launch_bounds__(1024) sdp_kernel(const __grid_constant__ SdpLa
   const int32_t* a = args.insts ? in.a : args.one_offs;
   const int32_t a1 = a[0];
   const int32_t ak = a[k - 1];
-  if (n <= a1) return;
+  if (in.n <= a1) return;
   const int W = ak < (int)blockDim.x ? ak : (int)blockDim.x;
   const int nstep = (W + 31) & ~31;  // threads that take part in the steps (blockDim is a multiple of 32)
   // per-offset read displacement: -a_j words (table), -4 a_j bytes (masked
@@ -154,6 +224,15 @@ __global__ void __launch_bounds__(1024) sdp_kernel(const __grid_constant__ SdpLa
     }
     if (tid < n - a1 - whole * W) put(cell());
   }
+  if (in.tail_from > 0 && (int)gridDim.x == args.ninst) {
+    // the rest of the table repeats its last g computed cells
+    const int g = in.g;
+    __syncthreads();
+    uint32_t* cls = sm;
+    for (int64_t x = n - g + tid; x < n; x += blockDim.x) cls[x % g] = st[x];
+    __syncthreads();
+    fill_classes(st, n, in.n, cls, g, 0, 1);
+  }
 }
 
 template <int OP, int RING, int KP, int G, bool FULL>
@@ -161,7 +240,7 @@ cudaError_t launch_variant(const SdpLaunchArgs& a, size_t smem, cudaStream_t str
   auto kern = sdp_kernel<OP, RING, KP, G, FULL>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<a.ninst, a.threads, smem, stream>>>(a);
+  kern<<<a.ninst + a.fill_blocks, a.threads, smem, stream>>>(a);
   return cudaGetLastError();
 }
 

@@ -14,6 +14,15 @@
 // global memory.  Consecutive threads handle
 // consecutive cells, so for any offset the ring reads of a warp are 32
 // consecutive words: bank-conflict free.
+//
+// Periodic tail of (x) = min.  Unrolled down to the preset, ST[N] = min over
+// the preset positions s that reach N, that is for which some offset a_j with
+// s + a_j >= a_1 leaves N - s - a_j a sum of offsets.  With g the gcd of the
+// offsets every such s is congruent to N modulo g, and from some N0 on every
+// s congruent to N modulo g does reach N, because all large multiples of g
+// are sums of offsets (SdpInstDev::tail_from; dph::sdp_min_tail finds N0 from
+// the offsets alone).  From N0 on a cell is therefore the minimum of its
+// residue class of the preset, and the table is written, not computed.
 #pragma once
 
 #include <cstdint>
@@ -32,6 +41,9 @@ struct SdpInstDev {
   const int32_t* a;    // offsets on the device (batched path)
   int32_t k;
   int32_t a_off;       // offset of this instance's offsets in a shared array
+  int64_t tail_from;   // min: cells from here on repeat with period g (0: compute every cell)
+  int32_t g;           // gcd of the offsets, when tail_from > 0
+  int32_t pad_;
 };
 
 struct SdpLaunchArgs {
@@ -42,7 +54,7 @@ struct SdpLaunchArgs {
   int32_t ring_log2;         // 0: no ring (read the table in global memory)
   int32_t threads;
   int32_t same_k;            // 1: every instance has exactly one.k offsets
-  int32_t pad_;
+  int32_t fill_blocks;       // single table with a tail: blocks that fill it beside the block that computes
   uint32_t* st_all;          // batched tables
   const int64_t* st_off;
   int32_t* status;

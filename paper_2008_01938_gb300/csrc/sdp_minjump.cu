@@ -470,7 +470,7 @@ bool sdp_min_jump_eligible(int64_t n, const int32_t* a, int32_t k) {
 }
 
 int sdp_min_jump_plan(int64_t n, const int32_t* a, int32_t k, int sms, int64_t out[5]) {
-  const int chunks = sdp_min_jump_chunks(n, a, k, sms);
+  const int chunks = sdp_min_jump_chunks(n, a, k, sms, 0);
   for (int i = 0; i < 5; ++i) out[i] = 0;
   if (chunks < 2) return 0;
   const MjPlan p = mj_plan_for(n, a[0], chunks);
@@ -482,10 +482,11 @@ int sdp_min_jump_plan(int64_t n, const int32_t* a, int32_t k, int sms, int64_t o
   return chunks;
 }
 
-int sdp_min_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms) {
+int sdp_min_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms, int64_t tail_from) {
   if (!sdp_min_jump_eligible(n, a, k)) return 0;
   const int32_t A = a[0], ak = a[k - 1];
-  double best = 0.8 * mj_plain_us(n - A, ak, k);  // the jump must win clearly
+  double best = 0.8 * mj_plain_us((tail_from > 0 ? tail_from : n) - A, ak, k);  // the jump must win clearly
+  if (best < 38.0) return 0;  // less than the jump's fixed cost and one product level
   int bestP = 0;
   for (int c = 2; c <= sms; ++c) {
     const MjPlan p = mj_plan_for(n, A, c);

@@ -216,23 +216,26 @@ dp_status launch_mcm_group(Server* S, const std::vector<Req*>& reqs, bool i64, L
 
 // A group of S-DP requests with one operator.  Requests long enough for the
 // chunked paths of sdp_solve (sdp_jump.cu for +, sdp_minjump.cu for min; the
-// same cost models decide) run through those, spread over the SMs; the
-// others share one launch of the S-DP kernel, one block each.  Everything is
+// same cost models decide) or with a long periodic tail run through those,
+// spread over the SMs; the others share one launch of the S-DP kernel, one block each.  Everything is
 // enqueued on the launch's stream, so one event covers the group.
 dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Launch* L) {
   int threads = 32, kmax = 1, ring_log2 = 1;
   DevState* ds = nullptr;
   dp_status rc0 = current_dev(&ds);
   if (rc0 != DP_OK) return rc0;
-  std::vector<int> chunks(reqs.size(), 0);
+  std::vector<SdpRoute> route(reqs.size());
   std::vector<size_t> bat;  // requests of the shared launch
+  // a request in chunks, or with a tail long enough to fill from several SMs
+  // (one SM writes 2^18 cells in about 10 us)
+  auto own_launch = [&](size_t b) {
+    return route[b].chunks >= 2 || (route[b].tail_from > 0 && reqs[b]->n - route[b].tail_from > (1 << 18));
+  };
   for (size_t b = 0; b < reqs.size(); ++b) {
     const Req* r = reqs[b];
     const int k = (int)r->offs.size();
-    if (r->n > r->offs[0])
-      chunks[b] = op == DP_OP_MIN ? sdp_min_jump_chunks(r->n, r->offs.data(), k, ds->sms)
-                                  : sdp_jump_chunks(r->n, r->offs.data(), k, ds->sms);
-    if (chunks[b] < 2) bat.push_back(b);
+    if (r->n > r->offs[0]) route[b] = sdp_route(r->n, r->offs.data(), k, op, ds->sms);
+    if (!own_launch(b)) bat.push_back(b);
   }
   bool ring_ok = true, same_k = true;
   std::vector<int64_t> st_off(reqs.size());
@@ -282,7 +285,7 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
   uint8_t* ws = nullptr;
   if ((e = cudaMallocAsync(reinterpret_cast<void**>(&ws), in_bytes + 256, st)) != cudaSuccess)
     return fail_cuda(e, "serve: workspace allocation");
-  std::vector<dpk::SdpInstDev> insts(bat.size());
+  std::vector<dpk::SdpInstDev> insts(bat.size());  // value-initialised
   std::vector<int64_t> bat_off(bat.size());
   std::vector<int64_t> a_at(reqs.size());
   int64_t ao = 0;
@@ -299,6 +302,8 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
     insts[i].k = (int32_t)reqs[b]->offs.size();
     insts[i].a = reinterpret_cast<const int32_t*>(ws + o_offs) + a_at[b];
     insts[i].a_off = (int32_t)a_at[b];
+    insts[i].tail_from = ring_ok ? route[b].tail_from : 0;
+    insts[i].g = route[b].g;
     bat_off[i] = st_off[b];
   }
   memcpy(hp + o_insts, insts.data(), insts.size() * sizeof(dpk::SdpInstDev));
@@ -329,12 +334,19 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
     if ((e = dpk::launch_sdp(args, st)) != cudaSuccess) return fail_cuda(e, "serve: S-DP launch");
   }
   for (size_t b = 0; b < reqs.size(); ++b) {
-    if (chunks[b] < 2) continue;
+    if (!own_launch(b)) continue;
     const Req* r = reqs[b];
+    if (route[b].chunks < 2) {
+      dpk::SdpLaunchArgs args;
+      sdp_single_args(&args, st_all + st_off[b], r->n, r->offs.data(), (int)r->offs.size(), op, route[b], ds->sms,
+                      d_status);
+      if ((e = dpk::launch_sdp(args, st)) != cudaSuccess) return fail_cuda(e, "serve: S-DP launch");
+      continue;
+    }
     const dp_status rc = op == DP_OP_MIN
-                             ? sdp_min_jump(st_all + st_off[b], r->n, r->offs.data(), (int32_t)r->offs.size(), chunks[b],
+                             ? sdp_min_jump(st_all + st_off[b], r->n, r->offs.data(), (int32_t)r->offs.size(), route[b].chunks,
                                             d_status, st)
-                             : sdp_add_jump(st_all + st_off[b], r->n, r->offs.data(), (int32_t)r->offs.size(), chunks[b],
+                             : sdp_add_jump(st_all + st_off[b], r->n, r->offs.data(), (int32_t)r->offs.size(), route[b].chunks,
                                             d_status, st);
     if (rc != DP_OK) return rc;
   }

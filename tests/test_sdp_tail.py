@@ -1,0 +1,77 @@
+"""The periodic tail of a min S-DP table: where the host says it starts (CPU,
+against the oracle's whole tables), and the tables the GPU writes there."""
+import ctypes
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2008_01938_gb300 import native
+
+# (offsets, n): gcd 1 with 1, 2 and many offsets, consecutive ones, a common
+# factor (below and above 64, and a_1 itself), tables that end before or just
+# after the tail starts, offsets inside one word, k above the register limit
+CASES = [
+    ([1], 40), ([2, 1], 300), ([7, 5], 200), ([64, 63], 9000), ([1055 - i for i in range(32)], 60000),
+    ([96, 90, 84], 3000), ([130, 65], 2000), ([4096, 2048, 1024], 20000), ([500], 5001), ([900, 890, 700, 64], 9001),
+    ([3000, 2999, 1], 30000), ([8192, 7000, 5001, 3333, 1024], 200003), ([61, 53, 50, 40, 33, 17, 9], 1111),
+    ([2000 - 3 * i for i in range(48)], 40002), ([20000, 16000, 1500], 150000), ([40, 30], 111),
+]
+
+
+def tail(a, n):
+    a = np.asarray(a, np.int32)
+    g = ctypes.c_int32()
+    t = native.load().dp_test_sdp_min_tail(n, ctypes.c_void_p(a.ctypes.data), int(a.size), ctypes.byref(g))
+    return int(t), int(g.value)
+
+
+def table(a, n, seed):
+    preset = np.random.RandomState(seed).randint(0, 1 << 32, a[0], dtype=np.uint64).astype(np.uint32)
+    return preset, oracle.sdp(preset, n, np.asarray(a, np.int32), "min")
+
+
+@pytest.mark.parametrize("a,n", CASES)
+def test_tail_repeats_the_class_minima(a, n):
+    t, g = tail(a, n)
+    assert 0 <= t < n
+    if t == 0:
+        return
+    assert g == math.gcd(*a) and t > a[0]
+    preset, ref = table(a, n, len(a))
+    cls = np.array([preset[r::g].min() for r in range(g)], np.uint32)
+    at = np.arange(t - g, n)
+    assert np.array_equal(ref[t - g:], cls[at % g])
+
+
+def test_tail_is_found_where_it_matters():
+    assert tail([1055 - i for i in range(32)], 60000)[0] > 0
+    assert tail([8192, 7000, 5001, 3333, 1024], 200003)[0] > 0
+    assert tail([4096, 2048, 1024], 20000)[1] == 1024
+    assert tail([8192, 8191], 1 << 26)[0] == 0  # fills in too slowly to be found
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("a,n", CASES + [([8192, 7000, 5001, 3333, 1024], 5000003), ([1280, 768, 256], 1 << 20)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_tail_on_the_gpu(a, n, shift):
+    import torch
+    import paper_2008_01938_gb300 as dp
+    preset, ref = table(a, n, len(a) + 1)
+    buf = torch.full((n + 8,), -7, dtype=torch.int32, device="cuda")  # `shift`: a table off the 16-byte boundary
+    st = buf[shift:shift + n]
+    st[:a[0]] = torch.from_numpy(preset.view(np.int32)).cuda()
+    dp.sdp_solve(st, a, op="min")
+    plan = dp.SdpPlan([n, n - 1], [a, a], op="min")
+    both = torch.full((2 * n + 8,), -7, dtype=torch.int32, device="cuda")
+    off = torch.tensor([shift, n + shift + 1], device="cuda")
+    for o in (shift, n + shift + 1):
+        both[o:o + a[0]] = torch.from_numpy(preset.view(np.int32)).cuda()
+    plan.solve(both, off)
+    dp.sync_status()
+    assert np.array_equal(st.cpu().numpy().view(np.uint32), ref)
+    assert torch.all(buf[:shift] == -7) and torch.all(buf[shift + n:] == -7)
+    for o, c in ((shift, n), (n + shift + 1, n - 1)):
+        assert np.array_equal(both[o:o + c].cpu().numpy().view(np.uint32), ref[:c])
+    assert torch.all(both[n + shift:n + shift + 1] == -7) and torch.all(both[2 * n + shift:] == -7)
