@@ -102,6 +102,7 @@ dp_status current_dev(DevState** out) {
     if ((e = dpk::mcm_occupancy(c == 1, &ds.occ[c])) != cudaSuccess) return fail_cuda(e, "MCM occupancy");
     if (ds.occ[c] < 1) ds.occ[c] = 1;
   }
+  if ((e = traceback_configure()) != cudaSuccess) return fail_cuda(e, "configure traceback kernel");
   if ((e = cudaMalloc(&ds.status, 256)) != cudaSuccess) return fail_cuda(e, "cudaMalloc(status)");
   if ((e = cudaMemset(ds.status, 0, 256)) != cudaSuccess) return fail_cuda(e, "cudaMemset(status)");
   // keep freed stream-ordered allocations cached in the pool

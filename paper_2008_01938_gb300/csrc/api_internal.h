@@ -28,6 +28,8 @@ struct DevState {
 // Per-device state for the current device (created on first use).
 dp_status current_dev(DevState** out);
 
+cudaError_t traceback_configure();  // kernel attributes of the current device (traceback.cu)
+
 long long spin_limit();     // bounded-wait budget in clock cycles
 
 // Kernel timing (dp_profile_begin / dp_profile_end): when enabled, the

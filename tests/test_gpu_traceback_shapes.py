@@ -1,0 +1,59 @@
+"""mcm_traceback on split tables of chosen trees: combs, zigzags, balanced and
+random ones, at the sizes where the kernel changes its way of following them."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _split(shape, r, i, j, depth):
+    if shape == "left":       # (i, j-1) and one matrix: a left comb
+        return j - 1
+    if shape == "right":
+        return i
+    if shape == "zigzag":
+        return i if depth % 2 else j - 1
+    if shape == "balanced":
+        return (i + j) // 2
+    if shape == "steps":      # a right spine with 40-matrix subtrees hanging off it
+        return min(j - 1, i + 39)
+    return int(r.randint(i, j))
+
+
+def _tree(shape, n, seed):
+    r = np.random.RandomState(seed)
+    s = np.full((n, n), -1, np.int16)
+    order, stack = [], [(0, n - 1, 0)]
+    while stack:  # root, right, left: the reverse of post-order
+        i, j, d = stack.pop()
+        if i < j:
+            k = _split(shape, r, i, j, d)
+            s[i, j] = k
+            order.append((i, k, j))
+            stack += [(i, k, d + 1), (k + 1, j, d + 1)]
+    return s, np.array(order[::-1], np.int32).reshape(-1, 3)
+
+
+@pytest.mark.parametrize("shape", ["left", "right", "zigzag", "balanced", "steps", "random"])
+@pytest.mark.parametrize("n", [2, 31, 32, 33, 64, 257, 290, 1024, 1025, 2100, 4500])
+def test_chosen_trees(shape, n):
+    import torch
+    import paper_2008_01938_gb300 as dp
+    s, ref = _tree(shape, n, n)
+    got = dp.mcm_traceback(torch.from_numpy(s).cuda())
+    dp.sync_status()
+    assert np.array_equal(got.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("n,at", [(20, (3, 9)), (600, (300, 599)), (3000, (0, 2999)), (3000, (1500, 2999))])
+def test_a_split_outside_its_subtree_is_reported(n, at):
+    import torch
+    import paper_2008_01938_gb300 as dp
+    s, ref = _tree("balanced", n, 1)
+    nodes = {(int(i), int(j)) for i, _, j in ref}
+    i, j = at if at in nodes else next(iter(sorted(nodes)))
+    s[i, j] = j
+    dp.mcm_traceback(torch.from_numpy(s).cuda())
+    with pytest.raises(dp.native.DpError) as e:
+        dp.sync_status()
+    assert e.value.code == dp.native.DP_EINVAL
