@@ -237,7 +237,8 @@ dp_status mcm_plan_autotune(void *plan, const int32_t *p_all, const int64_t *p_o
                             int32_t *status_dev, void *stream);
 
 /* The configuration a plan currently uses (defaults until autotuned):
- * levels per bulk task, and resident blocks per SM (0 = the occupancy limit). */
+ * levels per bulk task, and resident blocks per SM (0 = chosen from the plan's
+ * queue). */
 dp_status mcm_plan_config(const void *plan, int32_t *levels_per_part, int32_t *blocks_per_sm);
 
 dp_status mcm_plan_destroy(void *plan);

@@ -220,7 +220,7 @@ class McmPlan:
         return self.config()
 
     def config(self):
-        """(levels per bulk task, resident blocks per SM; 0 = occupancy limit)"""
+        """(levels per bulk task, resident blocks per SM; 0 = chosen from the queue)"""
         lpp, bps = ctypes.c_int32(), ctypes.c_int32()
         check(native.load().mcm_plan_config(self._h, ctypes.byref(lpp), ctypes.byref(bps)))
         return int(lpp.value), int(bps.value)

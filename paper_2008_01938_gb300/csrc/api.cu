@@ -168,6 +168,7 @@ dp_status mcm_build_static(const std::vector<int32_t>& ns, bool i64, std::shared
     pp_base += (int64_t)in.nt * T + 32;
     pk_base += (int64_t)in.nt * T;
     sp->split_evals += ((double)n * n * n - n) / 6.0;
+    sp->max_nt = std::max(sp->max_nt, in.nt);
   }
   sp->ntiles = tile_base;
   sp->pp_total = pp_base;
@@ -202,18 +203,14 @@ dp_status mcm_build_static(const std::vector<int32_t>& ns, bool i64, std::shared
             part.r_lo = (int16_t)r0;
             part.r_hi = (int16_t)r1;
             part.kind = 1;
-            // ready at bucket r1 + 1; int32 parts other than the last one are
-            // deferred to kDeferBuckets diagonals before their finisher (int64
-            // plans keep the readiness order)
+            // ready at bucket r1 + 1; parts other than the last one are
+            // deferred to kDeferBuckets diagonals before their finisher
             const bool last = r1 == fin_lo - 1;
-            const int bucket = (i64 || last) ? r1 + 1 : std::max(r1 + 1, D - dpk::kDeferBuckets);
-            items.push_back({SortKey{bucket, 1, i64 ? 0 : D, (int32_t)b, I, J}, part});
+            const int bucket = last ? r1 + 1 : std::max(r1 + 1, D - dpk::kDeferBuckets);
+            items.push_back({SortKey{bucket, 1, D, (int32_t)b, I, J}, part});
             ++nparts;
           };
-          if (i64) {
-            for (int r0 = rmin; r0 < fin_lo; r0 += kLevelsPerPart)
-              add_part(r0, std::min(r0 + kLevelsPerPart - 1, fin_lo - 1));
-          } else if (fin_lo > rmin) {
+          if (fin_lo > rmin) {
             int r1 = fin_lo - 1;
             int r0 = std::max(rmin, r1 - dpk::kLastPartLevels + 1);
             add_part(r0, r1);
@@ -326,7 +323,14 @@ dp_status mcm_enqueue(const McmStatic& sp, const McmLayout& L, void* ws, const i
     return fail_cuda(e, "launch weight pass");
   if ((e = dpk::launch_mcm_prologue(a, sp.i64, st)) != cudaSuccess) return fail_cuda(e, "launch MCM prologue");
   const int c = sp.i64 ? 1 : 0;
-  const int bps = blocks_per_sm > 0 ? std::min(blocks_per_sm, ds->occ[c]) : ds->occ[c];
+  // int64 costs, where the queue holds fewer tasks per tile-diagonal than half
+  // as many again as there are SMs: one block per SM, which leaves a finisher's
+  // 64-bit arithmetic the SM to itself (n = 1500, 60 tasks: 927 against 1226
+  // us; n = 3000, 171: 2735 against 3508; batch of 50, 64: 325 against 367);
+  // above, the work bounds the solve and two are faster (batch of 200, 287
+  // tasks: 525 against 631 us; n = 4096, 279: 5896 against 6166)
+  const bool few = sp.i64 && 2 * (int64_t)sp.tasks.size() < 3 * (int64_t)ds->sms * sp.max_nt;
+  const int bps = blocks_per_sm > 0 ? std::min(blocks_per_sm, ds->occ[c]) : few ? 1 : ds->occ[c];
   const int grid = (int)std::max<int64_t>(2, std::min<int64_t>((int64_t)ds->sms * bps, (int64_t)sp.tasks.size()));
   const bool prof = profiling();
   if (prof) profile_mark(0, st, false);
@@ -495,7 +499,7 @@ struct McmPlan {
   std::vector<int32_t> ns;
   bool i64 = false;
   int levels_per_part = dpk::kLevelsPerPart;  // queue granularity (chosen by mcm_plan_autotune)
-  int blocks_per_sm = 0;                      // resident blocks per SM, 0 = occupancy limit
+  int blocks_per_sm = 0;                      // resident blocks per SM, 0 = chosen from the queue (mcm_enqueue)
 };
 
 struct SdpPlan {

@@ -49,6 +49,7 @@ struct McmStatic {
   std::vector<int32_t> accslot;
   int64_t ntiles = 0, nslots = 0, pp_total = 0, pk_total = 0;
   double split_evals = 0;
+  int32_t max_nt = 1;                    // tiles per side of the longest chain
   // device copies (immutable after creation)
   dpk::McmTask* d_tasks = nullptr;
   int32_t* d_accslot = nullptr;

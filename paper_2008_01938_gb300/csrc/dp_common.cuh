@@ -135,34 +135,11 @@ __device__ __forceinline__ void set_status(int32_t* status, int32_t code) {
   atomicCAS(status, 0, code);
 }
 
-// Spins until *flag >= target (relaxed polling with a short sleep -- a waiting
-// finisher is usually on the critical path -- then one acquire fence).
-// Returns false (and records DP_ETIMEOUT) if `limit` cycles pass first or if
-// another block already recorded an error.
-__device__ __forceinline__ bool wait_flag_geq(const int32_t* flag, int32_t target, long long limit,
-                                              int32_t* status) {
-  if (ld_acquire(flag) >= target) return true;
-  const long long t0 = clock64();
-  uint32_t backoff = 32;
-  while (true) {
-    if (ld_relaxed(flag) >= target) {
-      fence_acquire_gpu();
-      return true;
-    }
-    if (clock64() - t0 > limit) {
-      set_status(status, DP_ETIMEOUT);
-      return false;
-    }
-    if (*reinterpret_cast<volatile const int32_t*>(status) != 0) return false;
-    __nanosleep(backoff);
-    backoff = backoff < 64 ? backoff * 2 : 64;
-  }
-}
-
-// wait_flag_geq with the sleep between polls capped at CAP ns and acquire
-// loads for the polls (int32 MCM instances: every flag wait there is,
-// directly or through the tasks that follow, on the chain of
-// tile-diagonals).
+// Spins until *flag >= target, with acquire loads and a sleep of at most CAP
+// ns between them (a waiting block is usually on the chain of tile-diagonals,
+// directly or through the tasks that follow).  Returns false (and records
+// DP_ETIMEOUT) if `limit` cycles pass first or if another block already
+// recorded an error.
 template <uint32_t CAP>
 __device__ __forceinline__ bool wait_flag_geq_cap(const int32_t* flag, int32_t target, long long limit,
                                                   int32_t* status) {

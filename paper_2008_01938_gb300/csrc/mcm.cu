@@ -1,8 +1,9 @@
 // mcm.cu -- sm_103a kernels for the matrix-chain multiplication table
-// (paper Section IV-A, Eq. (2)).  See mcm_kernels.cuh for the decomposition
+// (paper Section IV-A, Eq. (2)): the main kernel of the int32-cost and
+// interval-DP solves, and the set-up kernels of all (mcm64.cu has the main
+// kernel of the int64-cost solves).  See mcm_kernels.cuh for the decomposition
 // and the packed cost encodings.
 #include <cstdint>
-#include <type_traits>
 
 #include "dp_common.cuh"
 #include "mcm_kernels.cuh"
@@ -15,21 +16,10 @@ constexpr int T = kTile;
 constexpr uint32_t kFinPollNs = 64;   // finisher mbarrier waits (int32): longest sleep between polls
 constexpr uint32_t kFlagPollNs = 32;  // flag and counter waits (int32): longest sleep between polls
 
-// Flag wait of the int32 instances (shorter polling), or the common one.
-template <bool I64>
-__device__ __forceinline__ bool wait_flag(const int32_t* flag, int32_t target, long long limit, int32_t* status) {
-  if constexpr (I64)
-    return wait_flag_geq(flag, target, limit, status);
-  else
-    return wait_flag_geq_cap<kFlagPollNs>(flag, target, limit, status);
-}
 constexpr int kDiagRows = 2 * T;  // cell diagonals e = lj - li in [-31, 31] (dI = e + 31), one spare row
 
-template <bool I64>
-struct Cost {
-  using E = typename std::conditional<I64, unsigned long long, uint32_t>::type;
-  static constexpr int KB = I64 ? 16 : 32;  // k bits in the 64-bit (value, k) key
-};
+using E = uint32_t;      // panel entries: (m << S) | (k mod 2^S)
+constexpr int KB = 32;   // k bits in the 64-bit (value, k) key
 
 __device__ __forceinline__ int64_t tile_index(const McmInstDev& in, int I, int J) {
   return in.tile_base + (int64_t)I * in.nt - (int64_t)I * (I - 1) / 2 + (J - I);
@@ -39,24 +29,17 @@ __device__ __forceinline__ int64_t tile_index(const McmInstDev& in, int I, int J
 //
 // In-tile wavefront arrays (finisher of an off-diagonal tile) start at STA and
 // reuse the bulk-copy stages (every copy of the task has landed before they
-// are written); where they need more room than the stages, the finisher
-// buffers that follow are moved up.  Row indices of the U^T / L tables:
-//   int32: row = t + 32 for t in [-32, 63] (96 rows, constant offsets per step)
-//   int64: row = t & 63 (64 rows; saves the shared memory that keeps two
-//          int64 blocks resident per SM)
-// Rows outside t = 0 .. 30 hold zeros.
-template <bool I64>
+// are written).  Row t of the U^T / L tables, t in [-32, 63], is at t + 32 (96
+// rows, constant offsets per step); rows outside t = 0 .. 30 hold zeros.  The
+// cell-value arrays Xr / Xc live outside the stage area, so their entries for
+// cells that do not exist are set to all ones once per block and stay so
+// (every existing cell is written before it is read).
 struct Smem {
-  static constexpr int ES = I64 ? 8 : 4;
+  static constexpr int ES = 4;
   static constexpr int TILE = T * T * ES;
-  static constexpr bool kPadRows = !I64;
-  // int32: the cell-value arrays Xr / Xc live outside the stage area, so
-  // their entries for cells that do not exist are set to all ones once per
-  // block and stay so (every existing cell is written before it is read).
-  static constexpr bool kXOut = !I64;
-  static constexpr int kRows = kPadRows ? 96 : 64;
-  static constexpr int kRowOff = kPadRows ? 32 : 0;
-  static constexpr int UPW = I64 ? 34 : 36;                       // U^T pitch: 16-byte rows, conflict-free
+  static constexpr int kRows = 96;
+  static constexpr int kRowOff = 32;
+  static constexpr int UPW = 36;                                 // U^T pitch: 16-byte rows, conflict-free
   static constexpr int BARS = 0;                                 // 9 mbarriers + task slot
   static constexpr int STA = 128;                                // [group][stage] row panels
   static constexpr int STB = STA + 4 * TILE;                     // [group][stage] column panels
@@ -67,8 +50,7 @@ struct Smem {
   static constexpr int WLP = WUP + ((kRows * UPW * ES + 127) / 128) * 128;  // Lp[row(u)][lj] = m[JT+u+1][JT+lj]
   static constexpr int WPKI = WLP + kRows * T * ES;               // PKIp[row(t)] = p[IT+t+1]
   static constexpr int WPKJ = WPKI + kRows * 4;                  // PKJp[row(u)] = p[JT+u+1]
-  static constexpr int WXIN = (WPKJ + kRows * 4 + 127) / 128 * 128;  // Xr, Xc when inside the stage area
-  static constexpr int WEND = kXOut ? WXIN : WXIN + 2 * XBYTES;
+  static constexpr int WEND = (WPKJ + kRows * 4 + 127) / 128 * 128;
   static constexpr int FINU = ((STEND > WEND ? STEND : WEND) + 127) / 128 * 128;  // row panel of (I,I)
   static constexpr int FINL = FINU + TILE;                       // column panel of diagonal tile (J,J)
   static constexpr int FINBROW = FINL + TILE;                    // boundary row (one tile row)
@@ -77,11 +59,11 @@ struct Smem {
   static constexpr int FINPKJ = FINPKI + 128;                    // p[32J+1 ..] << S
   static constexpr int FINACC = FINPKJ + 128;                    // bulk-task partial minima
   static constexpr int BEST = FINACC + T * T * 8;                // running (value, k) keys
-  static constexpr int WXR = kXOut ? BEST + T * T * 8 : WXIN;    // Xr[e+31][li]: final value of cell (li, li+e)
+  static constexpr int WXR = BEST + T * T * 8;                   // Xr[e+31][li]: final value of cell (li, li+e)
   static constexpr int WXC = WXR + XBYTES;                       // Xc[e+31][lj]: final value of cell (lj-e, lj)
-  static constexpr int TOTAL = kXOut ? WXC + XBYTES : BEST + T * T * 8;
+  static constexpr int TOTAL = WXC + XBYTES;
   static constexpr int XV = STA;                                 // diagonal tiles: the tile's values
-  __host__ __device__ static constexpr int row(int t) { return kPadRows ? t + kRowOff : (t & 63); }
+  __host__ __device__ static constexpr int row(int t) { return t + kRowOff; }
   static_assert(WXR % 16 == 0 && WUP % 16 == 0 && (UPW * ES) % 16 == 0, "16-byte vector rows");
 };
 
@@ -143,68 +125,28 @@ __device__ __forceinline__ E umin(E a, E b) { return a < b ? a : b; }
 // The smallest minimising split is recovered after the tile is published, by
 // scanning the splits of each cell in increasing k.
 // ---------------------------------------------------------------------------
-template <typename E>
 struct Vec4 {
   E v[4];
 };
 
-template <typename E>
-__device__ __forceinline__ Vec4<E> lds4(const E* p) {  // 4 consecutive elements, 16-byte aligned
-  Vec4<E> r;
-  if constexpr (sizeof(E) == 4) {
-    const uint4 q = *reinterpret_cast<const uint4*>(p);
-    r.v[0] = q.x, r.v[1] = q.y, r.v[2] = q.z, r.v[3] = q.w;
-  } else {
-    const ulonglong2 q0 = *reinterpret_cast<const ulonglong2*>(p);
-    const ulonglong2 q1 = *reinterpret_cast<const ulonglong2*>(p + 2);
-    r.v[0] = q0.x, r.v[1] = q0.y, r.v[2] = q1.x, r.v[3] = q1.y;
-  }
+__device__ __forceinline__ Vec4 lds4(const E* p) {  // 4 consecutive elements, 16-byte aligned
+  Vec4 r;
+  const uint4 q = *reinterpret_cast<const uint4*>(p);
+  r.v[0] = q.x, r.v[1] = q.y, r.v[2] = q.z, r.v[3] = q.w;
   return r;
 }
 
-// a[r] for a runtime r in 0..3 (any r: only its low two bits are used) as
-// a two-level tree of predicated selects (a C conditional chain here is
-// compiled to divergent branches, which cost several times more inside the
-// wavefront step).
-template <typename E>
-__device__ __forceinline__ E sel4(int r, E a0, E a1, E a2, E a3) {
-  if constexpr (sizeof(E) == 4) {
-    uint32_t v;
-    asm("{\n\t.reg .pred p0, p1;\n\t.reg .b32 lo, hi, b;\n\t"
-        "and.b32 b, %5, 1;\n\tsetp.ne.u32 p0, b, 0;\n\tand.b32 b, %5, 2;\n\tsetp.ne.u32 p1, b, 0;\n\t"
-        "selp.b32 lo, %2, %1, p0;\n\tselp.b32 hi, %4, %3, p0;\n\tselp.b32 %0, hi, lo, p1;\n\t}"
-        : "=r"(v)
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(r));
-    return v;
-  } else {
-    unsigned long long v;
-    asm("{\n\t.reg .pred p0, p1;\n\t.reg .b64 lo, hi;\n\t.reg .b32 b;\n\t"
-        "and.b32 b, %5, 1;\n\tsetp.ne.u32 p0, b, 0;\n\tand.b32 b, %5, 2;\n\tsetp.ne.u32 p1, b, 0;\n\t"
-        "selp.b64 lo, %2, %1, p0;\n\tselp.b64 hi, %4, %3, p0;\n\tselp.b64 %0, hi, lo, p1;\n\t}"
-        : "=l"(v)
-        : "l"(a0), "l"(a1), "l"(a2), "l"(a3), "r"(r));
-    return v;
-  }
-}
-
 // a[r] where p0 and p1 are bits 0 and 1 of r, already computed.
-template <typename E>
 __device__ __forceinline__ E sel4p(bool p0, bool p1, E a0, E a1, E a2, E a3) {
   const E lo = p0 ? a1 : a0, hi = p0 ? a3 : a2;
   return p1 ? hi : lo;
 }
 
 // Shared-memory store of v at 32-bit shared address addr when p holds.
-template <typename E>
 __device__ __forceinline__ void sts_if(bool p, uint32_t addr, E v) {
-  if constexpr (sizeof(E) == 4)
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.shared.u32 [%1], %2;\n\t}" ::"r"((uint32_t)p),
-                 "r"(addr), "r"(v)
-                 : "memory");
-  else
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.shared.u64 [%1], %2;\n\t}" ::"r"((uint32_t)p),
-                 "r"(addr), "l"(v)
-                 : "memory");
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.shared.u32 [%1], %2;\n\t}" ::"r"((uint32_t)p),
+               "r"(addr), "r"(v)
+               : "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -254,27 +196,6 @@ __device__ __forceinline__ void seg_i32(const uint32_t* __restrict__ A, const ui
   }
 }
 
-// int64 costs: entries already carry the split index in their low 16 bits.
-__device__ __forceinline__ void seg_i64(const unsigned long long* __restrict__ A,
-                                        const unsigned long long* __restrict__ B,
-                                        const uint32_t* __restrict__ PK, const uint32_t (&P)[4][2],
-                                        unsigned long long (&best)[4][2], int ty, int tx) {
-#pragma unroll 4
-  for (int kk = 0; kk < T; ++kk) {
-    const ulonglong2 a01 = *reinterpret_cast<const ulonglong2*>(A + kk * T + 4 * ty);
-    const ulonglong2 a23 = *reinterpret_cast<const ulonglong2*>(A + kk * T + 4 * ty + 2);
-    const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(B + kk * T + 2 * tx);
-    const uint32_t pk = PK[kk];
-    const unsigned long long av[4] = {a01.x, a01.y, a23.x, a23.y};
-    const unsigned long long bv[2] = {b.x, b.y};
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int c = 0; c < 2; ++c)
-        best[r][c] = umin(best[r][c], (unsigned long long)P[r][c] * pk + av[r] + bv[c]);
-  }
-}
-
 // Walks the external segments of a task in the order both roles agree on.
 template <typename F>
 __device__ __forceinline__ void for_each_segment(const McmTask& t, F&& body) {
@@ -291,11 +212,9 @@ __device__ __forceinline__ void for_each_segment(const McmTask& t, F&& body) {
   }
 }
 
-template <bool I64, bool W>
-__global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(const McmLaunchArgs a) {
-  using E = typename Cost<I64>::E;
-  constexpr int KB = Cost<I64>::KB;
-  using SM = Smem<I64>;
+template <bool W>
+__global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunchArgs a) {
+  using SM = Smem;
   extern __shared__ __align__(128) uint8_t smem[];
   uint64_t* bar_full = reinterpret_cast<uint64_t*>(smem + SM::BARS);      // [g*2+st]
   uint64_t* bar_empty = bar_full + 4;                                      // [g*2+st]
@@ -320,10 +239,8 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
   const long long limit = a.spin_limit;
   int32_t* status = a.status;
 
-  if constexpr (SM::kXOut) {
-    E* x = reinterpret_cast<E*>(smem + SM::WXR);
-    for (int i = tid; i < 2 * kDiagRows * T; i += blockDim.x) x[i] = ~(E)0;
-  }
+  E* x = reinterpret_cast<E*>(smem + SM::WXR);
+  for (int i = tid; i < 2 * kDiagRows * T; i += blockDim.x) x[i] = ~(E)0;
   if (tid == 0) {
     for (int i = 0; i < 4; ++i) {
       mbar_init(&bar_full[i], 1);
@@ -376,16 +293,11 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
           const int st = u % kStages;
           const uint32_t round = u / kStages;
           if (!ok) return;
-          if constexpr (I64) {
-            ok = wait_flag<I64>(a.flags + tile_index(inst, I, K), 1, limit, status) &&
-                 wait_flag<I64>(a.flags + tile_index(inst, K, J), 1, limit, status) &&
-                 wait_flag<I64>(a.flags + tile_index(inst, K + 1, J), 1, limit, status);
-          } else {  // the three tiles' flags in one round trip when they are set
-            const int32_t* const fl[3] = {a.flags + tile_index(inst, I, K), a.flags + tile_index(inst, K, J),
-                                          a.flags + tile_index(inst, K + 1, J)};
-            const int32_t tg[3] = {1, 1, 1};
-            ok = wait_flags_geq_cap<kFlagPollNs, 3>(fl, tg, limit, status);
-          }
+          // the three tiles' flags in one round trip when they are set
+                    const int32_t* const fl[3] = {a.flags + tile_index(inst, I, K), a.flags + tile_index(inst, K, J),
+                                                  a.flags + tile_index(inst, K + 1, J)};
+                    const int32_t tg[3] = {1, 1, 1};
+                    ok = wait_flags_geq_cap<kFlagPollNs, 3>(fl, tg, limit, status);
           if (!ok) return;
           fence_proxy_async_global();
           if (!mbar_wait(&bar_empty[g * kStages + st], (round & 1u) ^ 1u, limit)) {
@@ -404,23 +316,15 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
           last_parity[g][st] = round & 1u;
         });
         if (finisher && ok) {
-          if constexpr (I64) {
-            if (D >= 1)
-              ok = wait_flag<I64>(a.flags + tile_index(inst, I, I), 1, limit, status) &&
-                   wait_flag<I64>(a.flags + tile_index(inst, J, J), 1, limit, status) &&
-                   wait_flag<I64>(a.flags + tile_index(inst, I + 1, J), 1, limit, status);
-            if (ok && task.nparts > 0) ok = wait_flag<I64>(a.counters + tidx, task.nparts, limit, status);
-          } else {
-            // tiles (I, I), (J, J), (I+1, J) and the bulk-task counter in one
-            // round trip when they are ready; a diagonal tile has no
-            // neighbours, so its own flag stands in with target 0
-            const bool nb = D >= 1;
-            const int32_t* const fl[4] = {a.flags + (nb ? tile_index(inst, I, I) : tidx),
-                                          a.flags + (nb ? tile_index(inst, J, J) : tidx),
-                                          a.flags + (nb ? tile_index(inst, I + 1, J) : tidx), a.counters + tidx};
-            const int32_t tg[4] = {nb ? 1 : 0, nb ? 1 : 0, nb ? 1 : 0, task.nparts > 0 ? (int32_t)task.nparts : 0};
-            ok = wait_flags_geq_cap<kFlagPollNs, 4>(fl, tg, limit, status);
-          }
+          // tiles (I, I), (J, J), (I+1, J) and the bulk-task counter in one
+          // round trip when they are ready; a diagonal tile has no
+          // neighbours, so its own flag stands in with target 0
+          const bool nb = D >= 1;
+          const int32_t* const fl[4] = {a.flags + (nb ? tile_index(inst, I, I) : tidx),
+                                        a.flags + (nb ? tile_index(inst, J, J) : tidx),
+                                        a.flags + (nb ? tile_index(inst, I + 1, J) : tidx), a.counters + tidx};
+          const int32_t tg[4] = {nb ? 1 : 0, nb ? 1 : 0, nb ? 1 : 0, task.nparts > 0 ? (int32_t)task.nparts : 0};
+          ok = wait_flags_geq_cap<kFlagPollNs, 4>(fl, tg, limit, status);
           if (ok) {
             fence_proxy_async_global();
             uint32_t bytes = 3 * 128;
@@ -474,12 +378,9 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
         const uint32_t round = u / kStages;
         if (!ok) return;
         bool got;
-        if constexpr (I64) {
-          got = mbar_wait(&bar_full[g * kStages + st], round & 1u, limit);
-        } else {  // a finisher's segments are on the critical path: poll more often
-          got = finisher ? mbar_wait_cap(&bar_full[g * kStages + st], round & 1u, limit, kFinPollNs)
-                         : mbar_wait(&bar_full[g * kStages + st], round & 1u, limit);
-        }
+        // a finisher's segments are on the critical path: poll more often
+                got = finisher ? mbar_wait_cap(&bar_full[g * kStages + st], round & 1u, limit, kFinPollNs)
+                               : mbar_wait(&bar_full[g * kStages + st], round & 1u, limit);
         if (!got) {
           set_status(status, DP_ETIMEOUT);
           ok = false;
@@ -488,17 +389,13 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
         const E* A = stA + (g * kStages + st) * T * T;
         const E* B = stB + (g * kStages + st) * T * T;
         const uint32_t* PK = stPK + (g * kStages + st) * 32;
-        if constexpr (I64) {
-          seg_i64(A, B, PK, P, best, ty, tx);
-        } else {
-          const int logc = S < 5 ? S : 5;
-          switch (logc) {
-            case 5: seg_i32<5>(A, B, PK, P, best, ty, tx, S, K * T); break;
-            case 4: seg_i32<4>(A, B, PK, P, best, ty, tx, S, K * T); break;
-            case 3: seg_i32<3>(A, B, PK, P, best, ty, tx, S, K * T); break;
-            case 2: seg_i32<2>(A, B, PK, P, best, ty, tx, S, K * T); break;
-            default: seg_i32<1>(A, B, PK, P, best, ty, tx, S, K * T); break;
-          }
+        const int logc = S < 5 ? S : 5;
+        switch (logc) {
+          case 5: seg_i32<5>(A, B, PK, P, best, ty, tx, S, K * T); break;
+          case 4: seg_i32<4>(A, B, PK, P, best, ty, tx, S, K * T); break;
+          case 3: seg_i32<3>(A, B, PK, P, best, ty, tx, S, K * T); break;
+          case 2: seg_i32<2>(A, B, PK, P, best, ty, tx, S, K * T); break;
+          default: seg_i32<1>(A, B, PK, P, best, ty, tx, S, K * T); break;
         }
         mbar_arrive(&bar_empty[g * kStages + st]);
       });
@@ -541,17 +438,13 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
         }
         const uint32_t fpar = fin_cnt & 1u;
         bool fin_ok;
-        if constexpr (I64)
-          fin_ok = mbar_wait(bar_fin, fpar, limit);
-        else
-          fin_ok = mbar_wait_cap(bar_fin, fpar, limit, kFinPollNs);
+        fin_ok = mbar_wait_cap(bar_fin, fpar, limit, kFinPollNs);
         if (!fin_ok) set_status(status, DP_ETIMEOUT);
         const bool go = bar_compute_and(fin_ok && *reinterpret_cast<volatile int32_t*>(status) == 0);
-        const int shiftv = I64 ? 16 : S;
         const int n = inst.n;
         unsigned long long cb[4];
         E pi[4];
-        const E pj1 = (E)(finPKJ[lane] >> shiftv);  // p[JT + lane + 1]
+        const E pj1 = (E)(finPKJ[lane] >> S);  // p[JT + lane + 1]
         if (go) {
 #pragma unroll
           for (int r = 0; r < 4; ++r) {
@@ -567,52 +460,36 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
             E* Xc = reinterpret_cast<E*>(smem + SM::WXC);
             uint32_t* PKIp = reinterpret_cast<uint32_t*>(smem + SM::WPKI);
             uint32_t* PKJp = reinterpret_cast<uint32_t*>(smem + SM::WPKJ);
-            constexpr E kInf = ~(E)0;
             // boundary split k = IT + 31: U[li][31] + m[IT+32][j] + w
-            const E brow = finBrow[lane] >> shiftv;
-            const E pI32 = (E)(finPKI[T - 1] >> shiftv);
+            const E brow = finBrow[lane] >> S;
+            const E pI32 = (E)(finPKI[T - 1] >> S);
             E m[4], wv[4];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
               const int li = 4 * w + r;
               bestS[li * T + lane] = cb[r];  // external minimum: (value, smallest k)
               wv[r] = pi[r] * pj1;
-              const E bnd = (finU[(T - 1) * T + li] >> shiftv) + brow + wv[r] * pI32;
+              const E bnd = (finU[(T - 1) * T + li] >> S) + brow + wv[r] * pI32;
               m[r] = umin((E)(cb[r] >> KB), bnd);
             }
-            if constexpr (!I64) {
-              // 16-byte vectors: 8 per row, 3 per thread (all row pitches are 16-byte multiples)
-              for (int v = tid; v < SM::kRows * T / 4; v += kComputeThreads) {
-                const int q = v >> 3, x = (v & 7) * 4, t = q - SM::kRowOff;
-                uint4 uu = make_uint4(0u, 0u, 0u, 0u), ll = make_uint4(0u, 0u, 0u, 0u);
-                if (t >= 0 && t <= T - 2) {
-                  const uint4 fu = *reinterpret_cast<const uint4*>(finU + t * T + x);
-                  const uint4 fl = *reinterpret_cast<const uint4*>(finL + t * T + x);
-                  uu = make_uint4(fu.x >> S, fu.y >> S, fu.z >> S, fu.w >> S);
-                  ll = make_uint4(fl.x >> S, fl.y >> S, fl.z >> S, fl.w >> S);
-                }
-                *reinterpret_cast<uint4*>(Up + q * SM::UPW + x) = uu;
-                *reinterpret_cast<uint4*>(Lp + q * T + x) = ll;
+            // 16-byte vectors: 8 per row, 3 per thread (all row pitches are 16-byte multiples)
+            for (int v = tid; v < SM::kRows * T / 4; v += kComputeThreads) {
+              const int q = v >> 3, x = (v & 7) * 4, t = q - SM::kRowOff;
+              uint4 uu = make_uint4(0u, 0u, 0u, 0u), ll = make_uint4(0u, 0u, 0u, 0u);
+              if (t >= 0 && t <= T - 2) {
+                const uint4 fu = *reinterpret_cast<const uint4*>(finU + t * T + x);
+                const uint4 fl = *reinterpret_cast<const uint4*>(finL + t * T + x);
+                uu = make_uint4(fu.x >> S, fu.y >> S, fu.z >> S, fu.w >> S);
+                ll = make_uint4(fl.x >> S, fl.y >> S, fl.z >> S, fl.w >> S);
               }
-            } else {
-              for (int idx = tid; idx < SM::kRows * T; idx += kComputeThreads) {
-                const int q = idx >> 5, x = idx & 31, t = q - SM::kRowOff;
-                const bool in = t >= 0 && t <= T - 2;
-                Up[q * SM::UPW + x] = in ? (finU[t * T + x] >> shiftv) : (E)0;
-                Lp[idx] = in ? (finL[t * T + x] >> shiftv) : (E)0;
-              }
-            }
-            if constexpr (!SM::kXOut) {
-              for (int idx = tid; idx < kDiagRows * T; idx += kComputeThreads) {
-                Xr[idx] = kInf;
-                Xc[idx] = kInf;
-              }
+              *reinterpret_cast<uint4*>(Up + q * SM::UPW + x) = uu;
+              *reinterpret_cast<uint4*>(Lp + q * T + x) = ll;
             }
             if (tid < SM::kRows) {
               const int t = tid - SM::kRowOff;
               const bool in = t >= 0 && t <= T - 2;
-              PKIp[tid] = in ? (finPKI[t] >> shiftv) : 0u;
-              PKJp[tid] = in ? (finPKJ[t] >> shiftv) : 0u;
+              PKIp[tid] = in ? (finPKI[t] >> S) : 0u;
+              PKJp[tid] = in ? (finPKJ[t] >> S) : 0u;
             }
             const uint32_t sXr = smem_u32(Xr), sXc = smem_u32(Xc);
             const int e_last = T - 2 - 4 * w;  // the warp's last cell, (4w, 31), is final after this step
@@ -634,101 +511,59 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
               R[(1 + r) & 3] = Lp[SM::row(u) * T + lane];
               P[(1 + r) & 3] = PKJp[SM::row(u)];
             }
-            Vec4<E> u4 = lds4(Up + SM::row(lane + T - 2) * SM::UPW + 4 * w);  // t = lane - 1 - e
+            Vec4 u4 = lds4(Up + SM::row(lane + T - 2) * SM::UPW + 4 * w);  // t = lane - 1 - e
             E pkc = (E)PKIp[SM::row(lane + T - 2)];
             bar_compute();
-            if constexpr (!I64) {
-              // int32: the 62 steps are unrolled, so every shared-memory
-              // operand is a constant offset from a per-thread base. The
-              // operands of step e + 1 (independent of the tile values) are
-              // loaded at the start of step e, so the barrier after the step
-              // does not wait for them, and each candidate is a multiply-add
-              // plus a fused add-and-minimum. The row of the cell made final
-              // is chosen with predicates computed once: bit 0 of c0 - e
-              // flips every step, bit 1 repeats every four steps.
-              const E* Lb = Lp + SM::row(4 * w) * T + lane;                 // + u * T: L row u = 4w + e + r
-              const uint32_t* PJb = PKJp + SM::row(4 * w);                  // + u
-              const E* Ub = Up + SM::row(lane - 1) * SM::UPW + 4 * w;       // - (e + 1) * UPW: t = lane - 2 - e
-              const uint32_t* PIb = PKIp + SM::row(lane - 1);               // - (e + 1)
-              const E* Xcb = Xc + (T - 1) * T + lane;                       // + e * T: X[lane - e][lane]
-              const E* Xrb = Xr + (T - 1) * T + 4 * w;                      // + e * T: X[li][li + e]
-              const uint32_t sXcw = sXc + (uint32_t)((T * T + lane) * 4);      // + e * T * 4
-              const uint32_t sXrw = sXr + (uint32_t)((T * T + lane - 1) * 4);  // + e * (T - 1) * 4
-              const bool b0e = (c0 & 1) != 0;  // bit 0 of c0 - e for even e
-              bool b1[4];                      // bit 1 of c0 - e for e = k mod 4
+            // int32: the 62 steps are unrolled, so every shared-memory
+            // operand is a constant offset from a per-thread base. The
+            // operands of step e + 1 (independent of the tile values) are
+            // loaded at the start of step e, so the barrier after the step
+            // does not wait for them, and each candidate is a multiply-add
+            // plus a fused add-and-minimum. The row of the cell made final
+            // is chosen with predicates computed once: bit 0 of c0 - e
+            // flips every step, bit 1 repeats every four steps.
+            const E* Lb = Lp + SM::row(4 * w) * T + lane;                 // + u * T: L row u = 4w + e + r
+            const uint32_t* PJb = PKJp + SM::row(4 * w);                  // + u
+            const E* Ub = Up + SM::row(lane - 1) * SM::UPW + 4 * w;       // - (e + 1) * UPW: t = lane - 2 - e
+            const uint32_t* PIb = PKIp + SM::row(lane - 1);               // - (e + 1)
+            const E* Xcb = Xc + (T - 1) * T + lane;                       // + e * T: X[lane - e][lane]
+            const E* Xrb = Xr + (T - 1) * T + 4 * w;                      // + e * T: X[li][li + e]
+            const uint32_t sXcw = sXc + (uint32_t)((T * T + lane) * 4);      // + e * T * 4
+            const uint32_t sXrw = sXr + (uint32_t)((T * T + lane - 1) * 4);  // + e * (T - 1) * 4
+            const bool b0e = (c0 & 1) != 0;  // bit 0 of c0 - e for even e
+            bool b1[4];                      // bit 1 of c0 - e for e = k mod 4
 #pragma unroll
-              for (int k = 0; k < 4; ++k) b1[k] = ((c0 - k) & 2) != 0;
+            for (int k = 0; k < 4; ++k) b1[k] = ((c0 - k) & 2) != 0;
 #pragma unroll
-              for (int e = -(T - 1); e <= T - 2; ++e) {
-                const int s4 = (e + T - 1) & 3;
-                if (e <= e_last) {
-                  const E Rn = Lb[(e + 4) * T];
-                  const uint32_t Pn = PJb[e + 4];
-                  const Vec4<E> u4n = lds4(Ub - (e + 1) * SM::UPW);
-                  const E pkcn = (E)PIb[-(e + 1)];
-                  const E xc = Xcb[e * T];             // column operand X[lane - e][lane]
-                  const Vec4<E> x4 = lds4(Xrb + e * T);  // row operands X[li][li + e]
+            for (int e = -(T - 1); e <= T - 2; ++e) {
+              const int s4 = (e + T - 1) & 3;
+              if (e <= e_last) {
+                const E Rn = Lb[(e + 4) * T];
+                const uint32_t Pn = PJb[e + 4];
+                const Vec4 u4n = lds4(Ub - (e + 1) * SM::UPW);
+                const E pkcn = (E)PIb[-(e + 1)];
+                const E xc = Xcb[e * T];             // column operand X[lane - e][lane]
+                const Vec4 x4 = lds4(Xrb + e * T);  // row operands X[li][li + e]
 #pragma unroll
-                  for (int r = 0; r < 4; ++r) {
-                    const int q = (1 + s4 + r) & 3;
-                    m[r] = __viaddmin_u32(u4.v[r] + wv[r] * pkc, xc, m[r]);
-                    m[r] = __viaddmin_u32(R[q] + wv[r] * (E)P[q], x4.v[r], m[r]);
-                  }
-                  // the lane's cell on diagonal e + 1 (row 4w + c0 - e) is final now
-                  const bool p0 = (e & 1) ? !b0e : b0e;
-                  const bool p1 = b1[(e + 32) & 3];
-                  E v = sel4p(p0, p1, m[0], m[1], m[2], m[3]);
-                  if constexpr (W) v += sel4p(p0, p1, wt[0], wt[1], wt[2], wt[3]);
-                  const bool own = (unsigned)(c0 - e) <= 3u;
-                  sts_if(own, sXrw + (uint32_t)(e * (T - 1) * 4), v);
-                  sts_if(own, sXcw + (uint32_t)(e * T * 4), v);
-                  R[(1 + s4) & 3] = Rn;
-                  P[(1 + s4) & 3] = Pn;
-                  u4 = u4n;
-                  pkc = pkcn;
+                for (int r = 0; r < 4; ++r) {
+                  const int q = (1 + s4 + r) & 3;
+                  m[r] = __viaddmin_u32(u4.v[r] + wv[r] * pkc, xc, m[r]);
+                  m[r] = __viaddmin_u32(R[q] + wv[r] * (E)P[q], x4.v[r], m[r]);
                 }
-                bar_compute();
+                // the lane's cell on diagonal e + 1 (row 4w + c0 - e) is final now
+                const bool p0 = (e & 1) ? !b0e : b0e;
+                const bool p1 = b1[(e + 32) & 3];
+                E v = sel4p(p0, p1, m[0], m[1], m[2], m[3]);
+                if constexpr (W) v += sel4p(p0, p1, wt[0], wt[1], wt[2], wt[3]);
+                const bool own = (unsigned)(c0 - e) <= 3u;
+                sts_if(own, sXrw + (uint32_t)(e * (T - 1) * 4), v);
+                sts_if(own, sXcw + (uint32_t)(e * T * 4), v);
+                R[(1 + s4) & 3] = Rn;
+                P[(1 + s4) & 3] = Pn;
+                u4 = u4n;
+                pkc = pkcn;
               }
-            } else {
-#pragma unroll 1
-            for (int eb = -(T - 1); eb <= T - 2; eb += 4) {
-#pragma unroll
-              for (int s4 = 0; s4 < 4; ++s4) {
-                const int e = eb + s4;
-                if (e <= T - 2) {
-                  if (e <= e_last) {
-                    const int dI = e + T - 1;
-                    const E xc = Xc[dI * T + lane];             // column operand X[lane - e][lane]
-                    const Vec4<E> x4 = lds4(Xr + dI * T + 4 * w);  // row operands X[li][li + e]
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                      const int q = (1 + s4 + r) & 3;
-                      const E cc = u4.v[r] + xc + wv[r] * pkc;
-                      const E cr = x4.v[r] + R[q] + wv[r] * (E)P[q];
-                      if constexpr (I64)
-                        m[r] = umin(m[r], umin(cc, cr));
-                      else
-                        m[r] = __vimin3_u32(m[r], cc, cr);
-                    }
-                    // the lane's cell on diagonal e + 1 is final now
-                    const int rr = c0 - e;
-                    const bool own = (unsigned)rr <= 3u;
-                    E v = sel4(rr, m[0], m[1], m[2], m[3]);
-                    if constexpr (W) v += sel4(rr, wt[0], wt[1], wt[2], wt[3]);
-                    sts_if(own, sXr + (uint32_t)(((dI + 1) * T + 4 * w + rr) * (int)sizeof(E)), v);
-                    sts_if(own, sXc + (uint32_t)(((dI + 1) * T + lane) * (int)sizeof(E)), v);
-                    // operands of step e + 1 (independent of the tile values)
-                    const int un = 4 * w + e + 4;
-                    R[(1 + s4) & 3] = Lp[SM::row(un) * T + lane];
-                    P[(1 + s4) & 3] = PKJp[SM::row(un)];
-                    const int tn = lane - 2 - e;
-                    u4 = lds4(Up + SM::row(tn) * SM::UPW + 4 * w);
-                    pkc = (E)PKIp[SM::row(tn)];
-                  }
-                  bar_compute();
-                }
-              }
-            }
+              bar_compute();
             }
             // ---------------- panels needed by other tiles, then publish ----------------
             const int64_t nn = n;
@@ -740,22 +575,14 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
               E pa[4];
 #pragma unroll
               for (int r = 0; r < 4; ++r) {
-                if constexpr (I64)
-                  pa[r] = ((E)vals[r] << 16) | (E)(JT + lane);
-                else
-                  pa[r] = (vals[r] << S) | (E)(lane & ((1 << (S < 5 ? S : 5)) - 1));
+                pa[r] = (vals[r] << S) | (E)(lane & ((1 << (S < 5 ? S : 5)) - 1));
               }
-              if constexpr (I64) {
-                *reinterpret_cast<ulonglong2*>(af + lane * T + 4 * w) = make_ulonglong2(pa[0], pa[1]);
-                *reinterpret_cast<ulonglong2*>(af + lane * T + 4 * w + 2) = make_ulonglong2(pa[2], pa[3]);
-              } else {
-                *reinterpret_cast<uint4*>(af + lane * T + 4 * w) = make_uint4(pa[0], pa[1], pa[2], pa[3]);
-              }
+              *reinterpret_cast<uint4*>(af + lane * T + 4 * w) = make_uint4(pa[0], pa[1], pa[2], pa[3]);
               E* bf = static_cast<E*>(a.bf);
 #pragma unroll
               for (int r = 0; r < 4; ++r) {
                 const int li = 4 * w + r;
-                const E pb = vals[r] << shiftv;
+                const E pb = vals[r] << S;
                 if (li >= 1)
                   bf[tidx * T * T + (li - 1) * T + lane] = pb;
                 else if (I >= 1)
@@ -772,17 +599,11 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
               const int li = 4 * w + r;
               const int64_t i = IT + li, j = JT + lane;
               if (i < nn && j < nn) {
-                if constexpr (I64)
-                  static_cast<int64_t*>(inst.m)[i * nn + j] = (int64_t)vals[r];
-                else
-                  static_cast<int32_t*>(inst.m)[i * nn + j] = (int32_t)vals[r];
+                static_cast<int32_t*>(inst.m)[i * nn + j] = (int32_t)vals[r];
               }
               const int64_t i2 = JT + li, j2 = IT + lane;  // mirror tile (J, I)
               if (i2 < nn && j2 < nn) {
-                if constexpr (I64)
-                  static_cast<int64_t*>(inst.m)[i2 * nn + j2] = 0;
-                else
-                  static_cast<int32_t*>(inst.m)[i2 * nn + j2] = 0;
+                static_cast<int32_t*>(inst.m)[i2 * nn + j2] = 0;
                 inst.s[i2 * nn + j2] = -1;
               }
             }
@@ -794,129 +615,101 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
             const unsigned long long kmask = (1ull << KB) - 1ull;
 #pragma unroll 1
             for (int r = 0; r < 4; ++r) {
-              // int32: warp w scans rows w, w + 8, w + 16 and w + 24, a mix of
+              // warp w scans rows w, w + 8, w + 16 and w + 24, a mix of
               // long and short column scans, so that the warps finish together
-              // (the value, weight and multiplier of the row are read again);
-              // int64: the warp's own rows 4w .. 4w + 3
-              const int li = I64 ? 4 * w + r : w + 8 * r;
+              // (the value, weight and multiplier of the row are read again)
+              const int li = w + 8 * r;
               const int64_t i = IT + li, j = JT + lane;
               if (i >= nn || j >= nn) continue;
               // (register arrays are read through sel4: a runtime index would move them to local memory)
               E v;   // the minimum, less the cell's own weight
               E wr;  // the row's multiplier p[i] p[j+1]
-              if constexpr (I64) {
-                v = sel4(r, vals[0], vals[1], vals[2], vals[3]);
-                if constexpr (W) v -= sel4(r, wt[0], wt[1], wt[2], wt[3]);
-                wr = sel4(r, wv[0], wv[1], wv[2], wv[3]);
-              } else {
-                v = Xc[(lane - li + T - 1) * T + lane];
-                if constexpr (W) v -= static_cast<const E*>(inst.w)[i * inst.n + j];
-                wr = (E)finPP[li] * pj1;
-              }
+              v = Xc[(lane - li + T - 1) * T + lane];
+              if constexpr (W) v -= static_cast<const E*>(inst.w)[i * inst.n + j];
+              wr = (E)finPP[li] * pj1;
               int k = -1;
-              if constexpr (!I64) {
-                // int32: four splits per round with independent loads, the
-                // smallest matching one kept; a lane stops after the first
-                // round with a match
-                for (int t0 = li; t0 <= T - 2 && k < 0; t0 += 4) {
-                  E c4[4];
+              // four splits per round with independent loads, the
+              // smallest matching one kept; a lane stops after the first
+              // round with a match
+              for (int t0 = li; t0 <= T - 2 && k < 0; t0 += 4) {
+                E c4[4];
 #pragma unroll
-                  for (int d = 0; d < 4; ++d) {
-                    const int t = t0 + d <= T - 2 ? t0 + d : T - 2;
-                    c4[d] = Up[SM::row(t) * SM::UPW + li] + Xc[(lane - t - 1 + T - 1) * T + lane] + wr * (E)PKIp[SM::row(t)];
-                  }
+                for (int d = 0; d < 4; ++d) {
+                  const int t = t0 + d <= T - 2 ? t0 + d : T - 2;
+                  c4[d] = Up[SM::row(t) * SM::UPW + li] + Xc[(lane - t - 1 + T - 1) * T + lane] + wr * (E)PKIp[SM::row(t)];
+                }
 #pragma unroll
-                  for (int d = 3; d >= 0; --d)
-                    if (t0 + d <= T - 2 && c4[d] == v) k = IT + t0 + d;
-                }
-              } else {
-              for (int t = li; t <= T - 2; ++t) {
-                if (Up[SM::row(t) * SM::UPW + li] + Xc[(lane - t - 1 + T - 1) * T + lane] + wr * (E)PKIp[SM::row(t)] ==
-                    v) {
-                  k = IT + t;
-                  break;
-                }
+                for (int d = 3; d >= 0; --d)
+                  if (t0 + d <= T - 2 && c4[d] == v) k = IT + t0 + d;
               }
-              }
-              if (k < 0 && (finU[(T - 1) * T + li] >> shiftv) + brow + wr * pI32 == v) k = IT + T - 1;
+              if (k < 0 && (finU[(T - 1) * T + li] >> S) + brow + wr * pI32 == v) k = IT + T - 1;
               if (k < 0) {
                 const unsigned long long ek = bestS[li * T + lane];
                 if ((E)(ek >> KB) == v) k = (int)(ek & kmask);
               }
               if (k < 0) {
-                if constexpr (!I64) {
-                  for (int u0 = 0; u0 < lane && k < 0; u0 += 4) {
-                    E c4[4];
+                for (int u0 = 0; u0 < lane && k < 0; u0 += 4) {
+                  E c4[4];
 #pragma unroll
-                    for (int d = 0; d < 4; ++d) {
-                      const int u = u0 + d <= T - 2 ? u0 + d : T - 2;
-                      c4[d] = Xr[(u - li + T - 1) * T + li] + Lp[SM::row(u) * T + lane] + wr * (E)PKJp[SM::row(u)];
-                    }
+                  for (int d = 0; d < 4; ++d) {
+                    const int u = u0 + d <= T - 2 ? u0 + d : T - 2;
+                    c4[d] = Xr[(u - li + T - 1) * T + li] + Lp[SM::row(u) * T + lane] + wr * (E)PKJp[SM::row(u)];
+                  }
 #pragma unroll
-                    for (int d = 3; d >= 0; --d)
-                      if (u0 + d < lane && c4[d] == v) k = JT + u0 + d;
-                  }
-                } else {
-                for (int u = 0; u < lane; ++u) {
-                  if (Xr[(u - li + T - 1) * T + li] + Lp[SM::row(u) * T + lane] + wr * (E)PKJp[SM::row(u)] == v) {
-                    k = JT + u;
-                    break;
-                  }
-                }
+                  for (int d = 3; d >= 0; --d)
+                    if (u0 + d < lane && c4[d] == v) k = JT + u0 + d;
                 }
               }
               inst.s[i * nn + j] = (int16_t)k;
             }
           } else {
             // diagonal tile: ordinary MCM on the 32-matrix sub-chain
-            const E pj1d = (E)(finPKI[lane] >> shiftv);
+            const E pj1d = (E)(finPKI[lane] >> S);
             bool keyed = false;
-            if constexpr (!I64) {
-              if (S == 5) {
-                // int32 with a 5-bit shift: a cell's running minimum is one
-                // 32-bit key (value << 5) + (k - IT), whose unsigned minimum
-                // keeps the smallest split on ties, as the 64-bit keys below
-                // do; final values are stored shifted in Xv, and a candidate
-                // whose operands are not both final is not taken (a select,
-                // no branch)
-                uint32_t* Xs = reinterpret_cast<uint32_t*>(Xv);
-                uint32_t key[4], pij[4];
+            if (S == 5) {
+              // int32 with a 5-bit shift: a cell's running minimum is one
+              // 32-bit key (value << 5) + (k - IT), whose unsigned minimum
+              // keeps the smallest split on ties, as the 64-bit keys below
+              // do; final values are stored shifted in Xv, and a candidate
+              // whose operands are not both final is not taken (a select,
+              // no branch)
+              uint32_t* Xs = reinterpret_cast<uint32_t*>(Xv);
+              uint32_t key[4], pij[4];
+#pragma unroll
+              for (int r = 0; r < 4; ++r) {
+                key[r] = 0xFFFFFFFFu;
+                pij[r] = pi[r] * pj1d;
+              }
+#pragma unroll 1
+              for (int e = 0; e <= T - 2; ++e) {
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                  key[r] = 0xFFFFFFFFu;
-                  pij[r] = pi[r] * pj1d;
+                  const int li = 4 * w + r;
+                  if (lane - li == e) Xs[li * T + lane] = e == 0 ? 0u : (key[r] & ~31u) + (wt[r] << 5);
                 }
-#pragma unroll 1
-                for (int e = 0; e <= T - 2; ++e) {
+                bar_compute();
 #pragma unroll
-                  for (int r = 0; r < 4; ++r) {
-                    const int li = 4 * w + r;
-                    if (lane - li == e) Xs[li * T + lane] = e == 0 ? 0u : (key[r] & ~31u) + (wt[r] << 5);
-                  }
-                  bar_compute();
-#pragma unroll
-                  for (int r = 0; r < 4; ++r) {
-                    const int li = 4 * w + r;
-                    const int f = lane - li;
-                    // split k1 = li + e: left operand on diagonal e, right on f - e - 1
-                    const bool v1 = f > e && f - e - 1 <= e;
-                    const int k1 = v1 ? li + e : 0;
-                    const uint32_t c1 = Xs[li * T + k1] + pij[r] * finPKI[k1] + (uint32_t)k1;
-                    const uint32_t n1 = __viaddmin_u32(c1, Xs[(k1 + 1) * T + lane], key[r]);
-                    // split k2 = lane - 1 - e: right operand on diagonal e, left on f - 1 - e
-                    const bool v2 = f > e && f - 1 - e < e;
-                    const int k2 = v2 ? lane - 1 - e : 0;
-                    const uint32_t c2 = Xs[li * T + k2] + pij[r] * finPKI[k2] + (uint32_t)k2;
-                    const uint32_t n2 = __viaddmin_u32(c2, Xs[(k2 + 1) * T + lane], v1 ? n1 : key[r]);
-                    key[r] = v2 ? n2 : (v1 ? n1 : key[r]);
-                  }
+                for (int r = 0; r < 4; ++r) {
+                  const int li = 4 * w + r;
+                  const int f = lane - li;
+                  // split k1 = li + e: left operand on diagonal e, right on f - e - 1
+                  const bool v1 = f > e && f - e - 1 <= e;
+                  const int k1 = v1 ? li + e : 0;
+                  const uint32_t c1 = Xs[li * T + k1] + pij[r] * finPKI[k1] + (uint32_t)k1;
+                  const uint32_t n1 = __viaddmin_u32(c1, Xs[(k1 + 1) * T + lane], key[r]);
+                  // split k2 = lane - 1 - e: right operand on diagonal e, left on f - 1 - e
+                  const bool v2 = f > e && f - 1 - e < e;
+                  const int k2 = v2 ? lane - 1 - e : 0;
+                  const uint32_t c2 = Xs[li * T + k2] + pij[r] * finPKI[k2] + (uint32_t)k2;
+                  const uint32_t n2 = __viaddmin_u32(c2, Xs[(k2 + 1) * T + lane], v1 ? n1 : key[r]);
+                  key[r] = v2 ? n2 : (v1 ? n1 : key[r]);
                 }
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-                  cb[r] = key[r] == 0xFFFFFFFFu ? ~0ull
-                                                : ((unsigned long long)(key[r] >> 5) << KB) | (unsigned)(IT + (key[r] & 31u));
-                keyed = true;
               }
+#pragma unroll
+              for (int r = 0; r < 4; ++r)
+                cb[r] = key[r] == 0xFFFFFFFFu ? ~0ull
+                                              : ((unsigned long long)(key[r] >> 5) << KB) | (unsigned)(IT + (key[r] & 31u));
+              keyed = true;
             }
 #pragma unroll 1
             for (int e = 0; e <= T - 2 && !keyed; ++e) {
@@ -933,12 +726,12 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
                 if (f > e) {
                   if (f - e - 1 <= e) {  // split k = li + e: left operand on diagonal e
                     const E cand = Xv[li * T + li + e] + Xv[(li + e + 1) * T + lane] +
-                                   pi[r] * (E)(finPKI[li + e] >> shiftv) * pj1d;
+                                   pi[r] * (E)(finPKI[li + e] >> S) * pj1d;
                     cb[r] = umin(cb[r], ((unsigned long long)cand << KB) | (unsigned)(IT + li + e));
                   }
                   if (f - 1 - e < e) {  // split k = lane - 1 - e: right operand on diagonal e
                     const E cand = Xv[li * T + lane - 1 - e] + Xv[(lane - e) * T + lane] +
-                                   pi[r] * (E)(finPKI[lane - 1 - e] >> shiftv) * pj1d;
+                                   pi[r] * (E)(finPKI[lane - 1 - e] >> S) * pj1d;
                     cb[r] = umin(cb[r], ((unsigned long long)cand << KB) | (unsigned)(IT + lane - 1 - e));
                   }
                 }
@@ -957,19 +750,13 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
             const int kk = upper ? (int)(cb[r] & kmask) : -1;
             vals[r] = v;
             if (i < nn && j < nn) {
-              if constexpr (I64)
-                static_cast<int64_t*>(inst.m)[i * nn + j] = (int64_t)v;
-              else
-                static_cast<int32_t*>(inst.m)[i * nn + j] = (int32_t)v;
+              static_cast<int32_t*>(inst.m)[i * nn + j] = (int32_t)v;
               inst.s[i * nn + j] = (int16_t)kk;
             }
             if (D >= 1) {  // mirror tile (J, I) in the lower triangle
               const int64_t i2 = JT + li, j2 = IT + lane;
               if (i2 < nn && j2 < nn) {
-                if constexpr (I64)
-                  static_cast<int64_t*>(inst.m)[i2 * nn + j2] = 0;
-                else
-                  static_cast<int32_t*>(inst.m)[i2 * nn + j2] = 0;
+                static_cast<int32_t*>(inst.m)[i2 * nn + j2] = 0;
                 inst.s[i2 * nn + j2] = -1;
               }
             }
@@ -979,23 +766,15 @@ __global__ void __launch_bounds__(kMcmThreads, I64 ? 2 : 3) mcm_main_kernel(cons
           E pa[4];
 #pragma unroll
           for (int r = 0; r < 4; ++r) {
-            if constexpr (I64)
-              pa[r] = ((E)vals[r] << 16) | (E)(JT + lane);
-            else
-              pa[r] = (vals[r] << S) | (E)(lane & ((1 << (S < 5 ? S : 5)) - 1));
+            pa[r] = (vals[r] << S) | (E)(lane & ((1 << (S < 5 ? S : 5)) - 1));
           }
-          if constexpr (I64) {
-            *reinterpret_cast<ulonglong2*>(af + lane * T + 4 * w) = make_ulonglong2(pa[0], pa[1]);
-            *reinterpret_cast<ulonglong2*>(af + lane * T + 4 * w + 2) = make_ulonglong2(pa[2], pa[3]);
-          } else {
-            *reinterpret_cast<uint4*>(af + lane * T + 4 * w) = make_uint4(pa[0], pa[1], pa[2], pa[3]);
-          }
+          *reinterpret_cast<uint4*>(af + lane * T + 4 * w) = make_uint4(pa[0], pa[1], pa[2], pa[3]);
           // packed column panel, rows shifted by one: bf[tile(X, J)][row r] = m[32X + r + 1][.]
           E* bf = static_cast<E*>(a.bf);
 #pragma unroll
           for (int r = 0; r < 4; ++r) {
             const int li = 4 * w + r;
-            const E pb = vals[r] << shiftv;
+            const E pb = vals[r] << S;
             if (li >= 1)
               bf[tidx * T * T + (li - 1) * T + lane] = pb;
             else if (I >= 1)
@@ -1124,28 +903,24 @@ __global__ void __launch_bounds__(256) mcm_prologue_kernel(const McmLaunchArgs a
 
 }  // namespace
 
-size_t mcm_smem_bytes(bool i64) { return i64 ? Smem<true>::TOTAL : Smem<false>::TOTAL; }
+size_t mcm_smem_bytes(bool i64) { return i64 ? mcm64_smem_bytes() : Smem::TOTAL; }
 
 cudaError_t mcm_configure(bool i64) {
   cudaError_t e;
-  if (i64)
-    return cudaFuncSetAttribute(mcm_main_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)Smem<true>::TOTAL);
-  if ((e = cudaFuncSetAttribute(mcm_main_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)Smem<false>::TOTAL)) != cudaSuccess)
+  if (i64) return mcm64_configure();
+  if ((e = cudaFuncSetAttribute(mcm_main_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)Smem::TOTAL)) != cudaSuccess)
     return e;
-  return cudaFuncSetAttribute(mcm_main_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)Smem<false>::TOTAL);
+  return cudaFuncSetAttribute(mcm_main_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)Smem::TOTAL);
 }
 
 // Both instances of a cost type have the same launch bounds and shared
 // memory, hence the same occupancy.
 cudaError_t mcm_occupancy(bool i64, int* blocks_per_sm) {
-  if (i64)
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, mcm_main_kernel<true, false>, kMcmThreads,
-                                                         Smem<true>::TOTAL);
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, mcm_main_kernel<false, false>, kMcmThreads,
-                                                       Smem<false>::TOTAL);
+  if (i64) return mcm64_occupancy(blocks_per_sm);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, mcm_main_kernel<false>, kMcmThreads,
+                                                       Smem::TOTAL);
 }
 
 cudaError_t mcm_preload(bool i64) {
@@ -1153,10 +928,10 @@ cudaError_t mcm_preload(bool i64) {
   cudaError_t e;
   if (i64) {
     if ((e = cudaFuncGetAttributes(&fa, mcm_prologue_kernel<true, false>)) != cudaSuccess) return e;
-    return cudaFuncGetAttributes(&fa, mcm_main_kernel<true, false>);
+    return mcm64_preload();
   }
   if ((e = cudaFuncGetAttributes(&fa, mcm_prologue_kernel<false, false>)) != cudaSuccess) return e;
-  return cudaFuncGetAttributes(&fa, mcm_main_kernel<false, false>);
+  return cudaFuncGetAttributes(&fa, mcm_main_kernel<false>);
 }
 
 // The interval DP is built for int32 costs only (see launch_mcm_weight_max
@@ -1188,10 +963,10 @@ cudaError_t launch_mcm_main(const McmLaunchArgs& a, bool i64, int grid, cudaStre
   const bool w = a.w_all != nullptr;
   if (i64) {
     if (w) return cudaErrorNotSupported;
-    mcm_main_kernel<true, false><<<grid, kMcmThreads, Smem<true>::TOTAL, st>>>(a);
+    return launch_mcm64(a, grid, st);
   } else {
-    if (w) mcm_main_kernel<false, true><<<grid, kMcmThreads, Smem<false>::TOTAL, st>>>(a);
-    else mcm_main_kernel<false, false><<<grid, kMcmThreads, Smem<false>::TOTAL, st>>>(a);
+    if (w) mcm_main_kernel<true><<<grid, kMcmThreads, Smem::TOTAL, st>>>(a);
+    else mcm_main_kernel<false><<<grid, kMcmThreads, Smem::TOTAL, st>>>(a);
   }
   return cudaGetLastError();
 }

@@ -40,6 +40,8 @@
 //     2^min(S,5) aligned splits yields the minimum and its smallest k at once.
 //   int64 costs (bound < 2^47): entries are (m << 16) | k and m << 16, so one
 //     unsigned 64-bit min yields (value, smallest k) directly.
+// The panels of a diagonal tile are read by in-tile solves only: int32, like
+// those of any tile; int64, as the tables U and L of mcm_tile.cuh.
 #pragma once
 
 #include <cstdint>
@@ -48,6 +50,7 @@
 namespace dpk {
 
 constexpr int kTile = 32;
+// the int32 main kernel's blocks
 constexpr int kGroupThreads = 128;                     // one compute group
 constexpr int kComputeThreads = 2 * kGroupThreads;     // two groups
 constexpr int kMcmThreads = kComputeThreads + 32;      // + producer warp
@@ -59,17 +62,19 @@ constexpr int kStages = 2;                             // bulk-copy stages per g
 // kMinBulkLevels bulk levels is not split at all.
 constexpr int kLevelsPerPart = 8;
 constexpr int kMinBulkLevels = 2;
-// int32 plans cut a tile's bulk levels from the top: the part that ends at
-// the last bulk level D-2 -- the part the finisher is likeliest to wait for,
-// since it becomes ready only when tile-diagonal D-2 is complete -- holds
+// A tile's bulk levels are cut from the top: the part that ends at the last
+// bulk level D-2 -- the part the finisher is likeliest to wait for, since it
+// becomes ready only when tile-diagonal D-2 is complete -- holds
 // kLastPartLevels levels, and kLevelsPerPart-level parts cover the levels
 // below it.
 constexpr int kLastPartLevels = 4;
-// Queue position of the other int32 parts: not before they become ready, and
-// not earlier than kDeferBuckets tile-diagonals before their finisher. Work
-// that is not needed soon then waits behind the tasks of the chain in the
-// middle diagonals (where blocks are scarce) and fills the blocks that the
-// last diagonals leave idle.
+// Queue position of the other parts: not before they become ready, and not
+// earlier than kDeferBuckets tile-diagonals before their finisher. Work that
+// is not needed soon then waits behind the tasks of the chain in the middle
+// diagonals (where blocks are scarce) and fills the blocks that the last
+// diagonals leave idle.  int64 chains, against parts cut from the lowest level
+// up and queued as they become ready: n = 1500 1006 -> 927 us, n = 2048 1457 ->
+// 1264, n = 4096 6154 -> 5896; batches of 50 to 2000 uneven chains within 3 %.
 constexpr int kDeferBuckets = 3;
 
 struct McmInstDev {
@@ -125,15 +130,21 @@ struct McmLaunchArgs {
   const void* w_all;
 };
 
+// The int64-cost main kernel (mcm64.cu); the functions below route to it.
+size_t mcm64_smem_bytes();
+cudaError_t mcm64_configure();
+cudaError_t mcm64_occupancy(int* blocks_per_sm);
+cudaError_t mcm64_preload();
+cudaError_t launch_mcm64(const McmLaunchArgs& a, int grid, cudaStream_t st);
+
 size_t mcm_smem_bytes(bool i64);
 cudaError_t mcm_configure(bool i64);
 cudaError_t mcm_occupancy(bool i64, int* blocks_per_sm);
 // With a.w_all set, the prologue and main kernel are the interval-DP
 // instances, and launch_mcm_weight_max must run first (it fills
 // McmInstDev::wmax, from which the prologue derives the cost bound).  The
-// interval-DP instances exist for int32 costs only: the int64 one faulted on
-// the GPU for a reason that was not found, so it is not built, and these
-// calls return cudaErrorNotSupported for i64 with weights.
+// interval DP exists for int32 costs only: these calls return
+// cudaErrorNotSupported for i64 with weights.
 cudaError_t launch_mcm_weight_max(const McmLaunchArgs& a, bool i64, int sms, cudaStream_t st);
 cudaError_t launch_mcm_prologue(const McmLaunchArgs& a, bool i64, cudaStream_t st);
 cudaError_t launch_mcm_main(const McmLaunchArgs& a, bool i64, int grid, cudaStream_t st);
