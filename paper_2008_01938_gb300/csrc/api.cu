@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
@@ -365,6 +366,17 @@ void sdp_shape(int32_t a1, int32_t ak, int* threads, int* ring_log2) {
   while ((1ll << lg) < (long long)a1 + W) ++lg;
   *threads = th;
   *ring_log2 = lg <= dpk::kSdpRingMaxLog2 ? std::max(lg, 1) : 0;
+}
+
+// Clocks per step of W = min(a_k, 1024) cells, fitted to measurements of one
+// block (clocks at 2.07 GHz): k = 4, W = 32: 161; k = 16, W = 64: 206, W = 200:
+// 266, W = 600: 530; k = 32, W = 64: 319, W = 1024: 1250; with more offsets
+// than registers k = 48, W = 64: 1030, W = 1024: 2770.
+double sdp_plain_us(int64_t cells, int32_t ak, int32_t k) {
+  if (cells <= 0) return 0.0;
+  const double W = std::min<int32_t>(ak, 1024);
+  const double clocks = 110.0 + (k > dpk::kSdpMaxKRegs ? 18.0 : 4.0) * k + W * (k + 2) / 32.0;
+  return std::ceil((double)cells / W) * clocks / 2.07e3;
 }
 
 int64_t sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g_out) {

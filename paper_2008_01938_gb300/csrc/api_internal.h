@@ -81,6 +81,8 @@ dp_status mcm_enqueue(const McmStatic& sp, const McmLayout& L, void* ws, const i
 // S-DP
 // ---------------------------------------------------------------------------
 dp_status sdp_validate(int64_t n, const int32_t* a, int32_t k, int op);
+// Approximate device time of the step kernel for `cells` cells, microseconds.
+double sdp_plain_us(int64_t cells, int32_t ak, int32_t k);
 void sdp_shape(int32_t a1, int32_t ak, int* threads, int* ring_log2);
 // (x) = min: the first cell from which the table repeats its last g cells, g
 // the gcd of the offsets (host arithmetic on the offsets only; see

@@ -349,18 +349,12 @@ namespace dph {
 
 namespace {
 // Approximate device times, in microseconds, for the choice between the
-// plain path and the jump path.  The plain kernel takes about 220 + W (k +
-// 2) / 32 clocks per step of W = min(a_k, 1024) cells (measured at k = 32:
-// 1299 clocks per step).  A Toeplitz product runs at about 14 T
-// multiply-adds/s (measured); a product modulo chi costs about 1.7 a_1^2 of
-// them in three launches, a window a_1^2, and the three launches of one
-// product level on small batches about 35 us (measured: 16, 13 and 5 us).
-double plain_us(int64_t cells, int32_t ak, int32_t k) {
-  if (cells <= 0) return 0.0;
-  const double W = std::min<int32_t>(ak, 1024);
-  const double step_us = (220.0 + W * (k + 2) / 32.0) / 2.0e3;
-  return std::ceil((double)cells / W) * step_us;
-}
+// plain path and the jump path: the step kernel's (sdp_plain_us); a Toeplitz
+// product runs at about 14 T multiply-adds/s (measured); a product modulo chi
+// costs about 1.7 a_1^2 of them in three launches, a window a_1^2, and the
+// three launches of one product level on small batches about 35 us (measured:
+// 16, 13 and 5 us).
+constexpr double kLevelUs = 35.0;
 
 int ceil_log2(int64_t x) {
   int l = 0;
@@ -411,8 +405,8 @@ double jump_us(int64_t n, int32_t A, int32_t ak, int32_t k, const JumpPlan& p) {
   const int products = p.s + (p.P2 - 1) + std::max(p.P1e - 2, 0);
   const int levels = p.s + ceil_log2(p.P2) + ceil_log2(std::max(p.P1e - 1, 1)) + 4;
   const double mads = products * 1.7 * A2 + (p.P - 1) * A2;
-  return plain_us(std::min<int64_t>(p.L, n) - A, ak, k) + plain_us(A, ak, k) +
-         std::max(plain_us(A, ak, k), plain_us(p.Gm + 1, ak, k)) + mads / 14.0e6 + levels * 35.0;
+  return sdp_plain_us(std::min<int64_t>(p.L, n) - A, ak, k) + sdp_plain_us(A, ak, k) +
+         std::max(sdp_plain_us(A, ak, k), sdp_plain_us(p.Gm + 1, ak, k)) + mads / 14.0e6 + levels * kLevelUs;
 }
 
 dp_status launch_records(const dpk::SdpInstDev* insts, int count, int32_t k, int32_t threads, int32_t ring_log2,
@@ -454,17 +448,23 @@ int sdp_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms) {
   int32_t tl = 0, rl = 0;
   sdp_shape(A, ak, &tl, &rl);
   if (rl <= 0) return 0;  // the chunks need the window on chip
-  double best = 0.8 * plain_us(n - A, ak, k);  // the jump must win clearly
+  double best = 0.8 * sdp_plain_us(n - A, ak, k);  // the jump must win clearly
+  if (best <= 4 * kLevelUs) return 0;                // less than the levels of any plan
   int bestP = 0;
-  for (int c = 2; c <= sms; ++c) {
+  auto at = [&](int c) {
     const JumpPlan p = plan_for(n, A, c, jump_reach(n, A, ak, k, c));
-    if (p.P < 2) break;
+    if (p.P < 2) return false;
     const double t = jump_us(n, A, ak, k, p);
     if (t < best) {
       best = t;
       bestP = c;
     }
-  }
+    return true;
+  };
+  // the time is flat around its minimum: a grid of about 50 counts, a twelfth
+  // apart, costs the host 10 us, every count 100
+  for (int c = 2; c <= sms; c += std::max(1, c / 12))
+    if (!at(c)) break;
   return bestP;
 }
 

@@ -398,14 +398,6 @@ __global__ void __launch_bounds__(256) mj_setup_kernel(const MjSetup s) {
 namespace dph {
 
 namespace {
-// Plain-kernel time model, microseconds: about 220 + W (k + 2) / 32 clocks
-// per step of W = min(a_k, 1024) cells at 2 GHz (measured at k = 32).
-double mj_plain_us(int64_t cells, int32_t ak, int32_t k) {
-  if (cells <= 0) return 0.0;
-  const double W = std::min<int32_t>(ak, 1024);
-  return std::ceil((double)cells / W) * (220.0 + W * (k + 2) / 32.0) / 2.0e3;
-}
-
 struct MjPlan {
   int P = 0;
   int64_t L = 0;
@@ -441,7 +433,7 @@ int mj_levels(int64_t qmax) {
 // windows.
 double mj_jump_us(int64_t n, int32_t A, int32_t ak, int32_t k, const MjPlan& p) {
   const int levels = p.s + mj_levels(p.P - 1);
-  return mj_plain_us(std::min<int64_t>(p.L, n) - A, ak, k) + mj_plain_us(A, ak, k) + 8.0 * levels + 30.0;
+  return sdp_plain_us(std::min<int64_t>(p.L, n) - A, ak, k) + sdp_plain_us(A, ak, k) + 8.0 * levels + 30.0;
 }
 
 dp_status mj_launch_records(const dpk::SdpInstDev* insts, int count, int32_t k, int32_t threads, int32_t ring_log2,
@@ -485,7 +477,7 @@ int sdp_min_jump_plan(int64_t n, const int32_t* a, int32_t k, int sms, int64_t o
 int sdp_min_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms, int64_t tail_from) {
   if (!sdp_min_jump_eligible(n, a, k)) return 0;
   const int32_t A = a[0], ak = a[k - 1];
-  double best = 0.8 * mj_plain_us((tail_from > 0 ? tail_from : n) - A, ak, k);  // the jump must win clearly
+  double best = 0.8 * sdp_plain_us((tail_from > 0 ? tail_from : n) - A, ak, k);  // the jump must win clearly
   if (best < 38.0) return 0;  // less than the jump's fixed cost and one product level
   int bestP = 0;
   for (int c = 2; c <= sms; ++c) {
