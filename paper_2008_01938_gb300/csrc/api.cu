@@ -291,14 +291,19 @@ dp_status mcm_enqueue(const McmStatic& sp, const McmLayout& L, void* ws, const i
   if (rc != DP_OK) return rc;
   uint8_t* w = static_cast<uint8_t*>(ws);
   cudaError_t e;
-  if ((e = cudaMemsetAsync(w + L.zero_begin, 0, L.zero_bytes, st)) != cudaSuccess) return fail_cuda(e, "memset flags");
   if (sp.nslots > 0 && (e = cudaMemsetAsync(w + L.acc, 0xFF, (size_t)sp.nslots * T * T * 8, st)) != cudaSuccess)
     return fail_cuda(e, "memset accumulators");
-  if ((e = cudaMemcpyAsync(w + L.insts, sp.d_insts, sp.insts.size() * sizeof(dpk::McmInstDev),
-                           cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
-    return fail_cuda(e, "copy instances");
   dpk::McmLaunchArgs a{};
   a.insts = reinterpret_cast<dpk::McmInstDev*>(w + L.insts);
+  a.zero = w + L.zero_begin;
+  a.zero_bytes = (int64_t)L.zero_bytes;
+  if (w_all) {  // the weight pass, before the prologue, adds to the records
+    if ((e = cudaMemcpyAsync(w + L.insts, sp.d_insts, sp.insts.size() * sizeof(dpk::McmInstDev),
+                             cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
+      return fail_cuda(e, "copy instances");
+  } else {
+    a.insts_from = sp.d_insts;
+  }
   a.tasks = sp.d_tasks;
   a.ninst = (int32_t)sp.insts.size();
   a.ntasks = (int32_t)sp.tasks.size();
@@ -322,7 +327,7 @@ dp_status mcm_enqueue(const McmStatic& sp, const McmLayout& L, void* ws, const i
   a.w_all = w_all;
   if (w_all && (e = dpk::launch_mcm_weight_max(a, sp.i64, ds->sms, st)) != cudaSuccess)
     return fail_cuda(e, "launch weight pass");
-  if ((e = dpk::launch_mcm_prologue(a, sp.i64, st)) != cudaSuccess) return fail_cuda(e, "launch MCM prologue");
+  if ((e = dpk::launch_mcm_prologue(a, sp.i64, sp.max_nt * T, ds->sms, st)) != cudaSuccess) return fail_cuda(e, "launch MCM prologue");
   const int c = sp.i64 ? 1 : 0;
   // int64 costs, where the queue holds fewer tasks per tile-diagonal than half
   // as many again as there are SMs: one block per SM, which leaves a finisher's

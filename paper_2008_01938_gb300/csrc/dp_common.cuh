@@ -103,6 +103,12 @@ __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
+// Programmatic dependent launch: lets the next kernel of the stream start its
+// blocks early / waits until the previous kernel has completed and its writes
+// are visible (at once when the launch does not overlap it).
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------
 // global flags
 // ---------------------------------------------------------------------------

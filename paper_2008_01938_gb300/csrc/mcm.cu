@@ -251,6 +251,8 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
   }
   __syncthreads();
 
+  grid_dependency_wait();  // the set-up kernel's writes
+
   // Per-role running counters (each role walks the same segment sequence).
   uint32_t use_cnt[2] = {0u, 0u};   // producer: stage uses issued per group; consumer: own group
   uint32_t fin_cnt = 0;             // finisher-barrier uses
@@ -831,13 +833,27 @@ __global__ void __launch_bounds__(256) mcm_weight_max_kernel(const McmLaunchArgs
 }
 
 // One block per chain: validates dims, derives the cost bound and the packing
-// shift, writes the padded / shifted dim arrays and the chain's pointers.
+// shift, writes the padded / shifted dim arrays and the chain's record.  The
+// blocks also set the flags, counters and queue to zero.  (As a memset, a copy
+// of the records and this kernel, all before the main kernel's launch, the
+// set-up took 8 of the 54 us of a 128-matrix solve.  Further blocks that set
+// the accumulators too cost more than the memset they replace: the main
+// kernel's first blocks, which take the head of the queue, are then not spread
+// over the SMs one by one, n = 1000 355 -> 360 us.)
 template <bool I64, bool W>
-__global__ void __launch_bounds__(256) mcm_prologue_kernel(const McmLaunchArgs a) {
-  __shared__ int32_t s_max[8], s_min[8];
+__global__ void __launch_bounds__(1024) mcm_prologue_kernel(const McmLaunchArgs a) {
+  __shared__ int32_t s_max[32], s_min[32];
   __shared__ int32_t s_shift;
+  launch_dependents();  // the main kernel's blocks may set themselves up meanwhile
   const int b = blockIdx.x;
+  uint4* zero = reinterpret_cast<uint4*>(a.zero);
+  for (int64_t x = (int64_t)b * blockDim.x + threadIdx.x; x < a.zero_bytes / 16; x += (int64_t)gridDim.x * blockDim.x)
+    zero[x] = make_uint4(0u, 0u, 0u, 0u);
   McmInstDev* inst = a.insts + b;
+  if (a.insts_from) {
+    if (threadIdx.x == 0) *inst = a.insts_from[b];
+    __syncthreads();
+  }
   const int n = inst->n;
   const int32_t* p = a.p_off ? a.p_all + a.p_off[b] : a.p_all;
   int32_t mx = 0, mn = 0x7fffffff;
@@ -911,8 +927,7 @@ cudaError_t mcm_configure(bool i64) {
   if ((e = cudaFuncSetAttribute(mcm_main_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)Smem::TOTAL)) != cudaSuccess)
     return e;
-  return cudaFuncSetAttribute(mcm_main_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)Smem::TOTAL);
+  return cudaFuncSetAttribute(mcm_main_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Smem::TOTAL);
 }
 
 // Both instances of a cost type have the same launch bounds and shared
@@ -945,15 +960,18 @@ cudaError_t launch_mcm_weight_max(const McmLaunchArgs& a, bool i64, int sms, cud
   return cudaGetLastError();
 }
 
-cudaError_t launch_mcm_prologue(const McmLaunchArgs& a, bool i64, cudaStream_t st) {
+cudaError_t launch_mcm_prologue(const McmLaunchArgs& a, bool i64, int max_n, int sms, cudaStream_t st) {
   if (a.ninst <= 0) return cudaSuccess;
+  // few chains: their dims in few rounds of a large block (n = 4096: 12 us with
+  // 256 threads); many chains: many small blocks per SM
+  const int threads = max_n > 256 && a.ninst <= sms ? 1024 : 256;
   const bool w = a.w_all != nullptr;
   if (i64) {
     if (w) return cudaErrorNotSupported;
-    mcm_prologue_kernel<true, false><<<a.ninst, 256, 0, st>>>(a);
+    mcm_prologue_kernel<true, false><<<a.ninst, threads, 0, st>>>(a);
   } else {
-    if (w) mcm_prologue_kernel<false, true><<<a.ninst, 256, 0, st>>>(a);
-    else mcm_prologue_kernel<false, false><<<a.ninst, 256, 0, st>>>(a);
+    if (w) mcm_prologue_kernel<false, true><<<a.ninst, threads, 0, st>>>(a);
+    else mcm_prologue_kernel<false, false><<<a.ninst, threads, 0, st>>>(a);
   }
   return cudaGetLastError();
 }
@@ -961,14 +979,9 @@ cudaError_t launch_mcm_prologue(const McmLaunchArgs& a, bool i64, cudaStream_t s
 cudaError_t launch_mcm_main(const McmLaunchArgs& a, bool i64, int grid, cudaStream_t st) {
   if (a.ntasks <= 0) return cudaSuccess;
   const bool w = a.w_all != nullptr;
-  if (i64) {
-    if (w) return cudaErrorNotSupported;
-    return launch_mcm64(a, grid, st);
-  } else {
-    if (w) mcm_main_kernel<true><<<grid, kMcmThreads, Smem::TOTAL, st>>>(a);
-    else mcm_main_kernel<false><<<grid, kMcmThreads, Smem::TOTAL, st>>>(a);
-  }
-  return cudaGetLastError();
+  if (i64) return w ? cudaErrorNotSupported : launch_mcm64(a, grid, st);
+  return w ? launch_dependent(mcm_main_kernel<true>, grid, kMcmThreads, Smem::TOTAL, st, a)
+           : launch_dependent(mcm_main_kernel<false>, grid, kMcmThreads, Smem::TOTAL, st, a);
 }
 
 }  // namespace dpk

@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) mcm64_kernel(const McmLaunc
   const int ty = tid >> 4, tx = tid & 15;  // segment reductions: cells (2 ty + r, 2 tx + c)
   const U64* const af = static_cast<const U64*>(a.af);
   const U64* const bf = static_cast<const U64*>(a.bf);
+  grid_dependency_wait();  // the set-up kernel's writes
 
   while (true) {
     if (tid == 0) {
@@ -366,8 +367,7 @@ cudaError_t mcm64_preload() {
 }
 
 cudaError_t launch_mcm64(const McmLaunchArgs& a, int grid, cudaStream_t st) {
-  mcm64_kernel<<<grid, kThreads, sizeof(Smem64), st>>>(a);
-  return cudaGetLastError();
+  return launch_dependent(mcm64_kernel, grid, kThreads, sizeof(Smem64), st, a);
 }
 
 }  // namespace dpk

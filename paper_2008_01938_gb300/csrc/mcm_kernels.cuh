@@ -103,6 +103,7 @@ struct McmTask {
 
 struct McmLaunchArgs {
   McmInstDev* insts;
+  const McmInstDev* insts_from;  // static fields of the records, copied by the prologue (nullptr: already there)
   const McmTask* tasks;
   int32_t ninst;
   int32_t ntasks;
@@ -115,6 +116,8 @@ struct McmLaunchArgs {
   int32_t* pp;                   // padded dims
   uint32_t* pk;                  // pk[x] = p[x+1] << S
   int32_t* queue;                // task counter
+  void* zero;                    // state the prologue sets to zero (16-byte aligned) ...
+  int64_t zero_bytes;            // ... and its size; 0: already done
   int32_t* status;               // device status word
   long long spin_limit;          // clock cycles a wait may take before DP_ETIMEOUT
   int32_t drop_task;             // fault injection: this queue entry is popped but never run (-1: none)
@@ -137,6 +140,27 @@ cudaError_t mcm64_occupancy(int* blocks_per_sm);
 cudaError_t mcm64_preload();
 cudaError_t launch_mcm64(const McmLaunchArgs& a, int grid, cudaStream_t st);
 
+// Launches a main kernel; the blocks of a grid of at most kEarlyGrid may become
+// resident while the previous kernel of the stream (the prologue) still runs
+// (they call grid_dependency_wait before they read anything it writes).  A
+// larger grid starts after it: placed around the prologue's blocks, two blocks
+// of a one-per-SM grid land on one SM (int64, n = 1500: 926 -> 1357 us).
+constexpr int kEarlyGrid = 64;
+template <typename K>
+cudaError_t launch_dependent(K kernel, int grid, int threads, size_t smem, cudaStream_t st, const McmLaunchArgs& a) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = grid <= kEarlyGrid ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
 size_t mcm_smem_bytes(bool i64);
 cudaError_t mcm_configure(bool i64);
 cudaError_t mcm_occupancy(bool i64, int* blocks_per_sm);
@@ -146,7 +170,7 @@ cudaError_t mcm_occupancy(bool i64, int* blocks_per_sm);
 // interval DP exists for int32 costs only: these calls return
 // cudaErrorNotSupported for i64 with weights.
 cudaError_t launch_mcm_weight_max(const McmLaunchArgs& a, bool i64, int sms, cudaStream_t st);
-cudaError_t launch_mcm_prologue(const McmLaunchArgs& a, bool i64, cudaStream_t st);
+cudaError_t launch_mcm_prologue(const McmLaunchArgs& a, bool i64, int max_n, int sms, cudaStream_t st);
 cudaError_t launch_mcm_main(const McmLaunchArgs& a, bool i64, int grid, cudaStream_t st);
 // Loads the prologue, main and split-pass kernels into the current context
 // (with lazy module loading a kernel is otherwise loaded at its first launch).
