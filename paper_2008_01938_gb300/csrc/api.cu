@@ -282,6 +282,21 @@ McmLayout mcm_layout(const McmStatic& sp) {
   return L;
 }
 
+// What decides is how many tasks the queue holds per tile-diagonal of the
+// longest chain, q.  Where they are few the chain of diagonals bounds the
+// solve, and a finisher that shares its SM with nobody is faster: int32, one /
+// two / three blocks per SM, n = 1000 (q = 34) 325 / 347 / 351 us, n = 2000 (q
+// = 92) 648 / 703 / 743, n = 2500 (q = 130) 1010 / 909 / 982, n = 3000 (q = 170)
+// 1526 / 1125 / 1241, n = 4096 (q = 279) 3373 / 2174 / 1987; batches of 50 (q =
+// 64) 189 / 196 / 199 and of 200 uneven chains (q = 287) 457 / 311 / 280.  int64,
+// one / two: n = 3000 2735 / 3508, n = 4096 6166 / 5896, batches of 50 325 / 367
+// and 200 631 / 525.
+int mcm_blocks_per_sm(int64_t ntasks, int max_nt, bool i64, int sms, int occ) {
+  const int64_t q = ntasks / std::max(max_nt, 1);
+  if (i64) return 2 * q < 3 * sms ? 1 : occ;
+  return 4 * q < 3 * sms ? 1 : 2 * q < 3 * sms ? std::min(2, occ) : occ;
+}
+
 dp_status mcm_enqueue(const McmStatic& sp, const McmLayout& L, void* ws, const int32_t* p_all,
                       const int64_t* p_off, const int64_t* tab_off, void* m_all, int16_t* s_all,
                       int32_t* status, cudaStream_t st, long long limit_override, int32_t drop_task,
@@ -329,14 +344,8 @@ dp_status mcm_enqueue(const McmStatic& sp, const McmLayout& L, void* ws, const i
     return fail_cuda(e, "launch weight pass");
   if ((e = dpk::launch_mcm_prologue(a, sp.i64, sp.max_nt * T, ds->sms, st)) != cudaSuccess) return fail_cuda(e, "launch MCM prologue");
   const int c = sp.i64 ? 1 : 0;
-  // int64 costs, where the queue holds fewer tasks per tile-diagonal than half
-  // as many again as there are SMs: one block per SM, which leaves a finisher's
-  // 64-bit arithmetic the SM to itself (n = 1500, 60 tasks: 927 against 1226
-  // us; n = 3000, 171: 2735 against 3508; batch of 50, 64: 325 against 367);
-  // above, the work bounds the solve and two are faster (batch of 200, 287
-  // tasks: 525 against 631 us; n = 4096, 279: 5896 against 6166)
-  const bool few = sp.i64 && 2 * (int64_t)sp.tasks.size() < 3 * (int64_t)ds->sms * sp.max_nt;
-  const int bps = blocks_per_sm > 0 ? std::min(blocks_per_sm, ds->occ[c]) : few ? 1 : ds->occ[c];
+  const int bps = blocks_per_sm > 0 ? std::min(blocks_per_sm, ds->occ[c])
+                                    : mcm_blocks_per_sm((int64_t)sp.tasks.size(), sp.max_nt, sp.i64, ds->sms, ds->occ[c]);
   const int grid = (int)std::max<int64_t>(2, std::min<int64_t>((int64_t)ds->sms * bps, (int64_t)sp.tasks.size()));
   const bool prof = profiling();
   if (prof) profile_mark(0, st, false);

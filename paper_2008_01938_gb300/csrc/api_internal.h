@@ -69,6 +69,8 @@ struct McmLayout {
 dp_status mcm_build_static(const std::vector<int32_t>& ns, bool i64, std::shared_ptr<McmStatic>* out,
                            bool upload = true, int levels_per_part = 0);
 McmLayout mcm_layout(const McmStatic& sp);
+// Resident blocks per SM for a queue of ntasks tasks over max_nt tile-diagonals.
+int mcm_blocks_per_sm(int64_t ntasks, int max_nt, bool i64, int sms, int occ);
 // Enqueues memsets + prologue + main kernel for a static plan on `ws`.
 // w_all != nullptr: the interval DP with per-cell weights laid out like m_all
 // (a weight pass is enqueued before the prologue).

@@ -289,7 +289,8 @@ extern "C" dp_status mcm_solve_noalloc(const int32_t* p, int32_t n, int32_t* m, 
   a.s_all = s;
   if ((e = dpk::launch_mcm_prologue(a, false, n, 1, st)) != cudaSuccess)
     return dph::fail_cuda(e, "mcm_solve_noalloc: launch prologue");
-  const int grid = (int)std::max<int64_t>(2, std::min<int64_t>((int64_t)d.sms * d.occ, ntasks));
+  const int bps = dph::mcm_blocks_per_sm(ntasks, nt, false, d.sms, d.occ);
+  const int grid = (int)std::max<int64_t>(2, std::min<int64_t>((int64_t)d.sms * bps, ntasks));
   if ((e = dpk::launch_mcm_main(a, false, grid, st)) != cudaSuccess)
     return dph::fail_cuda(e, "mcm_solve_noalloc: launch MCM kernel");
   return DP_OK;
