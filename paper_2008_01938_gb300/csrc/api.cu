@@ -106,6 +106,8 @@ dp_status current_dev(DevState** out) {
   if ((e = traceback_configure()) != cudaSuccess) return fail_cuda(e, "configure traceback kernel");
   if ((e = cudaMalloc(&ds.status, 256)) != cudaSuccess) return fail_cuda(e, "cudaMalloc(status)");
   if ((e = cudaMemset(ds.status, 0, 256)) != cudaSuccess) return fail_cuda(e, "cudaMemset(status)");
+  if ((e = cudaStreamCreateWithFlags(&ds.aux, cudaStreamNonBlocking)) != cudaSuccess)
+    return fail_cuda(e, "create plan stream");
   // keep freed stream-ordered allocations cached in the pool
   cudaMemPool_t pool;
   if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
@@ -133,27 +135,12 @@ McmStatic::~McmStatic() {
   }
 }
 
-namespace {
-using dpk::kMinBulkLevels;
-
-// Queue order: by bucket, a tile-diagonal no earlier than the one at which the
-// task becomes ready (every task therefore waits only for tasks queued before
-// it); within a bucket, finishers (the critical path) before bulk tasks, and
-// bulk tasks by the tile-diagonal of the finisher that needs them.
-struct SortKey {
-  int32_t bucket, kind, need, inst, I, J;
-  bool operator<(const SortKey& o) const {
-    return std::tie(bucket, kind, need, inst, I, J) < std::tie(o.bucket, o.kind, o.need, o.inst, o.I, o.J);
-  }
-};
-}  // namespace
-
 dp_status mcm_build_static(const std::vector<int32_t>& ns, bool i64, std::shared_ptr<McmStatic>* out, bool upload,
                            int levels_per_part) {
-  const int kLevelsPerPart = levels_per_part > 0 ? levels_per_part : dpk::kLevelsPerPart;
   auto sp = std::make_shared<McmStatic>();
   sp->i64 = i64;
   sp->ns = ns;
+  sp->levels_per_part = levels_per_part > 0 ? levels_per_part : dpk::kLevelsPerPart;
   int64_t tile_base = 0, pp_base = 0, pk_base = 0;
   for (size_t b = 0; b < ns.size(); ++b) {
     const int32_t n = ns[b];
@@ -174,88 +161,80 @@ dp_status mcm_build_static(const std::vector<int32_t>& ns, bool i64, std::shared
   sp->ntiles = tile_base;
   sp->pp_total = pp_base;
   sp->pk_total = pk_base;
-  sp->accslot.assign((size_t)tile_base, -1);
-
-  std::vector<std::pair<SortKey, dpk::McmTask>> items;
-  for (size_t b = 0; b < ns.size(); ++b) {
-    const dpk::McmInstDev& in = sp->insts[b];
-    const int nt = in.nt;
-    for (int I = 0; I < nt; ++I) {
-      for (int J = I; J < nt; ++J) {
-        const int D = J - I;
-        const int64_t tix = in.tile_base + (int64_t)I * nt - (int64_t)I * (I - 1) / 2 + (J - I);
-        dpk::McmTask fin{};
-        fin.inst = (int32_t)b;
-        fin.I = (int16_t)I;
-        fin.J = (int16_t)J;
-        fin.kind = 0;
-        fin.r_lo = 1;
-        fin.r_hi = 0;  // empty range
-        if (D >= 2) {
-          const int rmin = (D + 1) / 2, rmax = D - 1;
-          int fin_lo = rmax;  // the finisher keeps the last level (both neighbours)
-          if (fin_lo - rmin < kMinBulkLevels) fin_lo = rmin;
-          int nparts = 0;
-          auto add_part = [&](int r0, int r1) {
-            dpk::McmTask part{};
-            part.inst = (int32_t)b;
-            part.I = (int16_t)I;
-            part.J = (int16_t)J;
-            part.r_lo = (int16_t)r0;
-            part.r_hi = (int16_t)r1;
-            part.kind = 1;
-            // ready at bucket r1 + 1; parts other than the last one are
-            // deferred to kDeferBuckets diagonals before their finisher
-            const bool last = r1 == fin_lo - 1;
-            const int bucket = last ? r1 + 1 : std::max(r1 + 1, D - dpk::kDeferBuckets);
-            items.push_back({SortKey{bucket, 1, D, (int32_t)b, I, J}, part});
-            ++nparts;
-          };
-          if (fin_lo > rmin) {
-            int r1 = fin_lo - 1;
-            int r0 = std::max(rmin, r1 - dpk::kLastPartLevels + 1);
-            add_part(r0, r1);
-            for (r1 = r0 - 1; r1 >= rmin; r1 = r0 - 1) {
-              r0 = std::max(rmin, r1 - kLevelsPerPart + 1);
-              add_part(r0, r1);
-            }
-          }
-          if (nparts > 0) sp->accslot[(size_t)tix] = (int32_t)sp->nslots++;
-          fin.r_lo = (int16_t)fin_lo;
-          fin.r_hi = (int16_t)rmax;
-          fin.nparts = (int16_t)nparts;
-        }
-        items.push_back({SortKey{D, 0, 0, (int32_t)b, I, J}, fin});
-      }
-    }
+  // tiles per tile-diagonal, all chains together, and from them the bins
+  const int nb = sp->max_nt;
+  std::vector<int64_t> chains((size_t)nb + 2, 0), tiles((size_t)nb + 2, 0);
+  for (const auto& in : sp->insts) ++chains[in.nt];
+  for (int D = nb - 1, c = 0; D >= 0; --D) {  // c: chains with a diagonal D
+    c += (int)chains[D + 1];
+    tiles[D] = tiles[D + 1] + c;
   }
-  std::stable_sort(items.begin(), items.end(),
-                   [](const std::pair<SortKey, dpk::McmTask>& x, const std::pair<SortKey, dpk::McmTask>& y) {
-                     return x.first < y.first;
-                   });
-  sp->tasks.reserve(items.size());
-  for (auto& it : items) sp->tasks.push_back(it.second);
+  std::vector<int64_t> bins((size_t)3 * nb + 1, 0);
+  for (int D = 0; D < nb; ++D) {
+    const int parts = dpk::mcm_split(D, sp->levels_per_part).nparts;
+    bins[dpk::mcm_bin_finisher(D)] = tiles[D];
+    if (parts > 0) bins[dpk::mcm_bin_last(D)] = tiles[D], sp->nslots += tiles[D];
+    if (parts > 1) bins[dpk::mcm_bin_other(D)] = tiles[D] * (parts - 1);
+  }
+  for (int x = 0; x < 3 * nb; ++x) {
+    if (sp->ntasks > INT32_MAX) break;
+    sp->cursors.push_back((int32_t)sp->ntasks);
+    sp->ntasks += bins[x];
+  }
+  if (sp->ntasks > INT32_MAX) return fail(DP_EINVAL, "the chains need more than 2^31 - 1 tasks");
+  sp->cursors.push_back(0);
 
   if (!upload) {
     *out = sp;
     return DP_OK;
   }
+  DevState* ds = nullptr;
+  dp_status rc = current_dev(&ds);
+  if (rc != DP_OK) return rc;
+  sp->device = ds->device;
+  const size_t ib = sp->insts.size() * sizeof(dpk::McmInstDev), cb = sp->cursors.size() * 4;
   cudaError_t e;
-  if ((e = cudaGetDevice(&sp->device)) != cudaSuccess) return fail_cuda(e, "cudaGetDevice");
-  const size_t tb = sp->tasks.size() * sizeof(dpk::McmTask);
-  const size_t ab = sp->accslot.size() * sizeof(int32_t);
-  const size_t ib = sp->insts.size() * sizeof(dpk::McmInstDev);
-  if ((e = cudaMalloc(&sp->d_tasks, std::max<size_t>(tb, 16))) != cudaSuccess) return fail_cuda(e, "cudaMalloc(tasks)");
-  if ((e = cudaMalloc(&sp->d_accslot, std::max<size_t>(ab, 16))) != cudaSuccess) return fail_cuda(e, "cudaMalloc(accslot)");
+  int32_t* d_cursors = nullptr;
+  if ((e = cudaMalloc(&sp->d_tasks, std::max<size_t>(sp->ntasks * sizeof(dpk::McmTask), 16))) != cudaSuccess)
+    return fail_cuda(e, "cudaMalloc(tasks)");
+  if ((e = cudaMalloc(&sp->d_accslot, std::max<size_t>(sp->ntiles * 4, 16))) != cudaSuccess)
+    return fail_cuda(e, "cudaMalloc(accslot)");
   if ((e = cudaMalloc(&sp->d_insts, std::max<size_t>(ib, 16))) != cudaSuccess) return fail_cuda(e, "cudaMalloc(insts)");
-  if (tb && (e = cudaMemcpy(sp->d_tasks, sp->tasks.data(), tb, cudaMemcpyHostToDevice)) != cudaSuccess)
-    return fail_cuda(e, "upload tasks");
-  if (ab && (e = cudaMemcpy(sp->d_accslot, sp->accslot.data(), ab, cudaMemcpyHostToDevice)) != cudaSuccess)
-    return fail_cuda(e, "upload accslot");
-  if (ib && (e = cudaMemcpy(sp->d_insts, sp->insts.data(), ib, cudaMemcpyHostToDevice)) != cudaSuccess)
-    return fail_cuda(e, "upload instances");
+  if ((e = cudaMallocAsync(reinterpret_cast<void**>(&d_cursors), cb, ds->aux)) != cudaSuccess)
+    return fail_cuda(e, "allocate queue bins");
+  if ((ib && (e = cudaMemcpyAsync(sp->d_insts, sp->insts.data(), ib, cudaMemcpyHostToDevice, ds->aux)) != cudaSuccess) ||
+      (e = cudaMemcpyAsync(d_cursors, sp->cursors.data(), cb, cudaMemcpyHostToDevice, ds->aux)) != cudaSuccess)
+    rc = fail_cuda(e, "upload instances");
+  if (rc == DP_OK) rc = mcm_build_queue(*sp, d_cursors, ds->aux);
+  cudaFreeAsync(d_cursors, ds->aux);
+  if ((e = cudaStreamSynchronize(ds->aux)) != cudaSuccess && rc == DP_OK) rc = fail_cuda(e, "build queue");
+  if (rc != DP_OK) return rc;
   *out = sp;
   return DP_OK;
+}
+
+dp_status mcm_build_queue(const McmStatic& sp, int32_t* d_cursors, cudaStream_t st) {
+  dpk::McmQueueArgs q{};
+  q.insts = sp.d_insts;
+  q.tasks = sp.d_tasks;
+  q.accslot = sp.d_accslot;
+  q.cursors = d_cursors;
+  q.ninst = (int32_t)sp.insts.size();
+  q.max_nt = sp.max_nt;
+  q.levels_per_part = sp.levels_per_part;
+  const cudaError_t e = dpk::launch_mcm_queue(q, st);
+  return e == cudaSuccess ? DP_OK : fail_cuda(e, "launch queue kernel");
+}
+
+std::vector<dpk::McmTask> mcm_host_queue(const McmStatic& sp) {
+  std::vector<dpk::McmTask> tasks((size_t)sp.ntasks);
+  std::vector<int32_t> at = sp.cursors;
+  for (size_t b = 0; b < sp.insts.size(); ++b)
+    for (int I = 0; I < sp.insts[b].nt; ++I)
+      for (int J = I; J < sp.insts[b].nt; ++J)
+        dpk::mcm_tile_tasks((int32_t)b, I, J, sp.levels_per_part,
+                            [&](int bin, int, const dpk::McmTask& t) { tasks[(size_t)at[bin]++] = t; });
+  return tasks;
 }
 
 McmLayout mcm_layout(const McmStatic& sp) {
@@ -321,7 +300,7 @@ dp_status mcm_enqueue(const McmStatic& sp, const McmLayout& L, void* ws, const i
   }
   a.tasks = sp.d_tasks;
   a.ninst = (int32_t)sp.insts.size();
-  a.ntasks = (int32_t)sp.tasks.size();
+  a.ntasks = (int32_t)sp.ntasks;
   a.af = w + L.af;
   a.bf = w + L.bf;
   a.flags = reinterpret_cast<int32_t*>(w + L.flags);
@@ -345,8 +324,8 @@ dp_status mcm_enqueue(const McmStatic& sp, const McmLayout& L, void* ws, const i
   if ((e = dpk::launch_mcm_prologue(a, sp.i64, sp.max_nt * T, ds->sms, st)) != cudaSuccess) return fail_cuda(e, "launch MCM prologue");
   const int c = sp.i64 ? 1 : 0;
   const int bps = blocks_per_sm > 0 ? std::min(blocks_per_sm, ds->occ[c])
-                                    : mcm_blocks_per_sm((int64_t)sp.tasks.size(), sp.max_nt, sp.i64, ds->sms, ds->occ[c]);
-  const int grid = (int)std::max<int64_t>(2, std::min<int64_t>((int64_t)ds->sms * bps, (int64_t)sp.tasks.size()));
+                                    : mcm_blocks_per_sm(sp.ntasks, sp.max_nt, sp.i64, ds->sms, ds->occ[c]);
+  const int grid = (int)std::max<int64_t>(2, std::min<int64_t>((int64_t)ds->sms * bps, sp.ntasks));
   const bool prof = profiling();
   if (prof) profile_mark(0, st, false);
   if ((e = dpk::launch_mcm_main(a, sp.i64, std::max(grid, 1), st)) != cudaSuccess)
@@ -730,21 +709,35 @@ dp_status mcm_solve_host(const int32_t* p_host, int32_t n, dp_cost ct, void* m_h
   return rc;
 }
 
+static int32_t test_queue(const int32_t* ns, int32_t m, int32_t i64, int32_t* out, int32_t cap, bool device) {
+  if (!ns || m < 1) return -1;
+  std::shared_ptr<McmStatic> sp;
+  if (mcm_build_static(std::vector<int32_t>(ns, ns + m), i64 != 0, &sp, device) != DP_OK) return -1;
+  std::vector<dpk::McmTask> tasks((size_t)sp->ntasks);
+  if (!device) tasks = mcm_host_queue(*sp);
+  else if (cudaMemcpy(tasks.data(), sp->d_tasks, tasks.size() * sizeof(dpk::McmTask), cudaMemcpyDeviceToHost) !=
+           cudaSuccess)
+    return -1;
+  const int64_t nt = sp->ntasks;
+  for (int64_t x = 0; x < nt && x < cap && out; ++x) {
+    const dpk::McmTask& t = tasks[(size_t)x];
+    int32_t* o = out + 6 * x;
+    o[0] = t.inst, o[1] = t.I, o[2] = t.J, o[3] = t.kind, o[4] = t.r_lo, o[5] = t.r_hi;
+  }
+  return nt > INT32_MAX ? -1 : (int32_t)nt;
+}
+
 // Test hook (host only): the MCM work queue of a plan over chains of ns[0..m)
 // matrices, in pop order, 6 words per task: chain, I, J, kind (0 finisher,
 // 1 bulk part), first and last external level. Returns the number of tasks
 // (at most cap are written), or -1.
 int32_t dp_test_mcm_queue(const int32_t* ns, int32_t m, int32_t i64, int32_t* out, int32_t cap) {
-  if (!ns || m < 1) return -1;
-  std::shared_ptr<McmStatic> sp;
-  if (mcm_build_static(std::vector<int32_t>(ns, ns + m), i64 != 0, &sp, false) != DP_OK) return -1;
-  const int64_t nt = (int64_t)sp->tasks.size();
-  for (int64_t x = 0; x < nt && x < cap && out; ++x) {
-    const dpk::McmTask& t = sp->tasks[(size_t)x];
-    int32_t* o = out + 6 * x;
-    o[0] = t.inst, o[1] = t.I, o[2] = t.J, o[3] = t.kind, o[4] = t.r_lo, o[5] = t.r_hi;
-  }
-  return nt > INT32_MAX ? -1 : (int32_t)nt;
+  return test_queue(ns, m, i64, out, cap, false);
+}
+
+// Test hook: the same, read back from the device that built it.
+int32_t dp_test_mcm_device_queue(const int32_t* ns, int32_t m, int32_t i64, int32_t* out, int32_t cap) {
+  return test_queue(ns, m, i64, out, cap, true);
 }
 
 // Test hooks for the (x) = + jump path: the number of chunks sdp_solve would
@@ -943,7 +936,7 @@ dp_status mcm_plan_destroy(void* plan) {
 // Number of queue entries of a batched plan (for tests and benchmarks).
 int64_t dp_mcm_plan_tasks(void* plan) {
   auto* pl = static_cast<McmPlan*>(plan);
-  return pl ? (int64_t)pl->sp->tasks.size() : -1;
+  return pl ? pl->sp->ntasks : -1;
 }
 
 dp_status sdp_solve(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, dp_op op, int32_t* status_dev,

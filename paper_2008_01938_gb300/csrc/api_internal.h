@@ -23,6 +23,7 @@ struct DevState {
   int sms = 0;
   int occ[2] = {0, 0};        // MCM blocks per SM, int32 / int64 costs
   int32_t* status = nullptr;  // library-owned status word
+  cudaStream_t aux = nullptr; // plan building (waited for before a plan is used)
 };
 
 // Per-device state for the current device (created on first use).
@@ -45,9 +46,9 @@ struct McmStatic {
   int device = -1;
   std::vector<int32_t> ns;
   std::vector<dpk::McmInstDev> insts;   // static fields only
-  std::vector<dpk::McmTask> tasks;
-  std::vector<int32_t> accslot;
-  int64_t ntiles = 0, nslots = 0, pp_total = 0, pk_total = 0;
+  std::vector<int32_t> cursors;         // first place of each queue bin, then 0 (McmQueueArgs)
+  int64_t ntasks = 0, ntiles = 0, nslots = 0, pp_total = 0, pk_total = 0;
+  int32_t levels_per_part = 0;
   double split_evals = 0;
   int32_t max_nt = 1;                    // tiles per side of the longest chain
   // device copies (immutable after creation)
@@ -63,11 +64,15 @@ struct McmLayout {
   size_t zero_begin = 0, zero_bytes = 0, total = 0;
 };
 
-// Builds the work queue on the host; with upload=true also copies the queue,
-// slot table and chain records to fresh device memory owned by the result.
-// levels_per_part: external levels per bulk task (0 = the default).
+// Lays a plan out (host arithmetic, no queue); with upload=true the queue, the
+// slot table and the chain records are built in fresh device memory owned by
+// the result.  levels_per_part: external levels per bulk task (0 = the default).
 dp_status mcm_build_static(const std::vector<int32_t>& ns, bool i64, std::shared_ptr<McmStatic>* out,
                            bool upload = true, int levels_per_part = 0);
+// Enqueues the building of sp's queue from its records and cursors on the device.
+dp_status mcm_build_queue(const McmStatic& sp, int32_t* d_cursors, cudaStream_t st);
+// The queue on the host, in the order a single chain's has on the device.
+std::vector<dpk::McmTask> mcm_host_queue(const McmStatic& sp);
 McmLayout mcm_layout(const McmStatic& sp);
 // Resident blocks per SM for a queue of ntasks tasks over max_nt tile-diagonals.
 int mcm_blocks_per_sm(int64_t ntasks, int max_nt, bool i64, int sms, int occ);

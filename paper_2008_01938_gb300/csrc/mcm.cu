@@ -798,6 +798,32 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
   }
 }
 
+// A warp per tile row of a chain.  Single chains know each task's place in its
+// bin; the tasks of several chains take places as they come (the order inside
+// a bin does not matter to the result or to progress).
+constexpr int kQueueRows = 8;
+__global__ void __launch_bounds__(32 * kQueueRows) mcm_queue_kernel(const McmQueueArgs a) {
+  const int lane = threadIdx.x & 31, I = blockIdx.y * kQueueRows + (threadIdx.x >> 5);
+  const McmInstDev& in = a.insts[blockIdx.x];
+  if (I >= in.nt) return;
+  int32_t* slots = a.cursors + 3 * a.max_nt;
+  for (int J0 = I; J0 < in.nt; J0 += 32) {
+    const int J = J0 + lane;
+    bool split = false;
+    if (J < in.nt) {
+      split = mcm_split(J - I, a.levels_per_part).nparts > 0;
+      mcm_tile_tasks((int32_t)blockIdx.x, I, J, a.levels_per_part, [&](int bin, int place, const McmTask& t) {
+        a.tasks[a.ninst == 1 ? a.cursors[bin] + place : atomicAdd(a.cursors + bin, 1)] = t;
+      });
+    }
+    const unsigned with = __ballot_sync(0xffffffffu, split);
+    int32_t first = 0;
+    if (lane == 0 && with) first = atomicAdd(slots, __popc(with));
+    first = __shfl_sync(0xffffffffu, first, 0);
+    if (J < in.nt) a.accslot[tile_index(in, I, J)] = split ? first + __popc(with & ((1u << lane) - 1u)) : -1;
+  }
+}
+
 // Interval DP, before the prologue: the largest weight above the diagonal of
 // each chain (blockIdx.y), merged into McmInstDev::wmax; a negative weight
 // there is DP_EINVAL.  Entries on and below the diagonal are not read.
@@ -918,6 +944,13 @@ __global__ void __launch_bounds__(1024) mcm_prologue_kernel(const McmLaunchArgs 
 }
 
 }  // namespace
+
+cudaError_t launch_mcm_queue(const McmQueueArgs& a, cudaStream_t st) {
+  if (a.ninst <= 0) return cudaSuccess;
+  const dim3 grid((unsigned)a.ninst, (unsigned)((a.max_nt + kQueueRows - 1) / kQueueRows));
+  mcm_queue_kernel<<<grid, 32 * kQueueRows, 0, st>>>(a);
+  return cudaGetLastError();
+}
 
 size_t mcm_smem_bytes(bool i64) { return i64 ? mcm64_smem_bytes() : Smem::TOTAL; }
 

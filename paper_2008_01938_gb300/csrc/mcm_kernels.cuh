@@ -101,6 +101,65 @@ struct McmTask {
   int16_t kind, nparts;
 };
 
+// The tasks of a tile on tile-diagonal D: its finisher keeps the levels [lo,
+// hi], its bulk parts (0 the last one, then downwards) cover the ones below.
+struct McmSplit {
+  int lo, hi, nparts, rmin;
+};
+__host__ __device__ inline McmSplit mcm_split(int D, int levels_per_part) {
+  McmSplit t{1, 0, 0, 1};
+  if (D < 2) return t;
+  t.rmin = (D + 1) / 2;
+  t.hi = D - 1;
+  t.lo = t.hi - t.rmin < kMinBulkLevels ? t.rmin : t.hi;  // the last level: both neighbours
+  const int bulk = t.lo - t.rmin;
+  if (bulk > 0) t.nparts = 1 + (bulk > kLastPartLevels ? (bulk - kLastPartLevels + levels_per_part - 1) / levels_per_part : 0);
+  return t;
+}
+
+// The queue is sorted into bins, 3 per tile-diagonal b: the finishers of
+// diagonal b, the last parts of diagonal b + 1 and the other parts of diagonal
+// b + kDeferBuckets.  A last part is ready when diagonal b is complete; the
+// others were ready earlier, and wait behind the tasks of the chain.  So every
+// task comes after every task it waits for.
+__host__ __device__ inline int mcm_bin_finisher(int D) { return 3 * D; }
+__host__ __device__ inline int mcm_bin_last(int D) { return 3 * (D - 1) + 1; }
+__host__ __device__ inline int mcm_bin_other(int D) { return 3 * (D - kDeferBuckets) + 2; }
+static_assert(kLastPartLevels + 1 >= kDeferBuckets, "the other parts are ready in their bin");
+
+// Calls emit(bin, place, task) for each task of tile (I, J); place numbers the
+// tasks that tiles of one chain have in the bin.
+#pragma nv_exec_check_disable
+template <typename F>
+__host__ __device__ inline void mcm_tile_tasks(int32_t inst, int I, int J, int levels_per_part, F&& emit) {
+  const int D = J - I;
+  const McmSplit t = mcm_split(D, levels_per_part);
+  McmTask task{inst, (int16_t)I, (int16_t)J, (int16_t)t.lo, (int16_t)t.hi, 0, (int16_t)t.nparts};
+  emit(mcm_bin_finisher(D), I, task);
+  task.kind = 1;
+  task.nparts = 0;
+  int r1 = t.lo - 1;
+  for (int q = 0; q < t.nparts; ++q) {
+    const int r0 = r1 - (q == 0 ? kLastPartLevels : levels_per_part) + 1;
+    task.r_lo = (int16_t)(r0 > t.rmin ? r0 : t.rmin);
+    task.r_hi = (int16_t)r1;
+    if (q == 0) emit(mcm_bin_last(D), I, task);
+    else emit(mcm_bin_other(D), I * (t.nparts - 1) + q - 1, task);
+    r1 = task.r_lo - 1;
+  }
+}
+
+// Builds the queue and the split-K slots of a plan on the device.  cursors:
+// 3 max_nt first places of the bins, then the slot count (0); consumed.
+struct McmQueueArgs {
+  const McmInstDev* insts;
+  McmTask* tasks;
+  int32_t* accslot;
+  int32_t* cursors;
+  int32_t ninst, max_nt, levels_per_part;
+};
+cudaError_t launch_mcm_queue(const McmQueueArgs& a, cudaStream_t st);
+
 struct McmLaunchArgs {
   McmInstDev* insts;
   const McmInstDev* insts_from;  // static fields of the records, copied by the prologue (nullptr: already there)

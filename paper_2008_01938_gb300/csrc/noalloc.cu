@@ -94,9 +94,9 @@ int64_t queue_length(int nt) {
 __device__ __forceinline__ int part_bucket(const TileSplit& t, int q) { return part_r1(t, q) + 1; }
 
 // Writes everything a solve expects in the scratch before it starts:
-//   * the work queue, in the order the host queue builder uses (by bucket;
-//     inside a bucket the finishers of tile-diagonal b by tile row, then the
-//     bulk parts by (tile row, tile column));
+//   * the work queue, by bucket (the tile-diagonal at which a task becomes
+//     ready); inside a bucket the finishers of tile-diagonal b by tile row,
+//     then the bulk parts by (tile row, tile column);
 //   * the chain record, the per-tile accumulator slot table (slot = tile
 //     index, -1 for a tile without bulk parts);
 //   * the state that must start at zero: tile flags, bulk counters and the

@@ -153,12 +153,11 @@ dp_status launch_mcm_group(Server* S, const std::vector<Req*>& reqs, bool i64, L
     dims += reqs[b]->n + 1;
   }
   const size_t m_bytes = align_up((size_t)cells * es, 256), s_bytes = align_up((size_t)cells * 2, 256);
-  // inputs staged in pinned memory: dims | p_off | tab_off | tasks | accslot | insts
+  // inputs staged in pinned memory: dims | p_off | tab_off | queue bins | insts
   size_t off = 0;
   auto take = [&](size_t b) { size_t o = off; off = align_up(off + std::max<size_t>(b, 16), 256); return o; };
   const size_t o_dims = take((size_t)dims * 4), o_poff = take(reqs.size() * 8), o_toff = take(reqs.size() * 8);
-  const size_t o_tasks = take(sp->tasks.size() * sizeof(dpk::McmTask));
-  const size_t o_acc = take(sp->accslot.size() * 4);
+  const size_t o_bins = take(sp->cursors.size() * 4);
   const size_t o_insts = take(sp->insts.size() * sizeof(dpk::McmInstDev));
   const size_t in_bytes = off;
   const size_t o_status = take(16);
@@ -173,26 +172,29 @@ dp_status launch_mcm_group(Server* S, const std::vector<Req*>& reqs, bool i64, L
     memcpy(hp + o_dims + p_off[b] * 4, reqs[b]->dims.data(), (reqs[b]->n + 1) * 4);
   memcpy(hp + o_poff, p_off.data(), reqs.size() * 8);
   memcpy(hp + o_toff, tab_off.data(), reqs.size() * 8);
-  memcpy(hp + o_tasks, sp->tasks.data(), sp->tasks.size() * sizeof(dpk::McmTask));
-  memcpy(hp + o_acc, sp->accslot.data(), sp->accslot.size() * 4);
+  memcpy(hp + o_bins, sp->cursors.data(), sp->cursors.size() * 4);
   memcpy(hp + o_insts, sp->insts.data(), sp->insts.size() * sizeof(dpk::McmInstDev));
 
   cudaStream_t st = S->streams[L->stream];
   auto block = std::make_shared<DeviceBlock>();
   cudaError_t e = cudaMallocAsync(&block->ptr, m_bytes + s_bytes, st);
   if (e != cudaSuccess) return fail_cuda(e, "serve: table allocation");
+  // device workspace: the staged inputs | status | task queue | slot table | the solve's scratch
+  const size_t w_tasks = in_bytes + 256, w_acc = w_tasks + align_up((size_t)sp->ntasks * sizeof(dpk::McmTask), 256);
+  const size_t w_scratch = w_acc + align_up((size_t)sp->ntiles * 4, 256);
   uint8_t* ws = nullptr;
-  e = cudaMallocAsync(reinterpret_cast<void**>(&ws), in_bytes + 256 + lay.total, st);
+  e = cudaMallocAsync(reinterpret_cast<void**>(&ws), w_scratch + lay.total, st);
   if (e != cudaSuccess) return fail_cuda(e, "serve: workspace allocation");
-  uint8_t* scratch = ws + in_bytes + 256;
+  uint8_t* scratch = ws + w_scratch;
   int32_t* d_status = reinterpret_cast<int32_t*>(ws + in_bytes);
-  sp->d_tasks = reinterpret_cast<dpk::McmTask*>(ws + o_tasks);
-  sp->d_accslot = reinterpret_cast<int32_t*>(ws + o_acc);
+  sp->d_tasks = reinterpret_cast<dpk::McmTask*>(ws + w_tasks);
+  sp->d_accslot = reinterpret_cast<int32_t*>(ws + w_acc);
   sp->d_insts = reinterpret_cast<dpk::McmInstDev*>(ws + o_insts);
 
   if ((e = cudaMemcpyAsync(ws, hp, in_bytes, cudaMemcpyHostToDevice, st)) != cudaSuccess)
     return fail_cuda(e, "serve: upload");
   if ((e = cudaMemsetAsync(d_status, 0, 4, st)) != cudaSuccess) return fail_cuda(e, "serve: status");
+  if ((rc = mcm_build_queue(*sp, reinterpret_cast<int32_t*>(ws + o_bins), st)) != DP_OK) return rc;
   uint8_t* m_all = static_cast<uint8_t*>(block->ptr);
   int16_t* s_all = reinterpret_cast<int16_t*>(m_all + m_bytes);
   rc = mcm_enqueue(*sp, lay, scratch, reinterpret_cast<int32_t*>(ws + o_dims),
