@@ -82,7 +82,9 @@ __global__ void __launch_bounds__(kThreads, kBlocks) mcm64_kernel(const McmLaunc
   extern __shared__ __align__(128) uint8_t raw[];
   Smem64& sm = *reinterpret_cast<Smem64*>(raw);
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  const int ty = tid >> 4, tx = tid & 15;  // segment reductions: cells (2 ty + r, 2 tx + c)
+  // segment reductions: half the block takes the first 16 splits of every
+  // segment, half the others; cells (4 ty + r, 2 tx + c) per thread
+  const int half = tid >> 7, ty = (tid >> 4) & 7, tx = tid & 15;
   const U64* const af = static_cast<const U64*>(a.af);
   const U64* const bf = static_cast<const U64*>(a.bf);
   grid_dependency_wait();  // the set-up kernel's writes
@@ -143,7 +145,9 @@ __global__ void __launch_bounds__(kThreads, kBlocks) mcm64_kernel(const McmLaunc
       if (tid < 8) cp_async16(&sm.pk[st][4 * tid], a.pk + inst.pk_base + (int64_t)K * T + 4 * tid);
       cp_async_commit();
     };
-    U64 best[2][2] = {{kInf, kInf}, {kInf, kInf}};
+    U64 best[4][2];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) best[r][0] = best[r][1] = kInf;
     U64 ext[2][2], brow0 = 0, brow1 = 0;  // finisher: bulk minima and boundary row of its blocks' cells
     uint32_t pI32 = 0;
     if (finisher && D >= 1) {
@@ -170,12 +174,12 @@ __global__ void __launch_bounds__(kThreads, kBlocks) mcm64_kernel(const McmLaunc
     }
     if (seg.count > 0) {
       issue(0);
-      uint32_t P[2][2];
+      uint32_t P[4][2];
 #pragma unroll
-      for (int r = 0; r < 2; ++r)
+      for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int c = 0; c < 2; ++c)
-          P[r][c] = (uint32_t)a.pp[inst.pp_base + IT + 2 * ty + r] * (uint32_t)a.pp[inst.pp_base + JT + 2 * tx + c + 1];
+          P[r][c] = (uint32_t)a.pp[inst.pp_base + IT + 4 * ty + r] * (uint32_t)a.pp[inst.pp_base + JT + 2 * tx + c + 1];
 #pragma unroll 1
       for (int q = 0; q < seg.count; ++q) {
         if (q + 1 < seg.count) {
@@ -185,28 +189,48 @@ __global__ void __launch_bounds__(kThreads, kBlocks) mcm64_kernel(const McmLaunc
           cp_async_wait<0>();
         }
         __syncthreads();
-        const U64* A = sm.stage[q & 1][0] + 2 * ty;
-        const U64* B = sm.stage[q & 1][1] + 2 * tx;
-        const uint32_t* pk = sm.pk[q & 1];
-#pragma unroll 8
-        for (int k = 0; k < T; ++k) {
-          const ulonglong2 av = *reinterpret_cast<const ulonglong2*>(A + k * T);
+        const U64* A = sm.stage[q & 1][0] + half * (T / 2) * T + 4 * ty;
+        const U64* B = sm.stage[q & 1][1] + half * (T / 2) * T + 2 * tx;
+        const uint32_t* pk = sm.pk[q & 1] + half * (T / 2);
+#pragma unroll 4
+        for (int k = 0; k < T / 2; ++k) {
+          const ulonglong2 a01 = *reinterpret_cast<const ulonglong2*>(A + k * T);
+          const ulonglong2 a23 = *reinterpret_cast<const ulonglong2*>(A + k * T + 2);
           const ulonglong2 bv = *reinterpret_cast<const ulonglong2*>(B + k * T);
+          const U64 av[4] = {a01.x, a01.y, a23.x, a23.y};
           const uint32_t p = pk[k];
-          best[0][0] = umin64(best[0][0], (U64)P[0][0] * p + av.x + bv.x);
-          best[0][1] = umin64(best[0][1], (U64)P[0][1] * p + av.x + bv.y);
-          best[1][0] = umin64(best[1][0], (U64)P[1][0] * p + av.y + bv.x);
-          best[1][1] = umin64(best[1][1], (U64)P[1][1] * p + av.y + bv.y);
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            fold64(best[r][0], (U64)P[r][0] * p + av[r] + bv.x, a.one);
+            fold64(best[r][1], (U64)P[r][1] * p + av[r] + bv.y, a.one);
+          }
         }
         __syncthreads();
       }
+      // the two halves' minima; a finisher reads them from sm.best
+      ulonglong2* const mine = reinterpret_cast<ulonglong2*>(&sm.best[4 * ty * T + 2 * tx]);
+      if (half == 1) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) mine[r * (T / 2)] = make_ulonglong2(best[r][0], best[r][1]);
+      }
+      __syncthreads();
+      if (half == 0) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const ulonglong2 o = mine[r * (T / 2)];
+          best[r][0] = umin64(best[r][0], o.x);
+          best[r][1] = umin64(best[r][1], o.y);
+          if (finisher) {
+            mine[r * (T / 2)] = make_ulonglong2(best[r][0], best[r][1]);
+          } else {
+            U64* acc = a.acc + (int64_t)accslot * T * T + (4 * ty + r) * T + 2 * tx;
+            atomicMin(acc, best[r][0]);
+            atomicMin(acc + 1, best[r][1]);
+          }
+        }
+      }
     }
     if (!finisher) {
-      U64* acc = a.acc + (int64_t)accslot * T * T + 2 * tx;
-#pragma unroll
-      for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) atomicMin(acc + (2 * ty + r) * T + c, best[r][c]);
       __syncthreads();
       // release (cumulative over the block's merges before the barrier)
       if (tid == 0) red_release_add(a.counters + tidx, 1);
@@ -219,14 +243,9 @@ __global__ void __launch_bounds__(kThreads, kBlocks) mcm64_kernel(const McmLaunc
     if (D >= 1) {
       // the two blocks of 8 x 8 cells this warp owns (mcm_tile.cuh)
       const int g = lane >> 3, cc = lane & 7;
-      if (seg.count > 0) {
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-          *reinterpret_cast<ulonglong2*>(&sm.best[(2 * ty + r) * T + 2 * tx]) = make_ulonglong2(best[r][0], best[r][1]);
-      }
       cp_async_wait<0>();  // U, L and the dims, on their way since the task began
       __syncthreads();
-      const TileTabs tab{sm.u, sm.l, sm.x.xr, sm.x.xc, sm.pi, sm.pkj};
+      const TileTabs tab{sm.u, sm.l, sm.x.xr, sm.x.xc, sm.pi, sm.pkj, a.one};
       int passed = 0;  // waves whose barrier this warp has passed
 #pragma unroll 1
       for (int sl = 0; sl < 2; ++sl) {

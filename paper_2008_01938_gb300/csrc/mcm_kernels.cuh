@@ -190,6 +190,7 @@ struct McmLaunchArgs {
   // (chain b's n x n table at offset tab_off[b]); w[i][j], i < j, is added to
   // the minimum of cell (i, j), and p may then hold zeros.
   const void* w_all;
+  uint32_t one = 1;  // 1, as a value the compiler does not see (fold64 in mcm_tile.cuh)
 };
 
 // The int64-cost main kernel (mcm64.cu); the functions below route to it.
