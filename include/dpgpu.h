@@ -260,7 +260,7 @@ dp_status mcm_plan_destroy(void *plan);
  * table is cut into chunks that run side by side, each starting from a
  * window obtained by products modulo the recurrence's characteristic
  * polynomial.  That path enqueues a few dozen launches and takes a
- * workspace of a few MB from the stream-ordered allocator (released on the
+ * workspace of up to some 30 MB from the stream-ordered allocator (released on the
  * same stream).  Its result is bit-identical.
  * With DP_OP_MIN every cell from some position on is the minimum of its
  * residue class of the preset, modulo the gcd of the offsets.  Where the

@@ -18,6 +18,7 @@
 #include <tuple>
 
 #include "api_internal.h"
+#include "sdp_ntt.cuh"
 
 namespace dph {
 
@@ -104,6 +105,7 @@ dp_status current_dev(DevState** out) {
     if (ds.occ[c] < 1) ds.occ[c] = 1;
   }
   if ((e = traceback_configure()) != cudaSuccess) return fail_cuda(e, "configure traceback kernel");
+  if ((e = dpk::ntt_configure()) != cudaSuccess) return fail_cuda(e, "configure transforms");
   if ((e = cudaMalloc(&ds.status, 256)) != cudaSuccess) return fail_cuda(e, "cudaMalloc(status)");
   if ((e = cudaMemset(ds.status, 0, 256)) != cudaSuccess) return fail_cuda(e, "cudaMemset(status)");
   if ((e = cudaStreamCreateWithFlags(&ds.aux, cudaStreamNonBlocking)) != cudaSuccess)

@@ -25,9 +25,10 @@
 //   4. the windows at (i P2 + j) L by (J): the "major" ones (j = 0) from the
 //      preset via Q_i, each extended by a_1 - 1 values with the plain
 //      kernel, then the others from their major window via R_j: batched
-//      Hankel products;
-//   5. the chunks [pL, (p+1)L), one block each, side by side, by the S-DP
-//      kernel, each from its window.
+//      middle products, for a_1 in (2048, 8192] by transforms (sdp_ntt.cu) and
+//      then once more, from all of them via x^{L/2}, half a chunk further;
+//   5. the chunks [pL, (p+1)L) or their halves, one block each, side by side,
+//      by the S-DP kernel, each from its window.
 // Reduction of a product c (degree <= 2 a_1 - 2) modulo chi: let h[d] be the
 // multiple of x^{d - a_1} chi taken away at degree d, from the top down.
 // Then h[d] = c[d] + sum_j h[d + a_j], whose solution is h[d] = sum_m g[m]
@@ -43,6 +44,7 @@
 
 #include "api_internal.h"
 #include "sdp_kernels.cuh"
+#include "sdp_ntt.cuh"
 
 namespace dpk {
 namespace {
@@ -256,7 +258,9 @@ struct JumpSetup {
   int32_t A;
   int32_t P;    // chunks
   int32_t P1e;  // major windows, counting the preset's
+  int32_t W;    // windows to extend before their halves follow (0: the chunks are not halved)
   int64_t L;    // chunk length
+  int64_t WL;   // distance between the windows to extend
   int64_t ML;   // distance between major windows (P2 L)
   int64_t n;
   uint32_t* st;
@@ -265,6 +269,7 @@ struct JumpSetup {
   uint32_t* hbuf;
   SdpInstDev* insts;      // P chunk records
   SdpInstDev* ext_insts;  // P1e - 1 records extending major windows 1 .. P1e-1
+  SdpInstDev* win_insts;  // W records extending windows 0 .. W-1
   SdpInstDev* pre_insts;  // 2 records: ST up to 2A - 2, and the impulse response
 };
 
@@ -290,6 +295,15 @@ __global__ void __launch_bounds__(256) jump_setup_kernel(const JumpSetup s) {
     in.a = s.d_offs;
     in.k = s.k;
     s.insts[i] = in;
+  }
+  if (i < s.W) {
+    const int64_t pos = i * s.WL;
+    SdpInstDev in{};
+    in.st = s.st + pos;
+    in.n = s.n - pos < 2 * (int64_t)s.A - 1 ? s.n - pos : 2 * (int64_t)s.A - 1;
+    in.a = s.d_offs;
+    in.k = s.k;
+    s.win_insts[i] = in;
   }
   if (i + 1 < s.P1e) {
     const int64_t pos = (i + 1) * s.ML;
@@ -355,6 +369,12 @@ namespace {
 // three launches of one product level on small batches about 35 us (measured:
 // 16, 13 and 5 us).
 constexpr double kLevelUs = 35.0;
+// Windows by transforms (sdp_ntt.cu) where a window is long enough for them to
+// be the faster: with a_1 = 8192 63 windows take 36 us, 204 as direct products.
+// `count` windows: about 13 us per round of a block per SM, window and prime,
+// and 22.
+bool by_transforms(int32_t A) { return A > 2048 && A <= dpk::kNttMaxA; }
+double transform_us(int count, int sms) { return 22.0 + 13.0 * std::ceil(3.0 * count / sms); }
 
 int ceil_log2(int64_t x) {
   int l = 0;
@@ -373,11 +393,15 @@ struct JumpPlan {
   int64_t L0 = 0;  // <= Gm: x^L0 mod chi comes from the impulse response
   int64_t Gm = 0;  // the impulse response is computed for m <= Gm (at least A - 1)
   int s = 0;
+  // Each chunk in two halves: the window at q L + L / 2 follows from the one
+  // at q L by x^{L/2} mod chi, which the squarings pass through.
+  bool half = false;
+  int64_t chunk() const { return half ? L / 2 : L; }
 };
 
 // The plan for about `chunks` chunks with the impulse response up to Gm;
 // P = 0 when chunks of at least 2 A cells are impossible.
-JumpPlan plan_for(int64_t n, int32_t A, int chunks, int64_t Gm) {
+JumpPlan plan_for(int64_t n, int32_t A, int chunks, int64_t Gm, int sms) {
   JumpPlan p;
   if (chunks < 2 || A < 2) return p;
   const int64_t Lt = (n + chunks - 1) / chunks;
@@ -397,16 +421,20 @@ JumpPlan plan_for(int64_t n, int32_t A, int chunks, int64_t Gm) {
   p.P2 = std::max(1, (int)std::lround(std::sqrt((double)p.P)));
   p.P1 = (p.P + p.P2 - 1) / p.P2;
   p.P1e = (int)((n + (int64_t)p.P2 * p.L - 1) / ((int64_t)p.P2 * p.L));
+  p.half = by_transforms(A) && s >= 1 && p.L >= 4 * (int64_t)A && 2 * p.P <= sms;
   return p;
 }
 
-double jump_us(int64_t n, int32_t A, int32_t ak, int32_t k, const JumpPlan& p) {
+double jump_us(int64_t n, int32_t A, int32_t ak, int32_t k, const JumpPlan& p, int sms) {
   const double A2 = (double)A * A;
   const int products = p.s + (p.P2 - 1) + std::max(p.P1e - 2, 0);
   const int levels = p.s + ceil_log2(p.P2) + ceil_log2(std::max(p.P1e - 1, 1)) + 4;
-  const double mads = products * 1.7 * A2 + (p.P - 1) * A2;
-  return sdp_plain_us(std::min<int64_t>(p.L, n) - A, ak, k) + sdp_plain_us(A, ak, k) +
-         std::max(sdp_plain_us(A, ak, k), sdp_plain_us(p.Gm + 1, ak, k)) + mads / 14.0e6 + levels * kLevelUs;
+  const double mads = products * 1.7 * A2 + (by_transforms(A) ? 0.0 : (p.P - 1) * A2);
+  const double windows = by_transforms(A) ? transform_us(p.P - 1, sms) : 0.0;
+  const double halves = p.half ? transform_us(p.P, sms) + sdp_plain_us(A, ak, k) : 0.0;
+  return sdp_plain_us(std::min<int64_t>(p.chunk(), n) - A, ak, k) + sdp_plain_us(A, ak, k) +
+         std::max(sdp_plain_us(A, ak, k), sdp_plain_us(p.Gm + 1, ak, k)) + mads / 14.0e6 + windows + halves +
+         levels * kLevelUs;
 }
 
 dp_status launch_records(const dpk::SdpInstDev* insts, int count, int32_t k, int32_t threads, int32_t ring_log2,
@@ -426,13 +454,13 @@ dp_status launch_records(const dpk::SdpInstDev* insts, int count, int32_t k, int
 }
 // How far to compute the impulse response for `chunks` chunks: every
 // doubling of its reach saves one squaring and costs a longer plain run.
-int64_t jump_reach(int64_t n, int32_t A, int32_t ak, int32_t k, int chunks) {
+int64_t jump_reach(int64_t n, int32_t A, int32_t ak, int32_t k, int chunks, int sms) {
   int64_t best_gm = A - 1;
   double best = -1.0;
   for (int64_t gm : {(int64_t)A - 1, 2 * (int64_t)A, 4 * (int64_t)A, 8 * (int64_t)A, 16 * (int64_t)A}) {
-    const JumpPlan p = plan_for(n, A, chunks, gm);
+    const JumpPlan p = plan_for(n, A, chunks, gm, sms);
     if (p.P < 2) return A - 1;
-    const double t = jump_us(n, A, ak, k, p);
+    const double t = jump_us(n, A, ak, k, p, sms);
     if (best < 0.0 || t < best) {
       best = t;
       best_gm = gm;
@@ -452,18 +480,18 @@ int sdp_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms) {
   if (best <= 4 * kLevelUs) return 0;                // less than the levels of any plan
   int bestP = 0;
   auto at = [&](int c) {
-    const JumpPlan p = plan_for(n, A, c, jump_reach(n, A, ak, k, c));
+    const JumpPlan p = plan_for(n, A, c, jump_reach(n, A, ak, k, c, sms), sms);
     if (p.P < 2) return false;
-    const double t = jump_us(n, A, ak, k, p);
+    const double t = jump_us(n, A, ak, k, p, sms);
     if (t < best) {
       best = t;
       bestP = c;
     }
     return true;
   };
-  // the time is flat around its minimum: a grid of about 50 counts, a twelfth
-  // apart, costs the host 10 us, every count 100
-  for (int c = 2; c <= sms; c += std::max(1, c / 12))
+  // the time is flat around its minimum: a grid of about 80 counts, a 24th
+  // apart, costs the host 20 us, every count with five plans each 100
+  for (int c = 2; c <= sms; c += std::max(1, c / 24))
     if (!at(c)) break;
   return bestP;
 }
@@ -472,7 +500,7 @@ int sdp_jump_plan(int64_t n, const int32_t* a, int32_t k, int sms, int64_t out[8
   const int chunks = sdp_jump_chunks(n, a, k, sms);
   for (int i = 0; i < 8; ++i) out[i] = 0;
   if (chunks < 2) return 0;
-  const JumpPlan p = plan_for(n, a[0], chunks, jump_reach(n, a[0], a[k - 1], k, chunks));
+  const JumpPlan p = plan_for(n, a[0], chunks, jump_reach(n, a[0], a[k - 1], k, chunks, sms), sms);
   out[0] = p.P;
   out[1] = p.L;
   out[2] = p.L0;
@@ -492,7 +520,7 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
   if (rc != DP_OK) return rc;
   const int32_t A = a[0];
   if (A < 2) return fail(DP_EINVAL, "sdp jump: a_1 = %d, the table is constant", A);
-  const JumpPlan pl = plan_for(n, A, chunks, jump_reach(n, A, a[k - 1], k, chunks));
+  const JumpPlan pl = plan_for(n, A, chunks, jump_reach(n, A, a[k - 1], k, chunks, ds->sms), ds->sms);
   if (pl.P < 2)
     return fail(DP_EINVAL, "sdp jump: %d chunks of at least %d cells do not fit n = %lld", chunks, 2 * A,
                 (long long)n);
@@ -524,17 +552,28 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
   const size_t o_Q = take((size_t)std::max(P1e, 2) * A * 4);          // Q_0 .. Q_{P1e-1} (Q_0 unused)
   const size_t o_prod = take((size_t)nb * PS * 4);
   const size_t o_hf = take((size_t)nb * HS * 4);
+  const bool ntt = by_transforms(A);
   const int64_t nwin = std::max<int64_t>((int64_t)P1e * P2, 2);     // window scratch rows
-  const size_t o_win = take((size_t)nwin * A * 4);
+  const size_t o_win = take(ntt ? 0 : (size_t)nwin * A * 4);
   // the windows' middle products by one transposed Karatsuba step (A even,
   // and each half still a full output block of the Toeplitz kernel)
   const int64_t kh = A / 2;
-  const bool kara = A % 2 == 0 && kh >= dpk::kTB;
+  const bool kara = !ntt && A % 2 == 0 && kh >= dpk::kTB;
   const int64_t knlo = std::max<int64_t>({(int64_t)P1e, (int64_t)P2, 1});
   const size_t o_ku = take(kara ? (size_t)3 * knlo * kh * 4 : 0);
   const size_t o_kz = take(kara ? (size_t)3 * P1e * 2 * kh * 4 : 0);
   const size_t o_kout = take(kara ? (size_t)3 * nwin * kh * 4 : 0);
-  const size_t o_insts = take((size_t)P * sizeof(dpk::SdpInstDev));
+  // transforms: spectra of R or Q rows and of window rows, residues of a batch of windows
+  const int nchunks = (int)((n + pl.chunk() - 1) / pl.chunk());
+  const int64_t nu = std::max({P1e - 1, P2 - 1, 1}), nz = std::max(P1e, pl.half ? P : 1);
+  const int64_t npair = std::max<int64_t>({(int64_t)P1e - 1, (int64_t)P1e * (P2 - 1), pl.half ? P : 1, 1});
+  const size_t o_tab = take(ntt ? dpk::ntt_table_words() * 4 : 0);
+  const size_t o_su = take(ntt ? dpk::ntt_spectrum_words(nu) * 4 : 0);
+  const size_t o_sz = take(ntt ? dpk::ntt_spectrum_words(nz) * 4 : 0);
+  const size_t o_res = take(ntt ? (size_t)3 * npair * A * 4 : 0);
+  const size_t o_half = take(pl.half ? (size_t)A * 4 : 0);            // x^{L/2} mod chi
+  const size_t o_winrec = take(pl.half ? (size_t)P * sizeof(dpk::SdpInstDev) : 0);
+  const size_t o_insts = take((size_t)nchunks * sizeof(dpk::SdpInstDev));
   const size_t o_ext = take((size_t)std::max(P1e - 1, 1) * sizeof(dpk::SdpInstDev));
   const size_t o_pre = take(2 * sizeof(dpk::SdpInstDev));
   uint8_t* ws = nullptr;
@@ -568,9 +607,12 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
   for (int j = 0; j < k; ++j) su.offs[j] = a[j];
   su.k = k;
   su.A = A;
-  su.P = P;
+  su.P = nchunks;
   su.P1e = P1e;
-  su.L = pl.L;
+  su.W = pl.half ? P : 0;
+  su.L = pl.chunk();
+  su.WL = pl.L;
+  su.win_insts = reinterpret_cast<dpk::SdpInstDev*>(ws + o_winrec);
   su.ML = ML;
   su.n = n;
   su.st = ST;
@@ -580,7 +622,7 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
   su.insts = insts;
   su.ext_insts = ext_insts;
   su.pre_insts = pre_insts;
-  const int64_t su_n = std::max<int64_t>({(int64_t)k, (int64_t)A, (int64_t)P, (int64_t)P1e, 2});
+  const int64_t su_n = std::max<int64_t>({(int64_t)k, (int64_t)A, (int64_t)nchunks, (int64_t)P, (int64_t)P1e, 2});
   dpk::jump_setup_kernel<<<(unsigned)((su_n + 255) / 256), 256, 0, st>>>(su);
   if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaMemsetAsync(prod, 0, (size_t)nb * PS * 4, st)) != cudaSuccess)
     return done(fail_cuda(e, "sdp jump: set-up"));
@@ -718,9 +760,39 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
     return cudaSuccess;
   };
 
+  // the windows out + hi pitch_hi + lo pitch_lo (clipped at n) from the rows
+  // U_lo (stride A) and ST + hi zs_hi, by transforms
+  uint32_t* tables = reinterpret_cast<uint32_t*>(ws + o_tab);
+  uint32_t* spec_u = reinterpret_cast<uint32_t*>(ws + o_su);
+  uint32_t* spec_z = reinterpret_cast<uint32_t*>(ws + o_sz);
+  auto transforms = [&](const uint32_t* U, int64_t nlo, int64_t zs_hi, int64_t nhi, int64_t pos0, int64_t pitch_hi,
+                        int64_t pitch_lo) {
+    dpk::NttRows ru{}, rz{};
+    ru.src = U;
+    ru.pitch = A;
+    ru.len = A;
+    ru.limit = INT64_MAX;
+    ru.reverse = 1;
+    ru.rows = (int32_t)nlo;
+    rz.src = ST;
+    rz.pitch = zs_hi;
+    rz.len = 2 * (int64_t)A - 1;
+    rz.limit = n;
+    rz.rows = (int32_t)nhi;
+    if ((e = dpk::launch_ntt_forward(tables, ru, spec_u, rz, spec_z, st)) != cudaSuccess) return e;
+    return dpk::launch_ntt_windows(tables, spec_u, (int)nlo, spec_z, (int)nhi, A,
+                                   reinterpret_cast<uint32_t*>(ws + o_res), ST + pos0, pitch_hi, pitch_lo, n - pos0, st);
+  };
+
   // 3. R_1 = (x^L0)^(2^s); R_2 .. R_P2; Q_i = R_P2^i for i < P1e
-  for (int i = 0; i < pl.s; ++i)
+  if (ntt && (e = dpk::launch_ntt_tables(tables, st)) != cudaSuccess) return done(fail_cuda(e, "sdp jump: tables"));
+  uint32_t* R_half = reinterpret_cast<uint32_t*>(ws + o_half);
+  for (int i = 0; i < pl.s; ++i) {
+    if (pl.half && i == pl.s - 1 &&
+        (e = cudaMemcpyAsync(R_half, R + A, (size_t)A * 4, cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
+      return done(fail_cuda(e, "sdp jump: half power"));
     if ((e = mulmod(R + A, 0, R + A, 0, R + A, 1)) != cudaSuccess) return done(fail_cuda(e, "sdp jump: squaring"));
+  }
   if ((e = tree(R, P2)) != cudaSuccess) return done(fail_cuda(e, "sdp jump: product tree"));
   if (P1e > 1) {
     if ((e = cudaMemcpyAsync(Q + A, R + (int64_t)P2 * A, (size_t)A * 4, cudaMemcpyDeviceToDevice, st)) != cudaSuccess ||
@@ -730,17 +802,29 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
   // 4. major windows at i P2 L (1 <= i < P1e), from the preset; each
   // extended by A - 1 values; then the windows between them, from the
   // nearest major window: ST[(i P2 + j) L + t] = sum_s R_j[s] ST[i P2 L + s + t]
-  if ((e = windows(Q + A, A, 0, 0, 1, P1e - 1)) != cudaSuccess || (e = place(0, ML, ML, P1e - 1)) != cudaSuccess)
+  if (ntt) {
+    if (P1e > 1 && (e = transforms(Q + A, P1e - 1, 0, 1, ML, 0, ML)) != cudaSuccess)
+      return done(fail_cuda(e, "sdp jump: major windows"));
+  } else if ((e = windows(Q + A, A, 0, 0, 1, P1e - 1)) != cudaSuccess || (e = place(0, ML, ML, P1e - 1)) != cudaSuccess) {
     return done(fail_cuda(e, "sdp jump: major windows"));
+  }
   if ((rc = launch_records(ext_insts, P1e - 1, k, threads, ring_log2, status, st)) != DP_OK) return done(rc);
-  if (P2 > 1) {
+  if (ntt) {
+    if (P2 > 1 && (e = transforms(R + A, P2 - 1, ML, P1e, pl.L, ML, pl.L)) != cudaSuccess)
+      return done(fail_cuda(e, "sdp jump: windows"));
+    if (pl.half) {  // the windows half a chunk further, from all the others
+      if ((rc = launch_records(su.win_insts, P, k, threads, ring_log2, status, st)) != DP_OK) return done(rc);
+      if ((e = transforms(R_half, 1, pl.L, P, pl.L / 2, pl.L, 0)) != cudaSuccess)
+        return done(fail_cuda(e, "sdp jump: half windows"));
+    }
+  } else if (P2 > 1) {
     if ((e = windows(R + A, A, 0, ML, P1e, P2 - 1)) != cudaSuccess) return done(fail_cuda(e, "sdp jump: windows"));
     for (int64_t i = 0; i < P1e; ++i)
       if ((e = place(i * (P2 - 1), i * ML + pl.L, pl.L, P2 - 1)) != cudaSuccess)
         return done(fail_cuda(e, "sdp jump: windows"));
   }
   // 5. the chunks, side by side
-  if ((rc = launch_records(insts, P, k, threads, ring_log2, status, st)) != DP_OK) return done(rc);
+  if ((rc = launch_records(insts, nchunks, k, threads, ring_log2, status, st)) != DP_OK) return done(rc);
   return done(DP_OK);
 }
 
