@@ -43,6 +43,7 @@
 #include <cstdint>
 
 #include "api_internal.h"
+#include "dp_common.cuh"
 #include "sdp_kernels.cuh"
 #include "sdp_ntt.cuh"
 
@@ -54,23 +55,33 @@ namespace {
 //   CONV: out[b][t] (+)= sum_s u[b][s] z[b][t - s + zoff]
 //   CORR: out[b][t] (+)= sum_s u[b][s] z[b][t + s + zoff]
 // for t < tout, s < S, z read as 0 outside [0, zlen).  A block computes
-// kTB consecutive outputs over pieces of kSB splits: pieces blockIdx.y,
-// blockIdx.y + gridDim.y, ...  (with gridDim.y > 1 the outputs are added
-// with atomics into a zeroed buffer); blockIdx.z is the batch item.  A
+// kTB consecutive outputs over pieces of kSB splits (with gridDim.y > 1 the
+// outputs are added with atomics into a zeroed buffer); blockIdx.z is the batch item.  A
 // thread keeps kTo consecutive outputs and, per inner step of kTs splits,
 // the kTo + kTs - 1 z values they need in registers: 256 multiply-adds for
 // 12 shared-memory vector loads.  The staged z window is padded by 4 words
 // every 16, so that the 16-byte loads of a quarter-warp (threads 16 words
 // apart) fall into distinct banks.
+// Bound by the 32-bit multiply-add rate (a product of 8192 words: 3.4 us of
+// it on 152 SMs) and, with one product in a launch, by what surrounds it.  A
+// CONV block's outputs begin where its splits do, so that a piece of A words
+// is A / kTB whole blocks (plus one for the last 127 outputs) and never a
+// skew pair of half-filled ones.  Blocks of 2048 outputs rather than 4096, a
+// thread's staging loads all in flight, and sums added 32 neighbouring words
+// at a time: one squaring of 8192 words 16.8 -> 13.0 us and its reduction
+// 13.6 -> 9.8, four of each 36 -> 27.7 and 29.3 -> 21.3 (cold cache).  With
+// early launches and pieces of 64 splits for the products, 2^24 cells: a_1 =
+// 8192, k = 32: 748 -> 599 us, a_1 = 12000: 1423 -> 997.
 // ---------------------------------------------------------------------------
-constexpr int kTT = 256;                // threads per block
+constexpr int kTT = 128;                // threads per block
 constexpr int kTo = 16;                 // outputs per thread
 constexpr int kTs = 16;                 // splits per inner step
 constexpr int kTB = kTT * kTo;          // outputs per block
-constexpr int kSB = 128;                // splits per piece
-constexpr int kZW = kTB + kSB + 32;     // staged z words
+// splits per piece: short pieces for the products, of which a launch has few;
+// longer ones, which stage less per multiply-add, for the windows
+constexpr int kSBProduct = 64;
+constexpr int kSBWindow = 128;
 __host__ __device__ constexpr int zpad(int i) { return i + 4 * (i >> 4); }
-constexpr int kZS = zpad(kZW) + 4;      // padded staging words
 
 // Batch item b is (v, b_hi, b_lo): v = b / nvi (0 when nvi <= 0), then
 // (b_hi, b_lo) = (r / nlo, r % nlo) for r = b - v nvi; each operand moves by
@@ -93,19 +104,29 @@ struct ToepArgs {
   int64_t zero_len;
   int64_t nvi;       // items per variant (<= 0: one variant)
   int64_t ustride_v, zstride_v, ostride_v;
+  int64_t pieces;    // CONV: pieces of a block
 };
 
-template <bool CONV>
+template <bool CONV, int kSB>
 __global__ void __launch_bounds__(kTT) toeplitz_kernel(const ToepArgs a) {
+  constexpr int kZW = kTB + kSB + 32;  // staged z words
+  constexpr int kZS = zpad(kZW) + 4;   // with the padding
   __shared__ __align__(16) uint32_t us[kSB];
   __shared__ __align__(16) uint32_t zs[kZS];
   const int tid = threadIdx.x;
+  launch_dependents();
+  grid_dependency_wait();
   if (a.zero_len > 0) {
     const int64_t nthreads = (int64_t)gridDim.x * gridDim.y * gridDim.z * kTT;
     const int64_t blk = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     for (int64_t i = blk * kTT + tid; i < a.zero_len; i += nthreads) a.zero[i] = 0u;
   }
-  const int64_t T0 = (int64_t)blockIdx.x * kTB;
+  // the block's pieces of kSB splits: CONV neighbouring ones, its outputs
+  // beginning with the first that they reach; CORR every gridDim.y-th
+  const int64_t first = CONV ? (int64_t)blockIdx.y * a.pieces : blockIdx.y;
+  const int64_t step = CONV ? 1 : gridDim.y;
+  const int64_t last = CONV ? first + a.pieces : INT64_MAX / kSB;
+  const int64_t T0 = (int64_t)blockIdx.x * kTB + (CONV ? first * kSB : 0);
   const int64_t bv = a.nvi > 0 ? (int64_t)blockIdx.z / a.nvi : 0;
   const int64_t br = (int64_t)blockIdx.z - bv * (a.nvi > 0 ? a.nvi : 0);
   const int64_t b_hi = br / a.nlo, b_lo = br % a.nlo;
@@ -118,8 +139,8 @@ __global__ void __launch_bounds__(kTT) toeplitz_kernel(const ToepArgs a) {
   uint32_t acc[kTo];
 #pragma unroll
   for (int q = 0; q < kTo; ++q) acc[q] = 0u;
-  // pieces blockIdx.y, blockIdx.y + gridDim.y, ... of kSB splits each
-  for (int64_t S0 = (int64_t)blockIdx.y * kSB; S0 < a.S; S0 += (int64_t)gridDim.y * kSB) {
+  for (int64_t piece = first; piece < last && piece * kSB < a.S; piece += step) {
+    const int64_t S0 = piece * kSB;
     // z index of output t = T0 + i and split s = S0 + j: c + i - j (CONV) or
     // c + i + j (CORR); the piece's range of z indices:
     const int64_t c = CONV ? T0 - S0 + a.zoff : T0 + S0 + a.zoff;
@@ -129,12 +150,24 @@ __global__ void __launch_bounds__(kTT) toeplitz_kernel(const ToepArgs a) {
     // zs[i] holds z[zbase + i]; thread tid at inner step j reads the 32 words
     // from start(tid, j), a multiple of 16
     const int64_t zbase = CONV ? c - kSB - 15 : c;
-    __syncthreads();  // the previous piece's reads are done
-    for (int i = tid; i < kZW; i += kTT) {
-      const int64_t zi = zbase + i;
-      zs[zpad(i)] = (zi >= 0 && zi < zlen) ? zb[zi] : 0u;
+    // all of a thread's loads are in flight at once
+    const int ilo = zbase < 0 ? (int)-zbase : 0;  // (zmax >= 0 and zmin < zlen)
+    const int ihi = zlen - zbase < kZW ? (int)(zlen - zbase) : kZW;
+    const uint32_t* zp = zb + zbase;
+    constexpr int kLoads = (kZW + kTT - 1) / kTT;
+    uint32_t zl[kLoads];
+#pragma unroll
+    for (int q = 0; q < kLoads; ++q) {
+      const int i = tid + kTT * q;
+      zl[q] = i >= ilo && i < ihi ? zp[i] : 0u;
     }
-    for (int i = tid; i < kSB; i += kTT) us[i] = S0 + i < a.S ? ub[S0 + i] : 0u;
+    static_assert(kSB <= kTT, "at most one u word per thread");
+    const uint32_t ul = tid < kSB && S0 + tid < a.S ? ub[S0 + tid] : 0u;
+    __syncthreads();  // the previous piece's reads are done
+#pragma unroll
+    for (int q = 0; q < kLoads; ++q)
+      if (tid + kTT * q < kZW) zs[zpad(tid + kTT * q)] = zl[q];
+    if (tid < kSB) us[tid] = ul;
     __syncthreads();
 #pragma unroll 1
     for (int j = 0; j < kSB; j += kTs) {
@@ -168,20 +201,29 @@ __global__ void __launch_bounds__(kTT) toeplitz_kernel(const ToepArgs a) {
         for (int q = 0; q < kTo; ++q) acc[q] += ur[r] * zr[CONV ? 15 + q - r : q + r];
     }
   }
-  // every output of the block is written (zero where no piece contributed);
-  // with the split range divided between blocks (gridDim.y > 1) the pieces'
-  // sums are added into a zeroed buffer
+  // With the split range divided between blocks (gridDim.y > 1) the sums are
+  // added into a zeroed buffer: through shared memory, for 32 neighbouring
+  // words per instruction.  Otherwise every output of the block is written
+  // (zero where no piece contributed).
   const int64_t oo = bv * a.ostride_v + b_hi * a.ostride_hi + b_lo * a.ostride;
   uint32_t* ob = a.out + oo;
+  __syncthreads();
+#pragma unroll
+  for (int v = 0; v < kTo / 4; ++v)
+    *reinterpret_cast<uint4*>(zs + zpad(kTo * tid + 4 * v)) =
+        make_uint4(acc[4 * v], acc[4 * v + 1], acc[4 * v + 2], acc[4 * v + 3]);
+  __syncthreads();
   const bool split = gridDim.y > 1;
 #pragma unroll
   for (int q = 0; q < kTo; ++q) {
-    const int64_t t = T0 + (int64_t)kTo * tid + q;
+    const int i = tid + kTT * q;
+    const int64_t t = T0 + i;
+    const uint32_t x = zs[zpad(i)];
     if (t < a.tout && oo + t < a.olim) {
-      if (split)
-        atomicAdd(ob + t, acc[q]);
-      else
-        ob[t] = acc[q];
+      if (!split)
+        ob[t] = x;
+      else if (x != 0u)
+        atomicAdd(ob + t, x);
     }
   }
 }
@@ -230,24 +272,29 @@ __global__ void __launch_bounds__(256) kara_combine_kernel(uint32_t* out, const 
   out[r * 2 * h + h + t] = p0 + kout[(2 * rows + r) * h + t];
 }
 
+constexpr int kFold = 64;  // threads: small blocks, for the loads of a few hundred of them at once
+
 // r[b][e] = c[b][e] + sum_j h[b][e + a_j - A] over the j with A <= e + a_j <=
 // 2A - 2, for e < A: the remainder of the reduction modulo chi.  The
 // product c is not read again (its upper half was read by the previous
 // launch), so each thread clears c[b][e] and c[b][e + A] for the next
 // product, which adds into a zeroed buffer.
-__global__ void __launch_bounds__(256) fold_kernel(uint32_t* c, int64_t cstride, const uint32_t* h,
+__global__ void __launch_bounds__(kFold) fold_kernel(uint32_t* c, int64_t cstride, const uint32_t* h,
                                                    int64_t hstride, uint32_t* r, int64_t rstride,
                                                    const int32_t* offs, int k, int A) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t b = blockIdx.y;
+  launch_dependents();
+  grid_dependency_wait();
   if (e >= A) return;
   uint32_t v = c[b * cstride + e];
   c[b * cstride + e] = 0u;
   if (e + A < cstride) c[b * cstride + e + A] = 0u;
   const uint32_t* hb = h + b * hstride;
+#pragma unroll 8
   for (int j = 0; j < k; ++j) {
     const int d = e + offs[j];
-    if (d >= A && d <= 2 * A - 2) v += hb[d - A];
+    v += d >= A && d <= 2 * A - 2 ? hb[d - A] : 0u;
   }
   r[b * rstride + e] = v;
 }
@@ -337,23 +384,47 @@ __global__ void __launch_bounds__(256) jump_start_kernel(uint32_t* R1, const uin
   R1[A - 1 - t] = v;
 }
 
-cudaError_t toeplitz(bool conv, const ToepArgs& a, int64_t batch, int sblocks, cudaStream_t st) {
-  const dim3 grid((unsigned)((a.tout + kTB - 1) / kTB), (unsigned)sblocks, (unsigned)batch);
-  if (conv)
-    toeplitz_kernel<true><<<grid, kTT, 0, st>>>(a);
-  else
-    toeplitz_kernel<false><<<grid, kTT, 0, st>>>(a);
-  return cudaGetLastError();
+// The launches of a product level are short: each is started while the one
+// before it runs, and waits for its end (griddepcontrol) before it reads or
+// writes anything.
+template <class... P, class... T>
+cudaError_t launch_early(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t st, T... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
 }
 
-// split-range pieces for a product of `batch` items with `tblocks` output
-// blocks each: as many as keep the launch within one wave of five blocks per
-// SM, the most that are resident at once (registers and shared memory both
-// allow five).
-int split_count(int64_t S, int64_t tblocks, int64_t batch, int sms) {
-  const int64_t most = (S + kSB - 1) / kSB;
-  const int64_t want = (5 * (int64_t)sms) / (tblocks * batch);
-  return (int)std::max<int64_t>(1, std::min(most, want));
+// Blocks that share the split range of a product of `batch` items with
+// `tblocks` output blocks each, over pieces of sb splits: one piece a block
+// until there are ten blocks per SM, then as evenly as can be.
+int split_count(int64_t S, int sb, int64_t tblocks, int64_t batch, int sms) {
+  const int64_t most = (S + sb - 1) / sb;
+  const int64_t want = std::max<int64_t>(1, (10 * (int64_t)sms) / (tblocks * batch));
+  const int64_t pieces = (most + want - 1) / want;
+  return (int)((most + pieces - 1) / pieces);
+}
+
+cudaError_t conv(ToepArgs a, int64_t batch, int sms, cudaStream_t st) {
+  constexpr int sb = kSBProduct;
+  const int64_t all = (a.S + sb - 1) / sb;
+  const int sp = split_count(a.S, sb, (a.zlen + sb + kTB - 2) / kTB, batch, sms);
+  a.pieces = (all + sp - 1) / sp;
+  const int64_t reach = std::min(a.zlen + a.pieces * sb - 1, a.tout);  // outputs of a block column
+  return launch_early(toeplitz_kernel<true, sb>, dim3((unsigned)((reach + kTB - 1) / kTB), (unsigned)sp, (unsigned)batch),
+                      kTT, st, a);
+}
+
+template <int sb>
+cudaError_t corr(const ToepArgs& a, int64_t batch, int sp, cudaStream_t st) {
+  return launch_early(toeplitz_kernel<false, sb>,
+                      dim3((unsigned)((a.tout + kTB - 1) / kTB), (unsigned)sp, (unsigned)batch), kTT, st, a);
 }
 
 }  // namespace
@@ -636,8 +707,6 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
   auto mulmod = [&](const uint32_t* x, int64_t xs, const uint32_t* y, int64_t ys, uint32_t* dst, int64_t cnt) {
     // prod is all zero here (set-up, then every fold clears what it read);
     // the product launch clears hf for the reduction that follows it
-    const int64_t tb_prod = (2 * (int64_t)A - 1 + dpk::kTB - 1) / dpk::kTB;
-    const int sp = dpk::split_count(A, tb_prod, cnt, ds->sms);
     ToepArgs ta{};
     ta.zero = hf;
     ta.zero_len = cnt * HS;
@@ -653,9 +722,9 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
     ta.tout = 2 * (int64_t)A - 1;
     ta.olim = INT64_MAX;
     ta.nlo = cnt;
-    if ((e = dpk::toeplitz(true, ta, cnt, sp, st)) != cudaSuccess) return e;
+    if ((e = dpk::conv(ta, cnt, ds->sms, st)) != cudaSuccess) return e;
     const int64_t tb_h = (A - 1 + dpk::kTB - 1) / dpk::kTB;
-    const int sh = dpk::split_count(A - 1, tb_h, cnt, ds->sms);
+    const int sh = dpk::split_count(A - 1, dpk::kSBProduct, tb_h, cnt, ds->sms);
     ToepArgs th{};
     th.u = g;
     th.S = A - 1;
@@ -669,10 +738,9 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
     th.tout = A - 1;
     th.olim = INT64_MAX;
     th.nlo = cnt;
-    if ((e = dpk::toeplitz(false, th, cnt, sh, st)) != cudaSuccess) return e;
-    dpk::fold_kernel<<<dim3((unsigned)((A + 255) / 256), (unsigned)cnt), 256, 0, st>>>(prod, PS, hf, HS, dst, A,
-                                                                                       d_offs, k, A);
-    return cudaGetLastError();
+    if ((e = dpk::corr<dpk::kSBProduct>(th, cnt, sh, st)) != cudaSuccess) return e;
+    return dpk::launch_early(dpk::fold_kernel, dim3((unsigned)((A + dpk::kFold - 1) / dpk::kFold), (unsigned)cnt),
+                             dpk::kFold, st, prod, PS, hf, HS, dst, (int64_t)A, d_offs, k, A);
   };
   // X[q] = X[m] X[q - m] for q in (m, 2m], m = 1, 2, 4, ..., up to X[qmax]
   auto tree = [&](uint32_t* X, int64_t qmax) {
@@ -687,14 +755,9 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
   auto windows = [&](const uint32_t* U, int64_t us, int64_t us_hi, int64_t zs_hi, int64_t nhi, int64_t nlo) {
     if (nhi * nlo <= 0) return cudaSuccess;
     if (kara && us_hi == 0) {
-      // the three half-size products as one launch of 3 rows items; the
-      // split count divides the pieces evenly
+      // the three half-size products as one launch of 3 rows items
       const int64_t rows = nhi * nlo;
-      const int64_t pieces = (kh + dpk::kSB - 1) / dpk::kSB;
-      const int64_t want = std::max<int64_t>(1, (5 * (int64_t)ds->sms) / (3 * rows));
-      int64_t sp = 1;
-      for (int64_t d = 1; d <= pieces && d <= want; ++d)
-        if (pieces % d == 0) sp = d;
+      const int sp = dpk::split_count(kh, dpk::kSBWindow, (kh + dpk::kTB - 1) / dpk::kTB, 3 * rows, ds->sms);
       if (sp > 1 && (e = cudaMemsetAsync(kout, 0, (size_t)3 * rows * kh * 4, st)) != cudaSuccess) return e;
       dpk::kara_prep_kernel<<<dim3((unsigned)((2 * kh + 255) / 256), (unsigned)std::max(nlo, nhi)), 256, 0, st>>>(
           U, us, nlo, ST, zs_hi, 2 * (int64_t)A - 1, n, nhi, kh, ku, kz);
@@ -717,13 +780,13 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
       tk.olim = INT64_MAX;
       tk.nlo = nlo;
       tk.nvi = rows;
-      if ((e = dpk::toeplitz(false, tk, 3 * rows, (int)sp, st)) != cudaSuccess) return e;
+      if ((e = dpk::corr<dpk::kSBWindow>(tk, 3 * rows, sp, st)) != cudaSuccess) return e;
       dpk::kara_combine_kernel<<<dim3((unsigned)((kh + 255) / 256), (unsigned)rows), 256, 0, st>>>(win, kout, rows,
                                                                                                    kh);
       return cudaGetLastError();
     }
     const int64_t tb = (A + dpk::kTB - 1) / dpk::kTB;
-    const int sp = dpk::split_count(A, tb, nhi * nlo, ds->sms);
+    const int sp = dpk::split_count(A, dpk::kSBWindow, tb, nhi * nlo, ds->sms);
     if ((e = cudaMemsetAsync(win, 0, (size_t)nhi * nlo * A * 4, st)) != cudaSuccess) return e;
     ToepArgs tw{};
     tw.u = U;
@@ -741,7 +804,7 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
     tw.olim = INT64_MAX;
     tw.nlo = nlo;
     // with one piece the kernel stores instead of adding: same result on the zeroed rows
-    return dpk::toeplitz(false, tw, nhi * nlo, sp, st);
+    return dpk::corr<dpk::kSBWindow>(tw, nhi * nlo, sp, st);
   };
   // copies `rows` scratch rows, from row r0, to ST + pos0 + r * pitch,
   // clipped at n
