@@ -367,12 +367,11 @@ void sdp_shape(int32_t a1, int32_t ak, int* threads, int* ring_log2) {
 // block (clocks at 2.07 GHz): k = 4, W = 32: 161; k = 16, W = 64: 206, W = 200:
 // 266, W = 600: 530; k = 32, W = 64: 319, W = 1024: 1250; with more offsets
 // than registers k = 48, W = 64: 1030, W = 1024: 2770.
-double sdp_plain_us(int64_t cells, int32_t ak, int32_t k) {
-  if (cells <= 0) return 0.0;
-  const double W = std::min<int32_t>(ak, 1024);
-  const double clocks = 110.0 + (k > dpk::kSdpMaxKRegs ? 18.0 : 4.0) * k + W * (k + 2) / 32.0;
-  return std::ceil((double)cells / W) * clocks / 2.07e3;
+SdpSteps::SdpSteps(int32_t ak, int32_t k) : W(std::min<int32_t>(ak, 1024)) {
+  step_us = (110.0 + (k > dpk::kSdpMaxKRegs ? 18.0 : 4.0) * k + (double)W * (k + 2) / 32.0) / 2.07e3;
 }
+
+double sdp_plain_us(int64_t cells, int32_t ak, int32_t k) { return SdpSteps(ak, k).us(cells); }
 
 int64_t sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g_out) {
   int32_t g = a[0], gap = a[k - 1];
@@ -430,7 +429,7 @@ int64_t sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g_out) {
 SdpRoute sdp_route(int64_t n, const int32_t* a, int32_t k, int op, int sms) {
   SdpRoute r;
   if (op == DP_OP_ADD_MOD32) {
-    r.chunks = sdp_jump_chunks(n, a, k, sms);
+    r.chunks = sdp_jump_chunks(n, a, k, sms, &r.us);
     return r;
   }
   r.tail_from = sdp_min_tail(n, a, k, &r.g);

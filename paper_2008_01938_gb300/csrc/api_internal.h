@@ -90,6 +90,12 @@ dp_status mcm_enqueue(const McmStatic& sp, const McmLayout& L, void* ws, const i
 dp_status sdp_validate(int64_t n, const int32_t* a, int32_t k, int op);
 // Approximate device time of the step kernel for `cells` cells, microseconds.
 double sdp_plain_us(int64_t cells, int32_t ak, int32_t k);
+struct SdpSteps {  // the same for several lengths
+  SdpSteps(int32_t ak, int32_t k);
+  double us(int64_t cells) const { return cells <= 0 ? 0.0 : (double)((cells + W - 1) / W) * step_us; }
+  int64_t W;
+  double step_us;
+};
 void sdp_shape(int32_t a1, int32_t ak, int* threads, int* ring_log2);
 // (x) = min: the first cell from which the table repeats its last g cells, g
 // the gcd of the offsets (host arithmetic on the offsets only; see
@@ -101,6 +107,7 @@ struct SdpRoute {
   int chunks = 0;
   int64_t tail_from = 0;
   int32_t g = 0;
+  double us = 0.0;  // (x) = + in chunks: the model's time
 };
 SdpRoute sdp_route(int64_t n, const int32_t* a, int32_t k, int op, int sms);
 // Fills the arguments of the step kernel's launch for one table (not for chunks >= 2).
@@ -108,8 +115,9 @@ void sdp_single_args(dpk::SdpLaunchArgs* args, uint32_t* ST, int64_t n, const in
                      const SdpRoute& route, int sms, int32_t* status);
 // (x) = + on one instance, by chunks that start from jumped windows
 // (sdp_jump.cu): the number of chunks the cost model picks (0: solve step by
-// step), and the solve with a given number of chunks.
-int sdp_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms);
+// step; otherwise *us is the model's time), and the solve with a given number
+// of chunks.
+int sdp_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms, double* us = nullptr);
 // The plan behind it (host arithmetic only): P, L, L0, squarings, reach of
 // the impulse response, chunks per major window, major windows, chunks asked.
 int sdp_jump_plan(int64_t n, const int32_t* a, int32_t k, int sms, int64_t out[8]);

@@ -434,12 +434,15 @@ namespace dph {
 
 namespace {
 // Approximate device times, in microseconds, for the choice between the
-// plain path and the jump path: the step kernel's (sdp_plain_us); a Toeplitz
-// product runs at about 14 T multiply-adds/s (measured); a product modulo chi
-// costs about 1.7 a_1^2 of them in three launches, a window a_1^2, and the
-// three launches of one product level on small batches about 35 us (measured:
-// 16, 13 and 5 us).
-constexpr double kLevelUs = 35.0;
+// plain path and the jump path: the step kernel's (sdp_plain_us); a product
+// modulo chi costs about 1.7 a_1^2 multiply-adds, a window a_1^2, at 17.4 T
+// of them per second; the three launches of a level of products 14 besides,
+// and all the other launches of a solve together 80.  Fitted to 238 solves of
+// 5e4 to 2^26 cells with 2 to 152 chunks, of which it misses by 10% (rms); the
+// count it picks is within 8% of the best one's time in all 15 series.
+constexpr double kLevelUs = 14.0;
+constexpr double kFixedUs = 80.0;
+constexpr double kMadsPerUs = 17.4e6;
 // Windows by transforms (sdp_ntt.cu) where a window is long enough for them to
 // be the faster: with a_1 = 8192 63 windows take 36 us, 204 as direct products.
 // `count` windows: about 13 us per round of a block per SM, window and prime,
@@ -496,16 +499,15 @@ JumpPlan plan_for(int64_t n, int32_t A, int chunks, int64_t Gm, int sms) {
   return p;
 }
 
-double jump_us(int64_t n, int32_t A, int32_t ak, int32_t k, const JumpPlan& p, int sms) {
+double jump_us(int64_t n, int32_t A, const SdpSteps& plain, const JumpPlan& p, int sms) {
   const double A2 = (double)A * A;
   const int products = p.s + (p.P2 - 1) + std::max(p.P1e - 2, 0);
-  const int levels = p.s + ceil_log2(p.P2) + ceil_log2(std::max(p.P1e - 1, 1)) + 4;
+  const int levels = p.s + ceil_log2(p.P2) + ceil_log2(std::max(p.P1e - 1, 1));
   const double mads = products * 1.7 * A2 + (by_transforms(A) ? 0.0 : (p.P - 1) * A2);
   const double windows = by_transforms(A) ? transform_us(p.P - 1, sms) : 0.0;
-  const double halves = p.half ? transform_us(p.P, sms) + sdp_plain_us(A, ak, k) : 0.0;
-  return sdp_plain_us(std::min<int64_t>(p.chunk(), n) - A, ak, k) + sdp_plain_us(A, ak, k) +
-         std::max(sdp_plain_us(A, ak, k), sdp_plain_us(p.Gm + 1, ak, k)) + mads / 14.0e6 + windows + halves +
-         levels * kLevelUs;
+  const double halves = p.half ? transform_us(p.P, sms) + plain.us(A) : 0.0;
+  return plain.us(std::min<int64_t>(p.chunk(), n) - A) + plain.us(A) + plain.us(std::max<int64_t>(A, p.Gm + 1)) +
+         mads / kMadsPerUs + windows + halves + levels * kLevelUs + kFixedUs;
 }
 
 dp_status launch_records(const dpk::SdpInstDev* insts, int count, int32_t k, int32_t threads, int32_t ring_log2,
@@ -523,47 +525,56 @@ dp_status launch_records(const dpk::SdpInstDev* insts, int count, int32_t k, int
   const cudaError_t e = dpk::launch_sdp(args, stream);
   return e == cudaSuccess ? DP_OK : fail_cuda(e, "sdp jump: launch of the chunk kernel");
 }
-// How far to compute the impulse response for `chunks` chunks: every
-// doubling of its reach saves one squaring and costs a longer plain run.
-int64_t jump_reach(int64_t n, int32_t A, int32_t ak, int32_t k, int chunks, int sms) {
-  int64_t best_gm = A - 1;
-  double best = -1.0;
+// The plan for `chunks` chunks with the reach of the impulse response that is
+// the fastest (every doubling of it saves one squaring and costs a longer
+// plain run), and its time; P = 0 when there is none.
+JumpPlan best_plan(int64_t n, int32_t A, const SdpSteps& plain, int chunks, int sms, double* us = nullptr) {
+  JumpPlan best;
+  double best_us = 0.0;
   for (int64_t gm : {(int64_t)A - 1, 2 * (int64_t)A, 4 * (int64_t)A, 8 * (int64_t)A, 16 * (int64_t)A}) {
     const JumpPlan p = plan_for(n, A, chunks, gm, sms);
-    if (p.P < 2) return A - 1;
-    const double t = jump_us(n, A, ak, k, p, sms);
-    if (best < 0.0 || t < best) {
-      best = t;
-      best_gm = gm;
+    if (p.P < 2) break;
+    const double t = jump_us(n, A, plain, p, sms);
+    if (best.P == 0 || t < best_us) {
+      best = p;
+      best_us = t;
     }
+    if (p.s == 0) break;  // no squarings left to save
   }
-  return best_gm;
+  if (us) *us = best_us;
+  return best;
 }
 }  // namespace
 
-int sdp_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms) {
+int sdp_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms, double* us) {
   const int32_t A = a[0], ak = a[k - 1];
   if (A < 2 || n < 8 * (int64_t)A) return 0;
   int32_t tl = 0, rl = 0;
   sdp_shape(A, ak, &tl, &rl);
   if (rl <= 0) return 0;  // the chunks need the window on chip
-  double best = 0.8 * sdp_plain_us(n - A, ak, k);  // the jump must win clearly
-  if (best <= 4 * kLevelUs) return 0;                // less than the levels of any plan
+  const SdpSteps plain(ak, k);
+  double best = 0.8 * plain.us(n - A);               // the jump must win clearly
+  if (best <= kFixedUs + kLevelUs) return 0;         // less than any plan
   int bestP = 0;
   auto at = [&](int c) {
-    const JumpPlan p = plan_for(n, A, c, jump_reach(n, A, ak, k, c, sms), sms);
-    if (p.P < 2) return false;
-    const double t = jump_us(n, A, ak, k, p, sms);
+    double t = 0.0;
+    if (best_plan(n, A, plain, c, sms, &t).P < 2) return false;
     if (t < best) {
       best = t;
       bestP = c;
     }
     return true;
   };
-  // the time is flat around its minimum: a grid of about 80 counts, a 24th
-  // apart, costs the host 20 us, every count with five plans each 100
-  for (int c = 2; c <= sms; c += std::max(1, c / 24))
+  // the time is flat around its minimum: about 25 counts, a seventh apart, then
+  // the best one's neighbours (about 10 us of host time)
+  for (int c = 2; c <= sms; c += std::max(1, c / 7))
     if (!at(c)) break;
+  if (const int c0 = bestP)
+    for (int d = -4; d <= 4; ++d) {
+      const int c = c0 + (d * c0 + (d < 0 ? -20 : 20)) / 35;
+      if (c > 1 && c <= sms && c != c0) at(c);
+    }
+  if (us) *us = best;
   return bestP;
 }
 
@@ -571,7 +582,7 @@ int sdp_jump_plan(int64_t n, const int32_t* a, int32_t k, int sms, int64_t out[8
   const int chunks = sdp_jump_chunks(n, a, k, sms);
   for (int i = 0; i < 8; ++i) out[i] = 0;
   if (chunks < 2) return 0;
-  const JumpPlan p = plan_for(n, a[0], chunks, jump_reach(n, a[0], a[k - 1], k, chunks, sms), sms);
+  const JumpPlan p = best_plan(n, a[0], SdpSteps(a[k - 1], k), chunks, sms);
   out[0] = p.P;
   out[1] = p.L;
   out[2] = p.L0;
@@ -591,7 +602,7 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
   if (rc != DP_OK) return rc;
   const int32_t A = a[0];
   if (A < 2) return fail(DP_EINVAL, "sdp jump: a_1 = %d, the table is constant", A);
-  const JumpPlan pl = plan_for(n, A, chunks, jump_reach(n, A, a[k - 1], k, chunks, ds->sms), ds->sms);
+  const JumpPlan pl = best_plan(n, A, SdpSteps(a[k - 1], k), chunks, ds->sms);
   if (pl.P < 2)
     return fail(DP_EINVAL, "sdp jump: %d chunks of at least %d cells do not fit n = %lld", chunks, 2 * A,
                 (long long)n);

@@ -214,6 +214,37 @@ dp_status launch_mcm_group(Server* S, const std::vector<Req*>& reqs, bool i64, L
   return DP_OK;
 }
 
+// Solves in chunks run one after another, the blocks of the shared launch side
+// by side: of the requests with a route in chunks, the i that would hold the
+// shared launch up longest keep it, for the i with the least total time.
+// (A dozen requests of 2e5 cells, k = 16, a_k = 64: in chunks 170 us each, in
+// the shared launch 310 for all.)
+void sdp_share_launch(const std::vector<Req*>& reqs, SdpRoute* route) {
+  auto plain_us = [&](size_t b) {
+    return sdp_plain_us(reqs[b]->n - reqs[b]->offs[0], reqs[b]->offs.back(), (int32_t)reqs[b]->offs.size());
+  };
+  std::vector<std::pair<double, size_t>> by_time;  // requests with a route in chunks
+  double others = 0.0;
+  for (size_t b = 0; b < reqs.size(); ++b) {
+    if (route[b].chunks >= 2)
+      by_time.emplace_back(plain_us(b), b);
+    else
+      others = std::max(others, plain_us(b));
+  }
+  std::sort(by_time.rbegin(), by_time.rend());
+  size_t keep = 0;
+  double in_chunks = 0.0, best = -1.0;
+  for (size_t i = 0; i <= by_time.size(); ++i) {
+    const double total = in_chunks + (i < by_time.size() ? std::max(others, by_time[i].first) : others);
+    if (best < 0.0 || total < best) {
+      best = total;
+      keep = i;
+    }
+    if (i < by_time.size()) in_chunks += route[by_time[i].second].us;
+  }
+  for (size_t i = keep; i < by_time.size(); ++i) route[by_time[i].second] = SdpRoute{};
+}
+
 // A group of S-DP requests with one operator.  Requests long enough for the
 // chunked paths of sdp_solve (sdp_jump.cu for +, sdp_minjump.cu for min; the
 // same cost models decide) or with a long periodic tail run through those,
@@ -235,8 +266,10 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
     const Req* r = reqs[b];
     const int k = (int)r->offs.size();
     if (r->n > r->offs[0]) route[b] = sdp_route(r->n, r->offs.data(), k, op, ds->sms);
-    if (!own_launch(b)) bat.push_back(b);
   }
+  if (op == DP_OP_ADD_MOD32) sdp_share_launch(reqs, route.data());
+  for (size_t b = 0; b < reqs.size(); ++b)
+    if (!own_launch(b)) bat.push_back(b);
   bool ring_ok = true, same_k = true;
   std::vector<int64_t> st_off(reqs.size());
   int64_t cells = 0, noffs = 0;
