@@ -16,7 +16,8 @@ constexpr int T = kTile;
 constexpr uint32_t kFinPollNs = 64;   // finisher mbarrier waits (int32): longest sleep between polls
 constexpr uint32_t kFlagPollNs = 32;  // flag and counter waits (int32): longest sleep between polls
 
-constexpr int kDiagRows = 2 * T;  // cell diagonals e = lj - li in [-31, 31] (dI = e + 31), one spare row
+constexpr int kBlk = T / 2;                // 2x2-cell blocks of a tile, per side
+constexpr int kDiagRows = 2 * kBlk - 1;    // block diagonals E = bj - bi in [-15, 15]
 
 using E = uint32_t;      // panel entries: (m << S) | (k mod 2^S)
 constexpr int KB = 32;   // k bits in the 64-bit (value, k) key
@@ -29,28 +30,30 @@ __device__ __forceinline__ int64_t tile_index(const McmInstDev& in, int I, int J
 //
 // In-tile wavefront arrays (finisher of an off-diagonal tile) start at STA and
 // reuse the bulk-copy stages (every copy of the task has landed before they
-// are written).  Row t of the U^T / L tables, t in [-32, 63], is at t + 32 (96
-// rows, constant offsets per step); rows outside t = 0 .. 30 hold zeros.  The
-// cell-value arrays Xr / Xc live outside the stage area, so their entries for
+// are written), as 2x2-cell blocks of 16 bytes.  Rows of L and U blocks that a
+// step reaches beside the tables hold zeros where no cell stands behind them
+// (before row 0 of L, after row 15 of U); the others are read only for blocks
+// that are final already, and hold anything.  The cell-value arrays Xr / Xc live outside the stage area, so their entries for
 // cells that do not exist are set to all ones once per block and stay so
 // (every existing cell is written before it is read).
 struct Smem {
   static constexpr int ES = 4;
   static constexpr int TILE = T * T * ES;
-  static constexpr int kRows = 96;
-  static constexpr int kRowOff = 32;
-  static constexpr int UPW = 36;                                 // U^T pitch: 16-byte rows, conflict-free
   static constexpr int BARS = 0;                                 // 9 mbarriers + task slot
   static constexpr int STA = 128;                                // [group][stage] row panels
   static constexpr int STB = STA + 4 * TILE;                     // [group][stage] column panels
   static constexpr int STPK = STB + 4 * TILE;                    // [group][stage] 32 x u32 dims
   static constexpr int STEND = STPK + 4 * 128;
-  static constexpr int XBYTES = kDiagRows * T * ES;
-  static constexpr int WUP = STA;                                // Up[row(t)][li] = m[IT+li][IT+t]
-  static constexpr int WLP = WUP + ((kRows * UPW * ES + 127) / 128) * 128;  // Lp[row(u)][lj] = m[JT+u+1][JT+lj]
-  static constexpr int WPKI = WLP + kRows * T * ES;               // PKIp[row(t)] = p[IT+t+1]
-  static constexpr int WPKJ = WPKI + kRows * 4;                  // PKJp[row(u)] = p[JT+u+1]
-  static constexpr int WEND = (WPKJ + kRows * 4 + 127) / 128 * 128;
+  static constexpr int XBYTES = kDiagRows * kBlk * 16;
+  static constexpr int kQRows = 3 * kBlk - 3;                    // 45: every block row a step can reach
+  static constexpr int kLRow0 = kBlk - 1;                        // row of block row 0 of L, and of U
+  static constexpr int kURow0 = kBlk - 2;
+  static constexpr int UQW = 4 * kBlk + 4;                       // pitch of U rows: conflict-free down a column
+  static constexpr int WLQ = STA;                                // Lq[kLRow0 + u][bj]: L[2u + s][2 bj + c] at 2 s + c
+  static constexpr int WUQ = WLQ + kQRows * 4 * kBlk * ES;       // Uq[kURow0 + b][bi]: m[IT+2bi+r][IT+2b+s-1] at 2 r + s
+  static constexpr int WPJ = WUQ + kQRows * UQW * ES;            // p[JT + 2u + s + 1]
+  static constexpr int WPI = WPJ + kQRows * 8;                   // p[IT + 2b + s]
+  static constexpr int WEND = (WPI + kQRows * 8 + 127) / 128 * 128;
   static constexpr int FINU = ((STEND > WEND ? STEND : WEND) + 127) / 128 * 128;  // row panel of (I,I)
   static constexpr int FINL = FINU + TILE;                       // column panel of diagonal tile (J,J)
   static constexpr int FINBROW = FINL + TILE;                    // boundary row (one tile row)
@@ -59,12 +62,12 @@ struct Smem {
   static constexpr int FINPKJ = FINPKI + 128;                    // p[32J+1 ..] << S
   static constexpr int FINACC = FINPKJ + 128;                    // bulk-task partial minima
   static constexpr int BEST = FINACC + T * T * 8;                // running (value, k) keys
-  static constexpr int WXR = BEST + T * T * 8;                   // Xr[e+31][li]: final value of cell (li, li+e)
-  static constexpr int WXC = WXR + XBYTES;                       // Xc[e+31][lj]: final value of cell (lj-e, lj)
+  static constexpr int WXR = BEST + T * T * 8;                   // Xr[E+15][bi]: final values of block (bi, bi+E)
+  static constexpr int WXC = WXR + XBYTES;                       // Xc[E+15][bj]: final values of block (bj-E, bj)
   static constexpr int TOTAL = WXC + XBYTES;
   static constexpr int XV = STA;                                 // diagonal tiles: the tile's values
-  __host__ __device__ static constexpr int row(int t) { return t + kRowOff; }
-  static_assert(WXR % 16 == 0 && WUP % 16 == 0 && (UPW * ES) % 16 == 0, "16-byte vector rows");
+  static_assert(WXR % 16 == 0 && WLQ % 16 == 0 && WUQ % 16 == 0 && (UQW * ES) % 16 == 0 && WPJ % 8 == 0,
+                "vector rows");
 };
 
 __device__ __forceinline__ void bar_compute() {  // the 256 compute threads only
@@ -99,55 +102,40 @@ __device__ __forceinline__ E umin(E a, E b) { return a < b ? a : b; }
 // w = p[IT+li] p[k+1] p[JT+lj+1]; the boundary split k = IT + 31 and the
 // external splits are known before the solve starts.
 //
-// Cell (li, lj) lies on cell diagonal e = lj - li in [-31, 31] and depends
-// only on cells of lower diagonals, so the tile is solved in the paper's
-// diagonal order (Figs. 5-7), one diagonal per step: in step e every cell
-// pulls the candidate of its row split and of its column split whose operand
-// lies on diagonal e (exactly one of each), and the cells of diagonal e + 1,
-// whose last operands were on diagonal e, become final.  Warp w owns rows
-// 4w .. 4w+3 and lane = column.
+// A thread owns a block of 2x2 cells, (2 bi + r, 2 bj + c).  The block lies on
+// block diagonal E = bj - bi in [-15, 15] and depends only on blocks of lower
+// diagonals, so the tile is solved in the paper's diagonal order (Figs. 5-7),
+// one block diagonal per step: in step E every block pulls the candidates of
+// the two column splits and the two row splits per cell whose operands lie in
+// blocks of diagonal E, and the blocks of diagonal E + 1, whose last operands
+// those were, become final: their cells depend on one another through one
+// split each in one or two more links, in registers.  Warp w owns block rows
+// 2w and 2w + 1.
+//
+// The solve is a chain of steps (barrier, load, minima, store), and on it hangs
+// the time between two tile diagonals.  Cell by cell it is 62 steps of 170
+// clocks, by blocks 30 of about 210 for the same candidates: n = 128: 45.9 ->
+// 38.8 us, 1000 (tables to the host) 389 -> 322, 4096 1980 -> 1798, interval DP
+// of 2000 670 -> 579.  (Blocks of 8x8 cells, one warp each without barriers
+// inside, took 17.3 k clocks a tile against the cells' 10.5 k.)
 //
 // Each thread keeps one running minimum per cell (values only).  The operands
-// that do not depend on the tile move predictably from step to step and are
-// loaded ahead of the barrier: the row split of cell (li, lj) at step e uses
-// L[li + e][lj], the thread's 4 rows use 4 consecutive rows of L, so a
-// 4-entry register window gains one new row per step; U[li][lj - e - 1] and
-// p[IT + lj - e] come from one 16-byte load and one word per step.  The cell
-// values themselves are exchanged through two diagonal-major arrays written
-// once, when a cell becomes final: Xr (indexed by row, the row-split operand)
-// and Xc (indexed by column, the column-split operand).
+// that do not depend on the tile are laid out as blocks, one 16-byte load per
+// step each, loaded and multiplied ahead of the barrier.  The cell values
+// themselves are exchanged through two arrays of blocks by diagonal, written
+// once, when a block becomes final: Xr (indexed by block row, the row-split
+// operand) and Xc (indexed by block column, the column-split operand).
 //
 // Out-of-range operands are read from zero rows (U, L, dims) and from
 // all-ones entries (cells that do not exist), so no candidate needs a
 // predicate: a missing cell yields an all-ones candidate, and a candidate
 // whose operand exists but whose split is outside the cell's range only
-// arises after the cell was finalised (its running minimum is then dead).
+// arises after the block was finalised (its running minimum is then dead).
 // The smallest minimising split is recovered after the tile is published, by
 // scanning the splits of each cell in increasing k.
 // ---------------------------------------------------------------------------
-struct Vec4 {
-  E v[4];
-};
-
-__device__ __forceinline__ Vec4 lds4(const E* p) {  // 4 consecutive elements, 16-byte aligned
-  Vec4 r;
-  const uint4 q = *reinterpret_cast<const uint4*>(p);
-  r.v[0] = q.x, r.v[1] = q.y, r.v[2] = q.z, r.v[3] = q.w;
-  return r;
-}
-
-// a[r] where p0 and p1 are bits 0 and 1 of r, already computed.
-__device__ __forceinline__ E sel4p(bool p0, bool p1, E a0, E a1, E a2, E a3) {
-  const E lo = p0 ? a1 : a0, hi = p0 ? a3 : a2;
-  return p1 ? hi : lo;
-}
-
-// Shared-memory store of v at 32-bit shared address addr when p holds.
-__device__ __forceinline__ void sts_if(bool p, uint32_t addr, E v) {
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.shared.u32 [%1], %2;\n\t}" ::"r"((uint32_t)p),
-               "r"(addr), "r"(v)
-               : "memory");
-}
+__device__ __forceinline__ uint4 lds4(const E* p) { return *reinterpret_cast<const uint4*>(p); }  // 16-byte aligned
+__device__ __forceinline__ uint2 lds2(const E* p) { return *reinterpret_cast<const uint2*>(p); }  // 8-byte aligned
 
 // ---------------------------------------------------------------------------
 // Bulk segment reductions (one compute group, 128 threads, 4 x 2 cells each).
@@ -240,7 +228,7 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
   int32_t* status = a.status;
 
   E* x = reinterpret_cast<E*>(smem + SM::WXR);
-  for (int i = tid; i < 2 * kDiagRows * T; i += blockDim.x) x[i] = ~(E)0;
+  for (int i = tid; i < 2 * SM::XBYTES / SM::ES; i += blockDim.x) x[i] = ~(E)0;
   if (tid == 0) {
     for (int i = 0; i < 4; ++i) {
       mbar_init(&bar_full[i], 1);
@@ -427,14 +415,16 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
       if (finisher) {
         bar_compute();
         // ------------------ in-tile wavefront (finisher) ------------------
-        // layout: warp w owns rows 4w..4w+3, lane = column
+        // The thread's 4 cells: off-diagonal tiles, the 2x2 block (bi, bj); the
+        // diagonal tile, rows 4w .. 4w + 3 of column lane.
         const int w = warp;
-        // interval DP: the weights of the thread's 4 cells, loaded while the copies land
+        const int bi = 2 * w + (lane >> 4), bj = lane & (kBlk - 1);
+        // interval DP: the weights of the cells, loaded while the copies land
         E wt[4] = {0, 0, 0, 0};
         if constexpr (W) {
 #pragma unroll
           for (int r = 0; r < 4; ++r) {
-            const int64_t i = IT + 4 * w + r, j = JT + lane;
+            const int64_t i = IT + (D >= 1 ? 2 * bi + (r >> 1) : 4 * w + r), j = JT + (D >= 1 ? 2 * bj + (r & 1) : lane);
             if (i < j && j < inst.n) wt[r] = static_cast<const E*>(inst.w)[i * inst.n + j];
           }
         }
@@ -444,126 +434,144 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
         if (!fin_ok) set_status(status, DP_ETIMEOUT);
         const bool go = bar_compute_and(fin_ok && *reinterpret_cast<volatile int32_t*>(status) == 0);
         const int n = inst.n;
-        unsigned long long cb[4];
-        E pi[4];
         const E pj1 = (E)(finPKJ[lane] >> S);  // p[JT + lane + 1]
         if (go) {
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const int li = 4 * w + r;
-            pi[r] = (E)finPP[li];
-            cb[r] = bestS[li * T + lane];
-            if (task.nparts > 0) cb[r] = umin(cb[r], finAcc[li * T + lane]);
-          }
           if (D >= 1) {
-            E* Up = reinterpret_cast<E*>(smem + SM::WUP);
-            E* Lp = reinterpret_cast<E*>(smem + SM::WLP);
+            E* Lq = reinterpret_cast<E*>(smem + SM::WLQ);
+            E* Uq = reinterpret_cast<E*>(smem + SM::WUQ);
+            E* PJ = reinterpret_cast<E*>(smem + SM::WPJ);
+            E* PI = reinterpret_cast<E*>(smem + SM::WPI);
             E* Xr = reinterpret_cast<E*>(smem + SM::WXR);
             E* Xc = reinterpret_cast<E*>(smem + SM::WXC);
-            uint32_t* PKIp = reinterpret_cast<uint32_t*>(smem + SM::WPKI);
-            uint32_t* PKJp = reinterpret_cast<uint32_t*>(smem + SM::WPKJ);
-            // boundary split k = IT + 31: U[li][31] + m[IT+32][j] + w
-            const E brow = finBrow[lane] >> S;
-            const E pI32 = (E)(finPKI[T - 1] >> S);
-            E m[4], wv[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-              const int li = 4 * w + r;
-              bestS[li * T + lane] = cb[r];  // external minimum: (value, smallest k)
-              wv[r] = pi[r] * pj1;
-              const E bnd = (finU[(T - 1) * T + li] >> S) + brow + wv[r] * pI32;
-              m[r] = umin((E)(cb[r] >> KB), bnd);
-            }
-            // 16-byte vectors: 8 per row, 3 per thread (all row pitches are 16-byte multiples)
-            for (int v = tid; v < SM::kRows * T / 4; v += kComputeThreads) {
-              const int q = v >> 3, x = (v & 7) * 4, t = q - SM::kRowOff;
-              uint4 uu = make_uint4(0u, 0u, 0u, 0u), ll = make_uint4(0u, 0u, 0u, 0u);
-              if (t >= 0 && t <= T - 2) {
-                const uint4 fu = *reinterpret_cast<const uint4*>(finU + t * T + x);
-                const uint4 fl = *reinterpret_cast<const uint4*>(finL + t * T + x);
-                uu = make_uint4(fu.x >> S, fu.y >> S, fu.z >> S, fu.w >> S);
-                ll = make_uint4(fl.x >> S, fl.y >> S, fl.z >> S, fl.w >> S);
+            // operands in blocks (thread: block row tid / 16, block column tid % 16)
+            {
+              const int y = tid >> 4, x = tid & (kBlk - 1);
+              const uint2 l0 = lds2(finL + 2 * y * T + 2 * x), l1 = lds2(finL + (2 * y + 1) * T + 2 * x);
+              const bool in1 = y < kBlk - 1;  // L has 31 rows
+              *reinterpret_cast<uint4*>(Lq + ((SM::kLRow0 + y) * kBlk + x) * 4) =
+                  make_uint4(l0.x >> S, l0.y >> S, in1 ? l1.x >> S : 0u, in1 ? l1.y >> S : 0u);
+              const uint2 u1 = lds2(finU + 2 * y * T + 2 * x), u0 = lds2(finU + (y > 0 ? 2 * y - 1 : 0) * T + 2 * x);
+              *reinterpret_cast<uint4*>(Uq + (SM::kURow0 + y) * SM::UQW + 4 * x) =
+                  make_uint4(u0.x >> S, u1.x >> S, u0.y >> S, u1.y >> S);
+              if (y < kBlk - 1) {  // block rows that do not exist: -15 .. -1 of L, 16 .. 30 of U
+                *reinterpret_cast<uint4*>(Lq + (y * kBlk + x) * 4) = make_uint4(0u, 0u, 0u, 0u);
+                *reinterpret_cast<uint4*>(Uq + (SM::kURow0 + kBlk + y) * SM::UQW + 4 * x) = make_uint4(0u, 0u, 0u, 0u);
               }
-              *reinterpret_cast<uint4*>(Up + q * SM::UPW + x) = uu;
-              *reinterpret_cast<uint4*>(Lp + q * T + x) = ll;
+              if (tid < T) {
+                PJ[2 * SM::kLRow0 + tid] = finPKJ[tid] >> S;
+                PI[2 * SM::kURow0 + tid] = finPP[tid];
+              } else if (tid < 2 * T - 2) {
+                PJ[tid - T] = 0u;
+                PI[2 * (SM::kURow0 + kBlk) + tid - T] = 0u;
+              }
             }
-            if (tid < SM::kRows) {
-              const int t = tid - SM::kRowOff;
-              const bool in = t >= 0 && t <= T - 2;
-              PKIp[tid] = in ? (finPKI[t] >> S) : 0u;
-              PKJp[tid] = in ? (finPKJ[t] >> S) : 0u;
-            }
-            const uint32_t sXr = smem_u32(Xr), sXc = smem_u32(Xc);
-            const int e_last = T - 2 - 4 * w;  // the warp's last cell, (4w, 31), is final after this step
-            const int c0 = lane - 4 * w - 1;   // at step e the lane's cell in row 4w + c0 - e becomes final
-            bar_compute();
-            if (w == 7 && lane == 0) {  // cell (31, 0), the only cell of diagonal -31
-              Xr[T - 1] = m[3] + wt[3];
-              Xc[0] = m[3] + wt[3];
-            }
-            // Operands of the first step.  Window slot (u & 3) holds L[u][lane]
-            // and p[JT + u + 1] for u = 4w + e .. 4w + e + 3; with e = 1 mod 4
-            // at the start of each group of 4 steps, the slots are compile-time
-            // indices.
-            E R[4];
-            uint32_t P[4];
+            // boundary split k = IT + 31: U[li][31] + m[IT+32][j] + w
+            const E pI32 = (E)(finPKI[T - 1] >> S);
+            const E pib = finPP[2 * bi + 1], pjb = finPKJ[2 * bj] >> S;  // p[IT + 2 bi + 1], p[JT + 2 bj + 1]
+            E m[4], wv[4];  // cell (2 bi + r, 2 bj + c) at 2 r + c
+            E ib[4];        // multiplier terms of the splits inside the block: 0,0 / 1,1 / 0,1 by row / 0,1 by column
+            {
+              const uint2 br = lds2(finBrow + 2 * bj), pj = lds2(finPKJ + 2 * bj);
+              const uint2 ub = lds2(finU + (T - 1) * T + 2 * bi), pp = lds2(reinterpret_cast<const E*>(finPP) + 2 * bi);
+              wv[0] = pp.x * (pj.x >> S), wv[1] = pp.x * (pj.y >> S);
+              wv[2] = pp.y * (pj.x >> S), wv[3] = pp.y * (pj.y >> S);
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-              const int u = 4 * w - (T - 1) + r;
-              R[(1 + r) & 3] = Lp[SM::row(u) * T + lane];
-              P[(1 + r) & 3] = PKJp[SM::row(u)];
-            }
-            Vec4 u4 = lds4(Up + SM::row(lane + T - 2) * SM::UPW + 4 * w);  // t = lane - 1 - e
-            E pkc = (E)PKIp[SM::row(lane + T - 2)];
-            bar_compute();
-            // int32: the 62 steps are unrolled, so every shared-memory
-            // operand is a constant offset from a per-thread base. The
-            // operands of step e + 1 (independent of the tile values) are
-            // loaded at the start of step e, so the barrier after the step
-            // does not wait for them, and each candidate is a multiply-add
-            // plus a fused add-and-minimum. The row of the cell made final
-            // is chosen with predicates computed once: bit 0 of c0 - e
-            // flips every step, bit 1 repeats every four steps.
-            const E* Lb = Lp + SM::row(4 * w) * T + lane;                 // + u * T: L row u = 4w + e + r
-            const uint32_t* PJb = PKJp + SM::row(4 * w);                  // + u
-            const E* Ub = Up + SM::row(lane - 1) * SM::UPW + 4 * w;       // - (e + 1) * UPW: t = lane - 2 - e
-            const uint32_t* PIb = PKIp + SM::row(lane - 1);               // - (e + 1)
-            const E* Xcb = Xc + (T - 1) * T + lane;                       // + e * T: X[lane - e][lane]
-            const E* Xrb = Xr + (T - 1) * T + 4 * w;                      // + e * T: X[li][li + e]
-            const uint32_t sXcw = sXc + (uint32_t)((T * T + lane) * 4);      // + e * T * 4
-            const uint32_t sXrw = sXr + (uint32_t)((T * T + lane - 1) * 4);  // + e * (T - 1) * 4
-            const bool b0e = (c0 & 1) != 0;  // bit 0 of c0 - e for even e
-            bool b1[4];                      // bit 1 of c0 - e for e = k mod 4
-#pragma unroll
-            for (int k = 0; k < 4; ++k) b1[k] = ((c0 - k) & 2) != 0;
-#pragma unroll
-            for (int e = -(T - 1); e <= T - 2; ++e) {
-              const int s4 = (e + T - 1) & 3;
-              if (e <= e_last) {
-                const E Rn = Lb[(e + 4) * T];
-                const uint32_t Pn = PJb[e + 4];
-                const Vec4 u4n = lds4(Ub - (e + 1) * SM::UPW);
-                const E pkcn = (E)PIb[-(e + 1)];
-                const E xc = Xcb[e * T];             // column operand X[lane - e][lane]
-                const Vec4 x4 = lds4(Xrb + e * T);  // row operands X[li][li + e]
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                  const int q = (1 + s4 + r) & 3;
-                  m[r] = __viaddmin_u32(u4.v[r] + wv[r] * pkc, xc, m[r]);
-                  m[r] = __viaddmin_u32(R[q] + wv[r] * (E)P[q], x4.v[r], m[r]);
+              for (int r = 0; r < 2; ++r) {
+                ulonglong2* own = reinterpret_cast<ulonglong2*>(bestS + (2 * bi + r) * T + 2 * bj);
+                ulonglong2 cb = *own;
+                if (task.nparts > 0) {
+                  const ulonglong2 ac = *reinterpret_cast<const ulonglong2*>(finAcc + (2 * bi + r) * T + 2 * bj);
+                  cb.x = umin(cb.x, ac.x);
+                  cb.y = umin(cb.y, ac.y);
+                  *own = cb;  // external minimum: (value, smallest k)
                 }
-                // the lane's cell on diagonal e + 1 (row 4w + c0 - e) is final now
-                const bool p0 = (e & 1) ? !b0e : b0e;
-                const bool p1 = b1[(e + 32) & 3];
-                E v = sel4p(p0, p1, m[0], m[1], m[2], m[3]);
-                if constexpr (W) v += sel4p(p0, p1, wt[0], wt[1], wt[2], wt[3]);
-                const bool own = (unsigned)(c0 - e) <= 3u;
-                sts_if(own, sXrw + (uint32_t)(e * (T - 1) * 4), v);
-                sts_if(own, sXcw + (uint32_t)(e * T * 4), v);
-                R[(1 + s4) & 3] = Rn;
-                P[(1 + s4) & 3] = Pn;
-                u4 = u4n;
-                pkc = pkcn;
+                const E u31 = (r ? ub.y : ub.x) >> S;
+                m[2 * r] = umin((E)(cb.x >> KB), u31 + (br.x >> S) + wv[2 * r] * pI32);
+                m[2 * r + 1] = umin((E)(cb.y >> KB), u31 + (br.y >> S) + wv[2 * r + 1] * pI32);
+              }
+              ib[0] = wv[0] * pib, ib[1] = wv[3] * pjb, ib[2] = wv[1] * pjb, ib[3] = wv[1] * pib;
+            }
+            // The block's final values, in the order of its cell diagonals; the
+            // one split inside it adds a table value 0.
+            auto block_values = [&]() {
+              uint4 v;
+              v.z = m[2];
+              if constexpr (W) v.z += wt[2];
+              v.x = __viaddmin_u32(v.z, ib[0], m[0]);
+              v.w = __viaddmin_u32(v.z, ib[1], m[3]);
+              if constexpr (W) v.x += wt[0], v.w += wt[3];
+              v.y = __viaddmin_u32(v.x, ib[2], __viaddmin_u32(v.w, ib[3], m[1]));
+              if constexpr (W) v.y += wt[1];
+              return v;
+            };
+            const int fd = bj - bi;  // the block's diagonal
+            E* const xr0 = Xr + (kBlk - 1) * kBlk * 4 + 4 * bi;  // + 4 kBlk E: block (bi, bi + E)
+            E* const xc0 = Xc + (kBlk - 1) * kBlk * 4 + 4 * bj;  // + 4 kBlk E: block (bj - E, bj)
+            if (fd == 1 - kBlk) {  // block (15, 0), the only one of its diagonal
+              const uint4 v = block_values();
+              *reinterpret_cast<uint4*>(xr0 + 4 * kBlk * (1 - kBlk)) = v;
+              *reinterpret_cast<uint4*>(xc0 + 4 * kBlk * (1 - kBlk)) = v;
+            }
+            bar_compute();
+            // 30 steps, unrolled: every shared-memory operand is a constant
+            // offset from a per-thread base.  What does not depend on the tile
+            // is loaded at the start of the step before and multiplied at its
+            // end, so that after a barrier a candidate is one fused
+            // add-and-minimum.
+            const E* const l0 = Lq + (SM::kLRow0 + bi) * kBlk * 4 + 4 * bj;   // + 4 kBlk E
+            const E* const u0 = Uq + (SM::kURow0 + bj) * SM::UQW + 4 * bi;    // - UQW E
+            const E* const pj0 = PJ + 2 * (SM::kLRow0 + bi);                  // + 2 E
+            const E* const pi0 = PI + 2 * (SM::kURow0 + bj);                  // - 2 E
+            const int e_last = kBlk - 2 - 2 * w;  // the warp's last block, (2w, 15), is final after this step
+            E rc[8], cc[8];  // candidates less the tile value: cell 2 r + c, operand s at 2 (2 r + c) + s
+            auto terms = [&](const uint4& l, const uint4& u, const uint2& qj, const uint2& qi) {
+              rc[0] = l.x + wv[0] * qj.x, rc[1] = l.z + wv[0] * qj.y;
+              rc[2] = l.y + wv[1] * qj.x, rc[3] = l.w + wv[1] * qj.y;
+              rc[4] = l.x + wv[2] * qj.x, rc[5] = l.z + wv[2] * qj.y;
+              rc[6] = l.y + wv[3] * qj.x, rc[7] = l.w + wv[3] * qj.y;
+              cc[0] = u.x + wv[0] * qi.x, cc[1] = u.y + wv[0] * qi.y;
+              cc[2] = u.x + wv[1] * qi.x, cc[3] = u.y + wv[1] * qi.y;
+              cc[4] = u.z + wv[2] * qi.x, cc[5] = u.w + wv[2] * qi.y;
+              cc[6] = u.z + wv[3] * qi.x, cc[7] = u.w + wv[3] * qi.y;
+            };
+            terms(lds4(l0 + 4 * kBlk * (1 - kBlk)), lds4(u0 - SM::UQW * (1 - kBlk)), lds2(pj0 + 2 * (1 - kBlk)),
+                  lds2(pi0 - 2 * (1 - kBlk)));
+#pragma unroll
+            for (int e = 1 - kBlk; e <= kBlk - 2; ++e) {
+              if (e <= e_last) {
+                const uint4 xr = lds4(xr0 + 4 * kBlk * e);  // X[2 bi + r][2 (bi + e) + s] at 2 r + s
+                const uint4 xc = lds4(xc0 + 4 * kBlk * e);  // X[2 (bj - e) + s][2 bj + c] at 2 s + c
+                uint4 l = {}, u = {};
+                uint2 qj = {}, qi = {};
+                if (e < kBlk - 2) {
+                  l = lds4(l0 + 4 * kBlk * (e + 1));
+                  u = lds4(u0 - SM::UQW * (e + 1));
+                  qj = lds2(pj0 + 2 * (e + 1));
+                  qi = lds2(pi0 - 2 * (e + 1));
+                }
+                m[2] = __viaddmin_u32(rc[4], xr.z, m[2]);
+                m[0] = __viaddmin_u32(rc[0], xr.x, m[0]);
+                m[3] = __viaddmin_u32(rc[6], xr.z, m[3]);
+                m[1] = __viaddmin_u32(rc[2], xr.x, m[1]);
+                m[2] = __viaddmin_u32(rc[5], xr.w, m[2]);
+                m[0] = __viaddmin_u32(rc[1], xr.y, m[0]);
+                m[3] = __viaddmin_u32(rc[7], xr.w, m[3]);
+                m[1] = __viaddmin_u32(rc[3], xr.y, m[1]);
+                m[2] = __viaddmin_u32(cc[4], xc.x, m[2]);
+                m[0] = __viaddmin_u32(cc[0], xc.x, m[0]);
+                m[3] = __viaddmin_u32(cc[6], xc.y, m[3]);
+                m[1] = __viaddmin_u32(cc[2], xc.y, m[1]);
+                m[2] = __viaddmin_u32(cc[5], xc.z, m[2]);
+                m[0] = __viaddmin_u32(cc[1], xc.z, m[0]);
+                m[3] = __viaddmin_u32(cc[7], xc.w, m[3]);
+                m[1] = __viaddmin_u32(cc[3], xc.w, m[1]);
+                // blocks on diagonal e + 1 are final now
+                const uint4 v = block_values();
+                if (fd == e + 1) {
+                  *reinterpret_cast<uint4*>(xr0 + 4 * kBlk * (e + 1)) = v;
+                  *reinterpret_cast<uint4*>(xc0 + 4 * kBlk * (e + 1)) = v;
+                }
+                if (e < kBlk - 2) terms(l, u, qj, qi);
               }
               bar_compute();
             }
@@ -571,7 +579,8 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
             const int64_t nn = n;
             E vals[4];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) vals[r] = Xc[(lane - 4 * w - r + T - 1) * T + lane];
+            for (int r = 0; r < 4; ++r)  // cell (4w + r, lane)
+              vals[r] = Xc[(((lane >> 1) - 2 * w - (r >> 1) + kBlk - 1) * kBlk + (lane >> 1)) * 4 + 2 * (r & 1) + (lane & 1)];
             {
               E* af = static_cast<E*>(a.af) + tidx * T * T;
               E pa[4];
@@ -615,6 +624,11 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
             // external splits (smallest one kept with the external minimum),
             // row splits JT .. j-1.
             const unsigned long long kmask = (1ull << KB) - 1ull;
+            const E brow = finBrow[lane] >> S;
+            const int cb = lane >> 1, cc1 = lane & 1;  // the column's block, and which of its columns
+            // word offset of row or column x (x = t + 1 for column splits) in an
+            // array of blocks
+            auto at = [](int x, int pitch, int odd) { return (x >> 1) * pitch + (x & 1) * odd; };
 #pragma unroll 1
             for (int r = 0; r < 4; ++r) {
               // warp w scans rows w, w + 8, w + 16 and w + 24, a mix of
@@ -623,26 +637,32 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
               const int li = w + 8 * r;
               const int64_t i = IT + li, j = JT + lane;
               if (i >= nn || j >= nn) continue;
-              // (register arrays are read through sel4: a runtime index would move them to local memory)
+              const int lb = li >> 1, lr = li & 1;
               E v;   // the minimum, less the cell's own weight
               E wr;  // the row's multiplier p[i] p[j+1]
-              v = Xc[(lane - li + T - 1) * T + lane];
+              v = Xc[((cb - lb + kBlk - 1) * kBlk + cb) * 4 + 2 * lr + cc1];
               if constexpr (W) v -= static_cast<const E*>(inst.w)[i * inst.n + j];
               wr = (E)finPP[li] * pj1;
               int k = -1;
               // four splits per round with independent loads, the
               // smallest matching one kept; a lane stops after the first
-              // round with a match
+              // round with a match (reads past the last split stay inside
+              // shared memory and are not used)
+              const E* us = Uq + SM::kURow0 * SM::UQW + 4 * lb + 2 * lr;            // + at(x, UQW, 1)
+              const E* xs = Xc + ((cb + kBlk - 1) * kBlk + cb) * 4 + cc1;           // + at(x, -4 kBlk, 2)
+              const E* ps = PI + 2 * SM::kURow0;                                    // + x
+              int uo[4], xo[4];
+#pragma unroll
+              for (int d = 0; d < 4; ++d) uo[d] = at(li + 1 + d, SM::UQW, 1), xo[d] = at(li + 1 + d, -4 * kBlk, 2);
               for (int t0 = li; t0 <= T - 2 && k < 0; t0 += 4) {
                 E c4[4];
 #pragma unroll
-                for (int d = 0; d < 4; ++d) {
-                  const int t = t0 + d <= T - 2 ? t0 + d : T - 2;
-                  c4[d] = Up[SM::row(t) * SM::UPW + li] + Xc[(lane - t - 1 + T - 1) * T + lane] + wr * (E)PKIp[SM::row(t)];
-                }
+                for (int d = 0; d < 4; ++d) c4[d] = us[uo[d]] + xs[xo[d]] + wr * ps[t0 + 1 + d];
 #pragma unroll
                 for (int d = 3; d >= 0; --d)
                   if (t0 + d <= T - 2 && c4[d] == v) k = IT + t0 + d;
+                us += 2 * SM::UQW;
+                xs -= 8 * kBlk;
               }
               if (k < 0 && (finU[(T - 1) * T + li] >> S) + brow + wr * pI32 == v) k = IT + T - 1;
               if (k < 0) {
@@ -650,22 +670,33 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
                 if ((E)(ek >> KB) == v) k = (int)(ek & kmask);
               }
               if (k < 0) {
+                const E* rs = Xr + ((kBlk - 1 - lb) * kBlk + lb) * 4 + 2 * lr;  // + at(u, 4 kBlk, 1)
+                const E* ls = Lq + (SM::kLRow0 * kBlk + cb) * 4 + cc1;          // + at(u, 4 kBlk, 2)
                 for (int u0 = 0; u0 < lane && k < 0; u0 += 4) {
                   E c4[4];
 #pragma unroll
-                  for (int d = 0; d < 4; ++d) {
-                    const int u = u0 + d <= T - 2 ? u0 + d : T - 2;
-                    c4[d] = Xr[(u - li + T - 1) * T + li] + Lp[SM::row(u) * T + lane] + wr * (E)PKJp[SM::row(u)];
-                  }
+                  for (int d = 0; d < 4; ++d)
+                    c4[d] = rs[at(d, 4 * kBlk, 1)] + ls[at(d, 4 * kBlk, 2)] + wr * PJ[2 * SM::kLRow0 + u0 + d];
 #pragma unroll
                   for (int d = 3; d >= 0; --d)
                     if (u0 + d < lane && c4[d] == v) k = JT + u0 + d;
+                  rs += 8 * kBlk;
+                  ls += 8 * kBlk;
                 }
               }
               inst.s[i * nn + j] = (int16_t)k;
             }
           } else {
             // diagonal tile: ordinary MCM on the 32-matrix sub-chain
+            unsigned long long cb[4];
+            E pi[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+              const int li = 4 * w + r;
+              pi[r] = (E)finPP[li];
+              cb[r] = bestS[li * T + lane];
+              if (task.nparts > 0) cb[r] = umin(cb[r], finAcc[li * T + lane]);
+            }
             const E pj1d = (E)(finPKI[lane] >> S);
             bool keyed = false;
             if (S == 5) {
