@@ -118,22 +118,12 @@ __device__ __forceinline__ int32_t ld_acquire(const int32_t* p) {
   return v;
 }
 
-__device__ __forceinline__ int32_t ld_relaxed(const int32_t* p) {
-  int32_t v;
-  asm volatile("ld.relaxed.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
 __device__ __forceinline__ void st_release(int32_t* p, int32_t v) {
   asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
 __device__ __forceinline__ void red_release_add(int32_t* p, int32_t v) {
   asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-__device__ __forceinline__ void fence_acquire_gpu() {
-  asm volatile("fence.acq_rel.gpu;" ::: "memory");
 }
 
 // Records the first device-side error in *status (later errors are dropped).
@@ -162,28 +152,6 @@ __device__ __forceinline__ bool wait_flag_geq_cap(const int32_t* flag, int32_t t
     __nanosleep(backoff);
     backoff = backoff < CAP ? backoff * 2 : CAP;
   }
-}
-
-// Waits until f[x] >= target[x] for every x < N (int32 MCM instances).  The
-// first test issues all N acquire loads at once, so the words already set
-// cost one round trip together rather than one each; any still short are
-// then polled one at a time with wait_flag_geq_cap.  A target of 0 is met at
-// once.  Every word is read by an acquire load, so no fence follows.
-template <uint32_t CAP, int N>
-__device__ __forceinline__ bool wait_flags_geq_cap(const int32_t* const (&f)[N], const int32_t (&target)[N],
-                                                   long long limit, int32_t* status) {
-  int32_t v[N];
-#pragma unroll
-  for (int x = 0; x < N; ++x) v[x] = ld_acquire(f[x]);
-  bool all = true;
-#pragma unroll
-  for (int x = 0; x < N; ++x) all = all && v[x] >= target[x];
-  if (!all) {
-#pragma unroll
-    for (int x = 0; x < N; ++x)
-      if (v[x] < target[x] && !wait_flag_geq_cap<CAP>(f[x], target[x], limit, status)) return false;
-  }
-  return true;
 }
 
 }  // namespace dpk

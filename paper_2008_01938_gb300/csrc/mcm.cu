@@ -268,76 +268,131 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
     const int32_t accslot = a.accslot[tidx];
 
     if (warp == kComputeThreads / 32) {
-      // ===================== producer warp (lane 0) =====================
-      if (lane == 0) {
-        // the stage area was written and read through the generic proxy by the
-        // previous task's in-tile solve; order that before this task's copies
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        bool ok = true;
-        bool issued[2][kStages] = {{false, false}, {false, false}};
-        bool fin_issued = false;
-        uint32_t last_parity[2][kStages] = {{0u, 0u}, {0u, 0u}};
-        for_each_segment(task, [&](int K, int q) {
-          const int g = q & 1;
-          const uint32_t u = use_cnt[g]++;
-          const int st = u % kStages;
-          const uint32_t round = u / kStages;
-          if (!ok) return;
-          // the three tiles' flags in one round trip when they are set
-                    const int32_t* const fl[3] = {a.flags + tile_index(inst, I, K), a.flags + tile_index(inst, K, J),
-                                                  a.flags + tile_index(inst, K + 1, J)};
-                    const int32_t tg[3] = {1, 1, 1};
-                    ok = wait_flags_geq_cap<kFlagPollNs, 3>(fl, tg, limit, status);
-          if (!ok) return;
+      // ===================== producer warp =====================
+      // The lanes poll a flag each, so that all the flags waited for cost one
+      // round trip together; lane 0 issues the copies.
+      //
+      // The stage area was written and read through the generic proxy by the
+      // previous task's in-tile solve; order that before this task's copies.
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      bool ok = true;
+      bool issued[2][kStages] = {{false, false}, {false, false}};
+      bool fin_issued = false;
+      uint32_t last_parity[2][kStages] = {{0u, 0u}, {0u, 0u}};
+      const int32_t* const flags = a.flags + inst.tile_base;
+      auto tile = [&](int i, int j) { return i * inst.nt - i * (i - 1) / 2 + (j - i); };
+      // the lane's flag of segment K, for lanes 0 .. 2: tiles (I, K), (K, J), (K + 1, J)
+      auto segment_flag = [&](int K, int x) {
+        return flags + tile(x == 0 ? I : x == 1 ? K : K + 1, x == 0 ? K : J);
+      };
+      auto copy_segment = [&](int K, int g, uint32_t u) {
+        const int st = u % kStages;
+        const uint32_t round = u / kStages;
+        bool got = true;
+        if (lane == 0) {
           fence_proxy_async_global();
-          if (!mbar_wait(&bar_empty[g * kStages + st], (round & 1u) ^ 1u, limit)) {
+          got = mbar_wait(&bar_empty[g * kStages + st], (round & 1u) ^ 1u, limit);
+          if (got) {
+            uint64_t* fb = &bar_full[g * kStages + st];
+            mbar_arrive_expect_tx(fb, 2 * SM::TILE + 128);
+            bulk_g2s(stA + (g * kStages + st) * T * T,
+                     static_cast<const E*>(a.af) + tile_index(inst, I, K) * T * T, SM::TILE, fb);
+            bulk_g2s(stB + (g * kStages + st) * T * T,
+                     static_cast<const E*>(a.bf) + tile_index(inst, K, J) * T * T, SM::TILE, fb);
+            bulk_g2s(stPK + (g * kStages + st) * 32, a.pk + inst.pk_base + (int64_t)K * T, 128, fb);
+          } else {
             set_status(status, DP_ETIMEOUT);
-            ok = false;
-            return;
           }
-          uint64_t* fb = &bar_full[g * kStages + st];
-          mbar_arrive_expect_tx(fb, 2 * SM::TILE + 128);
-          bulk_g2s(stA + (g * kStages + st) * T * T,
-                   static_cast<const E*>(a.af) + tile_index(inst, I, K) * T * T, SM::TILE, fb);
-          bulk_g2s(stB + (g * kStages + st) * T * T,
-                   static_cast<const E*>(a.bf) + tile_index(inst, K, J) * T * T, SM::TILE, fb);
-          bulk_g2s(stPK + (g * kStages + st) * 32, a.pk + inst.pk_base + (int64_t)K * T, 128, fb);
+        }
+        got = __shfl_sync(~0u, (int)got, 0) != 0;
+        if (got) {
           issued[g][st] = true;
           last_parity[g][st] = round & 1u;
-        });
-        if (finisher && ok) {
-          // tiles (I, I), (J, J), (I+1, J) and the bulk-task counter in one
-          // round trip when they are ready; a diagonal tile has no
-          // neighbours, so its own flag stands in with target 0
-          const bool nb = D >= 1;
-          const int32_t* const fl[4] = {a.flags + (nb ? tile_index(inst, I, I) : tidx),
-                                        a.flags + (nb ? tile_index(inst, J, J) : tidx),
-                                        a.flags + (nb ? tile_index(inst, I + 1, J) : tidx), a.counters + tidx};
-          const int32_t tg[4] = {nb ? 1 : 0, nb ? 1 : 0, nb ? 1 : 0, task.nparts > 0 ? (int32_t)task.nparts : 0};
-          ok = wait_flags_geq_cap<kFlagPollNs, 4>(fl, tg, limit, status);
-          if (ok) {
-            fence_proxy_async_global();
-            uint32_t bytes = 3 * 128;
-            if (D >= 1) bytes += 2 * SM::TILE + T * (uint32_t)sizeof(E);
-            if (task.nparts > 0) bytes += T * T * 8;
-            mbar_arrive_expect_tx(bar_fin, bytes);
-            bulk_g2s(finPP, a.pp + inst.pp_base + IT, 128, bar_fin);
-            bulk_g2s(finPKI, a.pk + inst.pk_base + IT, 128, bar_fin);
-            bulk_g2s(finPKJ, a.pk + inst.pk_base + JT, 128, bar_fin);
-            if (D >= 1) {
-              bulk_g2s(finU, static_cast<const E*>(a.af) + tile_index(inst, I, I) * T * T, SM::TILE, bar_fin);
-              bulk_g2s(finL, static_cast<const E*>(a.bf) + tile_index(inst, J, J) * T * T, SM::TILE, bar_fin);
-              bulk_g2s(finBrow, static_cast<const E*>(a.bf) + tidx * T * T + (T - 1) * T, T * sizeof(E), bar_fin);
-            }
-            if (task.nparts > 0) bulk_g2s(finAcc, a.acc + (int64_t)accslot * T * T, T * T * 8, bar_fin);
-            fin_issued = true;
-          } else {
-            // keep the finisher barrier's phase sequence intact for the consumers
-            mbar_arrive(bar_fin);
-          }
-        } else if (finisher) {
-          mbar_arrive(bar_fin);
         }
+        return got;
+      };
+      // Polls the lanes' flags until `stop` (called with the mask of the lanes
+      // that are done) returns true; false after an error or `limit` clocks.
+      auto poll = [&](const int32_t* f, int32_t target, bool done, auto&& stop) {
+        const long long t0 = clock64();
+        for (int32_t failed = 0;; failed = *reinterpret_cast<volatile const int32_t*>(status)) {
+          if (!done) done = ld_acquire(f) >= target;
+          const uint32_t have = __ballot_sync(~0u, done);
+          __syncwarp();
+          if (stop(have)) return true;
+          const bool late = clock64() - t0 > limit;
+          if (late && lane == 0) set_status(status, DP_ETIMEOUT);
+          if (__shfl_sync(~0u, (int)(late || failed != 0), 0) != 0) return false;
+          __nanosleep(kFlagPollNs);
+        }
+      };
+      // A finisher's last two segments (its neighbours' tiles) and its own
+      // operands become ready at about the same time, in no fixed order: their
+      // flags are waited for together, one round trip a poll, and the copies
+      // of the segments go first.  (Flags one after the other in lane 0: the
+      // second segment arrived 1.3 k clocks after the first.  n = 300 89.3 ->
+      // 83.4 us, 1000 255 -> 230, 2000 559 -> 529, 3000 985 -> 963, 4096 1798
+      // -> 1811, interval DP of 2000 592 -> 569; operands' copies as soon as
+      // they may: 1 to 2% slower.)
+      int nseg = 0;
+      if (finisher) for_each_segment(task, [&](int, int q) { nseg = q + 1; });
+      int late_k[2] = {0, 0};
+      uint32_t late_u[2] = {0u, 0u};
+      for_each_segment(task, [&](int K, int q) {
+        const int g = q & 1;
+        const uint32_t u = use_cnt[g]++;
+        if (finisher && q >= nseg - 2) {
+          late_k[g] = K;
+          late_u[g] = u;
+          return;
+        }
+        if (!ok) return;
+        ok = poll(segment_flag(K, lane < 3 ? lane : 0), 1, lane >= 3, [&](uint32_t have) { return have == ~0u; }) &&
+             copy_segment(K, g, u);
+      });
+      if (finisher && ok) {
+        // lanes 0 .. 2 and 3 .. 5: the segments; 6 .. 8: tiles (I, I), (J, J),
+        // (I+1, J); 9: the bulk-task counter
+        bool want[2] = {nseg > 0, nseg > 1}, want_fin = true, got = true;
+        const int32_t* f = a.counters + tidx;
+        int32_t target = lane == 9 ? task.nparts : 0;
+        if (lane < 6) {
+          const int g = lane / 3;
+          if (want[g]) f = segment_flag(late_k[g], lane - 3 * g), target = 1;
+        } else if (lane < 9 && D >= 1) {
+          f = flags + (lane == 6 ? tile(I, I) : lane == 7 ? tile(J, J) : tile(I + 1, J));
+          target = 1;
+        }
+        const bool polled = poll(f, target, target == 0, [&](uint32_t have) {
+          if (want[0] && (have & 0x7u) == 0x7u) want[0] = false, got = got && copy_segment(late_k[0], 0, late_u[0]);
+          if (want[1] && (have & 0x38u) == 0x38u) want[1] = false, got = got && copy_segment(late_k[1], 1, late_u[1]);
+          if (want_fin && !want[0] && !want[1] && (have & 0x3C0u) == 0x3C0u) {
+            want_fin = false;
+            fin_issued = got;
+            if (got && lane == 0) {
+              fence_proxy_async_global();
+              uint32_t bytes = 3 * 128;
+              if (D >= 1) bytes += 2 * SM::TILE + T * (uint32_t)sizeof(E);
+              if (task.nparts > 0) bytes += T * T * 8;
+              mbar_arrive_expect_tx(bar_fin, bytes);
+              bulk_g2s(finPP, a.pp + inst.pp_base + IT, 128, bar_fin);
+              bulk_g2s(finPKI, a.pk + inst.pk_base + IT, 128, bar_fin);
+              bulk_g2s(finPKJ, a.pk + inst.pk_base + JT, 128, bar_fin);
+              if (D >= 1) {
+                bulk_g2s(finU, static_cast<const E*>(a.af) + tile_index(inst, I, I) * T * T, SM::TILE, bar_fin);
+                bulk_g2s(finL, static_cast<const E*>(a.bf) + tile_index(inst, J, J) * T * T, SM::TILE, bar_fin);
+                bulk_g2s(finBrow, static_cast<const E*>(a.bf) + tidx * T * T + (T - 1) * T, T * sizeof(E), bar_fin);
+              }
+              if (task.nparts > 0) bulk_g2s(finAcc, a.acc + (int64_t)accslot * T * T, T * T * 8, bar_fin);
+            }
+          }
+          return !got || (!want[0] && !want[1] && !want_fin);
+        });
+        ok = polled && got;
+      }
+      if (lane == 0) {
+        // keep the finisher barrier's phase sequence intact for the consumers
+        if (finisher && !fin_issued) mbar_arrive(bar_fin);
         // No bulk copy may still be in flight when the task ends.
         for (int g = 0; g < 2; ++g)
           for (int st = 0; st < kStages; ++st)
@@ -390,6 +445,8 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
         mbar_arrive(&bar_empty[g * kStages + st]);
       });
 
+      // (a finisher's look at the error status, early enough to be there when it is needed)
+      const int32_t failed = finisher ? *reinterpret_cast<volatile const int32_t*>(status) : 0;
       // merge the two groups' minima: group 1 publishes, group 0 combines
       if (g == 1) {
 #pragma unroll
@@ -432,7 +489,7 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
         bool fin_ok;
         fin_ok = mbar_wait_cap(bar_fin, fpar, limit, kFinPollNs);
         if (!fin_ok) set_status(status, DP_ETIMEOUT);
-        const bool go = bar_compute_and(fin_ok && *reinterpret_cast<volatile int32_t*>(status) == 0);
+        const bool go = bar_compute_and(fin_ok && failed == 0);
         const int n = inst.n;
         const E pj1 = (E)(finPKJ[lane] >> S);  // p[JT + lane + 1]
         if (go) {
