@@ -1,5 +1,6 @@
-"""The int32 in-tile solve by 2x2-cell blocks: lengths around the edges of
-blocks and tiles, many splits of equal cost, and the interval DP's weights."""
+"""The int32 in-tile solves (2x2-cell blocks; the triangle of a diagonal tile by
+pairs of rows): lengths around the edges of blocks, pairs and tiles, many splits
+of equal cost, and the interval DP's weights."""
 import numpy as np
 import pytest
 
@@ -7,7 +8,7 @@ import oracle
 
 pytestmark = pytest.mark.gpu
 
-NS = [33, 34, 35, 47, 48, 62, 63, 64, 65, 66, 96, 97, 127, 161, 290]
+NS = [2, 3, 15, 16, 17, 30, 31, 32, 33, 34, 35, 47, 48, 62, 63, 64, 65, 66, 96, 97, 127, 161, 290]
 
 
 @pytest.mark.parametrize("n", NS)
