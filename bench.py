@@ -342,6 +342,12 @@ def run_gb300(args):
         dist.destroy_process_group()
 
 
+def _min_tail(lib, n, offsets):
+    """The cell from which sdp_solve with min fills the table by residue classes (0: not on that path)."""
+    g = ctypes.c_int32()
+    return int(lib.dp_test_sdp_min_tail(n, ctypes.c_void_p(offsets.ctypes.data), int(offsets.size), ctypes.byref(g)))
+
+
 def bench_sdp(dp, native, lib, dev, args):
     import numpy as np
     import torch
@@ -381,12 +387,18 @@ def bench_sdp(dp, native, lib, dev, args):
         av = np.ascontiguousarray(big.offsets.astype(np.int32))
         hook = lib.dp_test_sdp_jump_chunks if op == "add" else lib.dp_test_sdp_min_jump_chunks
         chunks = hook(big.n, ctypes.c_void_p(av.ctypes.data), int(av.size))
-        if chunks >= 2:
+        tail = _min_tail(lib, big.n, av) if op == "min" else 0
+        if tail:
+            res[op]["path"] = (f"step by step on one SM up to cell {tail}, from where on a cell is the minimum of "
+                               f"its residue class of the preset; the others are filled by all SMs")
+            res[op]["roofline"]["note"] = f"the recurrence runs over {tail} cells, the rest is written once"
+        elif chunks >= 2:
             algebra = ("products modulo the characteristic polynomial over Z/2^32" if op == "add" else
                        "Boolean products modulo the characteristic polynomial (bitsets) and range minima")
             res[op]["path"] = (f"chunks from jumped windows: {chunks} chunks side by side, their windows from "
                                f"{algebra} (time covers the whole path)")
-            nsm = min(chunks, args.probe["sms"])
+            # (+) windows by transforms: two half chunks per window where the SMs suffice
+            nsm = args.probe["sms"] if op == "add" else min(chunks, args.probe["sms"])
             peak_w = nsm * smem_peak
             res[op]["smem_roofline"] = {"bound": f"shared memory of the {nsm} SMs the chunks run on",
                                         "achieved": cells * k / (kms / 1e3) / 1e9, "peak": peak_w,
@@ -418,7 +430,8 @@ def bench_sdp(dp, native, lib, dev, args):
     res["consecutive_min"] = {"workload": "same n, k=32 consecutive offsets 1055..1024 (the paper's conflict worst "
                                           "case), preset seed 6", "cells_per_s": (big.n - 1055) / (kms / 1e3),
                               "kernel_ms": kms,
-                              "path": ("chunks from jumped windows" if lib.dp_test_sdp_min_jump_chunks(
+                              "path": ("periodic tail" if _min_tail(lib, big.n, cons) else
+                                       "chunks from jumped windows" if lib.dp_test_sdp_min_jump_chunks(
                                   big.n, ctypes.c_void_p(cons.ctypes.data), int(cons.size)) >= 2
                                   else "step by step on one SM")}
     return res

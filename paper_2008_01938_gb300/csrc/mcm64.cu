@@ -6,11 +6,12 @@
 //
 // What bounds it.  A 64-bit split evaluation is one multiply-add and six
 // instructions on the ALU pipe (add, compare and select in two halves each),
-// about 13 clocks per warp and scheduler, so the work of a tile is issue
+// of which the selects are predicated multiply-adds by one on the FMA pipe
+// outside the in-tile solve, so the work of a tile is issue
 // slots, and a single chain is bound by its tile-diagonals' hand-offs and
 // wavefronts.  Batches of short chains are mostly finishers: one block of 256
-// threads per tile and three of them per SM keep the ALUs fed while others
-// wait at a barrier or for memory.
+// threads per tile and two of them per SM keep the ALUs fed while others
+// wait at a barrier or for memory (three need registers that spill).
 //
 // A block needs nothing but plain copies: every flag a task waits for is
 // polled by one lane of the first warp before the task starts (its other
