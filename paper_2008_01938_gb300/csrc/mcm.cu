@@ -276,9 +276,8 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
       // previous task's in-tile solve; order that before this task's copies.
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       bool ok = true;
-      bool issued[2][kStages] = {{false, false}, {false, false}};
+      uint32_t issued = 0u, parity = 0u;  // a bit per group and stage (arrays here lived in local memory: 4096 1799 -> 1781 us)
       bool fin_issued = false;
-      uint32_t last_parity[2][kStages] = {{0u, 0u}, {0u, 0u}};
       const int32_t* const flags = a.flags + inst.tile_base;
       auto tile = [&](int i, int j) { return i * inst.nt - i * (i - 1) / 2 + (j - i); };
       // the lane's flag of segment K, for lanes 0 .. 2: tiles (I, K), (K, J), (K + 1, J)
@@ -306,8 +305,9 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
         }
         got = __shfl_sync(~0u, (int)got, 0) != 0;
         if (got) {
-          issued[g][st] = true;
-          last_parity[g][st] = round & 1u;
+          const uint32_t bit = 1u << (g * kStages + st);
+          issued |= bit;
+          parity = (round & 1u) ? parity | bit : parity & ~bit;
         }
         return got;
       };
@@ -342,8 +342,8 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
         const int g = q & 1;
         const uint32_t u = use_cnt[g]++;
         if (finisher && q >= nseg - 2) {
-          late_k[g] = K;
-          late_u[g] = u;
+          if (g == 0) late_k[0] = K, late_u[0] = u;
+          else late_k[1] = K, late_u[1] = u;
           return;
         }
         if (!ok) return;
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
         int32_t target = lane == 9 ? task.nparts : 0;
         if (lane < 6) {
           const int g = lane / 3;
-          if (want[g]) f = segment_flag(late_k[g], lane - 3 * g), target = 1;
+          if (nseg > g) f = segment_flag(g == 0 ? late_k[0] : late_k[1], lane - 3 * g), target = 1;
         } else if (lane < 9 && D >= 1) {
           f = flags + (lane == 6 ? tile(I, I) : lane == 7 ? tile(J, J) : tile(I + 1, J));
           target = 1;
@@ -396,7 +396,8 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
         // No bulk copy may still be in flight when the task ends.
         for (int g = 0; g < 2; ++g)
           for (int st = 0; st < kStages; ++st)
-            if (issued[g][st]) mbar_wait(&bar_full[g * kStages + st], last_parity[g][st], limit * 4);
+            if (issued >> (g * kStages + st) & 1u)
+              mbar_wait(&bar_full[g * kStages + st], parity >> (g * kStages + st) & 1u, limit * 4);
         if (fin_issued) mbar_wait(bar_fin, fin_cnt & 1u, limit * 4);
       }
     } else {
