@@ -951,11 +951,16 @@ dp_status sdp_solve(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, dp_op 
   // long tables: chunks from jumped windows, side by side (sdp_jump.cu for +,
   // sdp_minjump.cu for min), or for min the cells before the periodic tail
   // beside its fill; the cost models decide
-  const SdpRoute route = sdp_route(n, a, k, op, ds->sms);
+  SdpRoute route = sdp_route(n, a, k, op, ds->sms);
   int32_t* status = status_dev ? status_dev : ds->status;
-  if (route.chunks >= 2)
-    return op == DP_OP_ADD_MOD32 ? sdp_add_jump(ST, n, a, k, route.chunks, status, static_cast<cudaStream_t>(stream))
-                                 : sdp_min_jump(ST, n, a, k, route.chunks, status, static_cast<cudaStream_t>(stream));
+  if (route.chunks >= 2 && op == DP_OP_MIN)
+    return sdp_min_jump(ST, n, a, k, route.chunks, status, static_cast<cudaStream_t>(stream));
+  if (route.chunks >= 2) {
+    bool no_scratch = false;
+    rc = sdp_add_jump(ST, n, a, k, route.chunks, status, static_cast<cudaStream_t>(stream), &no_scratch);
+    if (rc != DP_OK || !no_scratch) return rc;
+    route = SdpRoute{};
+  }
   dpk::SdpLaunchArgs args;
   sdp_single_args(&args, ST, n, a, k, op, route, ds->sms, status);
   const bool prof = profiling();

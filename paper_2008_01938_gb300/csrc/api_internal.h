@@ -121,8 +121,10 @@ int sdp_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms, double* us 
 // The plan behind it (host arithmetic only): P, L, L0, squarings, reach of
 // the impulse response, chunks per major window, major windows, chunks asked.
 int sdp_jump_plan(int64_t n, const int32_t* a, int32_t k, int sms, int64_t out[8]);
+// Without memory for its workspace it sets *no_scratch, where given, and enqueues
+// nothing: the table is then to be solved step by step.
 dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int chunks, int32_t* status,
-                       cudaStream_t st);
+                       cudaStream_t st, bool* no_scratch = nullptr);
 // (x) = min on one instance, by chunks whose windows come from Boolean
 // products modulo the characteristic polynomial (sdp_minjump.cu): whether the
 // path applies (a_k >= 32, a_1 <= 8192, a long enough table, the window on

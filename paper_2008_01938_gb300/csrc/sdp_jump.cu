@@ -595,7 +595,7 @@ int sdp_jump_plan(int64_t n, const int32_t* a, int32_t k, int sms, int64_t out[8
 }
 
 dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int chunks, int32_t* status,
-                       cudaStream_t st) {
+                       cudaStream_t st, bool* no_scratch) {
   using dpk::ToepArgs;
   DevState* ds = nullptr;
   dp_status rc = current_dev(&ds);
@@ -660,6 +660,11 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
   const size_t o_pre = take(2 * sizeof(dpk::SdpInstDev));
   uint8_t* ws = nullptr;
   cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&ws), off, st);
+  if (e == cudaErrorMemoryAllocation && no_scratch) {
+    cudaGetLastError();
+    *no_scratch = true;
+    return DP_OK;
+  }
   if (e != cudaSuccess) return fail_cuda(e, "sdp jump: workspace");
   int32_t* d_offs = reinterpret_cast<int32_t*>(ws + o_offs);
   uint32_t* hbuf = reinterpret_cast<uint32_t*>(ws + o_h);

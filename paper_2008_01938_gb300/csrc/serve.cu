@@ -376,12 +376,19 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
       if ((e = dpk::launch_sdp(args, st)) != cudaSuccess) return fail_cuda(e, "serve: S-DP launch");
       continue;
     }
+    bool no_scratch = false;
     const dp_status rc = op == DP_OP_MIN
                              ? sdp_min_jump(st_all + st_off[b], r->n, r->offs.data(), (int32_t)r->offs.size(), route[b].chunks,
                                             d_status, st)
                              : sdp_add_jump(st_all + st_off[b], r->n, r->offs.data(), (int32_t)r->offs.size(), route[b].chunks,
-                                            d_status, st);
+                                            d_status, st, &no_scratch);
     if (rc != DP_OK) return rc;
+    if (no_scratch) {
+      dpk::SdpLaunchArgs args;
+      sdp_single_args(&args, st_all + st_off[b], r->n, r->offs.data(), (int)r->offs.size(), op, SdpRoute{}, ds->sms,
+                      d_status);
+      if ((e = dpk::launch_sdp(args, st)) != cudaSuccess) return fail_cuda(e, "serve: S-DP launch");
+    }
   }
   if ((e = cudaMemcpyAsync(L->status_host, d_status, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
     return fail_cuda(e, "serve: status readback");
