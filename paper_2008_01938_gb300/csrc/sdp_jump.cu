@@ -68,10 +68,10 @@ namespace {
 // is A / kTB whole blocks (plus one for the last 127 outputs) and never a
 // skew pair of half-filled ones.  Blocks of 2048 outputs rather than 4096, a
 // thread's staging loads all in flight, and sums added 32 neighbouring words
-// at a time: one squaring of 8192 words 16.8 -> 13.0 us and its reduction
-// 13.6 -> 9.8, four of each 36 -> 27.7 and 29.3 -> 21.3 (cold cache).  With
-// early launches and pieces of 64 splits for the products, 2^24 cells: a_1 =
-// 8192, k = 32: 748 -> 599 us, a_1 = 12000: 1423 -> 997.
+// at a time, and short pieces: one squaring of 8192 words 16.8 -> 11.0 us and
+// its reduction 13.6 -> 9.0, four of each 36 -> 27.8 and 29.3 -> 18.7 (cold
+// cache).  With early launches too, 2^24 cells: a_1 = 8192, k = 32: 748 -> 599
+// us, a_1 = 12000: 1423 -> 997.
 // ---------------------------------------------------------------------------
 constexpr int kTT = 128;                // threads per block
 constexpr int kTo = 16;                 // outputs per thread
