@@ -391,8 +391,10 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
         ok = polled && got;
       }
       if (lane == 0) {
-        // keep the finisher barrier's phase sequence intact for the consumers
-        if (finisher && !fin_issued) mbar_arrive(bar_fin);
+        // (A finisher whose operands' flags did not come copies nothing, and its
+        // compute threads' wait runs out as well: the tile is then neither
+        // solved nor published, and with the status word set this is the block's
+        // last task.)
         // No bulk copy may still be in flight when the task ends.
         for (int g = 0; g < 2; ++g)
           for (int st = 0; st < kStages; ++st)

@@ -177,6 +177,39 @@ def test_bounded_wait_timeout_is_reported(dp):
     _check(dp, inputs.mcm_dims(120, 1, 32, seed=12), "i32")
 
 
+@pytest.mark.parametrize("cost", ["i32", "i64"])
+@pytest.mark.parametrize("entry, tile", [(3, (3, 3)), (0, (0, 0)), (8, (1, 2))])
+def test_tiles_without_operands_are_not_written(dp, cost, entry, tile):
+    """As above: a tile that waits for the dropped one in vain leaves m and s
+    as they were (the tile and its mirror image below the diagonal), the tiles
+    beside them are right or untouched.  Nearest neighbours have no external
+    splits, so nothing but the arrival of their operands holds them back."""
+    import ctypes
+
+    import torch
+    from paper_2008_01938_gb300 import native
+    n, T, unset = 200, 32, -7
+    dims = inputs.mcm_dims(n, 1, 32, seed=11)
+    p = torch.from_numpy(dims).cuda()
+    m = torch.full((n, n), unset, dtype=torch.int32 if cost == "i32" else torch.int64, device="cuda")
+    s = torch.full((n, n), unset, dtype=torch.int16, device="cuda")
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    rc = native.load().dp_test_mcm_drop_task(
+        ctypes.c_void_p(p.data_ptr()), n, int(cost == "i64"), ctypes.c_void_p(m.data_ptr()),
+        ctypes.c_void_p(s.data_ptr()), ctypes.c_void_p(status.data_ptr()),
+        ctypes.c_void_p(torch.cuda.current_stream().cuda_stream), entry, 2_000_000)
+    assert rc == 0
+    torch.cuda.synchronize()
+    assert int(status.item()) == native.DP_ETIMEOUT
+    want_m, want_s = oracle.mcm(dims)
+    at = np.arange(n) // T
+    lo, hi = np.minimum.outer(at, at), np.maximum.outer(at, at)
+    waits = (lo <= tile[0]) & (hi >= tile[1])
+    for got, want in ((m.cpu().numpy(), want_m), (s.cpu().numpy(), want_s)):
+        assert (got[waits] == unset).all()
+        assert ((got == want) | (got == unset))[~waits].all()
+
+
 def _sha(a):
     return hashlib.sha256(np.ascontiguousarray(a).tobytes()).hexdigest()
 
