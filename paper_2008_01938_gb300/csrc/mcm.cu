@@ -425,10 +425,9 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
         const int st = u % kStages;
         const uint32_t round = u / kStages;
         if (!ok) return;
-        bool got;
         // a finisher's segments are on the critical path: poll more often
-                got = finisher ? mbar_wait_cap(&bar_full[g * kStages + st], round & 1u, limit, kFinPollNs)
-                               : mbar_wait(&bar_full[g * kStages + st], round & 1u, limit);
+        const bool got = finisher ? mbar_wait_cap(&bar_full[g * kStages + st], round & 1u, limit, kFinPollNs)
+                                  : mbar_wait(&bar_full[g * kStages + st], round & 1u, limit);
         if (!got) {
           set_status(status, DP_ETIMEOUT);
           ok = false;
@@ -489,8 +488,7 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
           }
         }
         const uint32_t fpar = fin_cnt & 1u;
-        bool fin_ok;
-        fin_ok = mbar_wait_cap(bar_fin, fpar, limit, kFinPollNs);
+        const bool fin_ok = mbar_wait_cap(bar_fin, fpar, limit, kFinPollNs);
         if (!fin_ok) set_status(status, DP_ETIMEOUT);
         const bool go = bar_compute_and(fin_ok && failed == 0);
         const int n = inst.n;
@@ -754,8 +752,7 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
             for (int r = 0; r < 4; ++r) {
               const int li = 4 * w + r;
               pi[r] = (E)finPP[li];
-              cb[r] = bestS[li * T + lane];
-              if (task.nparts > 0) cb[r] = umin(cb[r], finAcc[li * T + lane]);
+              cb[r] = ~0ull;  // (no external splits)
             }
             const E pj1d = (E)(finPKI[lane] >> S);
             bool keyed = false;
@@ -856,20 +853,13 @@ __global__ void __launch_bounds__(kMcmThreads, 3) mcm_main_kernel(const McmLaunc
           for (int r = 0; r < 4; ++r) {
             const int li = 4 * w + r;
             const int64_t i = IT + li, j = JT + lane;
-            const bool upper = D >= 1 || li < lane;
+            const bool upper = li < lane;
             const E v = upper ? (E)(cb[r] >> KB) + wt[r] : (E)0;
             const int kk = upper ? (int)(cb[r] & kmask) : -1;
             vals[r] = v;
             if (i < nn && j < nn) {
               static_cast<int32_t*>(inst.m)[i * nn + j] = (int32_t)v;
               inst.s[i * nn + j] = (int16_t)kk;
-            }
-            if (D >= 1) {  // mirror tile (J, I) in the lower triangle
-              const int64_t i2 = JT + li, j2 = IT + lane;
-              if (i2 < nn && j2 < nn) {
-                static_cast<int32_t*>(inst.m)[i2 * nn + j2] = 0;
-                inst.s[i2 * nn + j2] = -1;
-              }
             }
           }
           // packed row panel: af[tile][k = lane][row]
