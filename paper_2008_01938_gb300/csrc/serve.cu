@@ -96,6 +96,7 @@ struct Server {
   int inflight = 0;
   uint64_t next_ticket = 1;
   std::vector<cudaStream_t> streams;
+  std::vector<cudaStream_t> sides;  // one beside each stream (Fork)
   int rr = 0;
   std::chrono::steady_clock::time_point t0;
   std::vector<std::pair<void*, size_t>> pinned_pool;  // free pinned buffers
@@ -214,12 +215,18 @@ dp_status launch_mcm_group(Server* S, const std::vector<Req*>& reqs, bool i64, L
   return DP_OK;
 }
 
+// How a request of an S-DP group is solved: by a block of the shared launch
+// of those whose window fits on chip, by one of the shared launch of those
+// whose does not, or in launches of its own.
+enum SdpShare : int32_t { kSharedRing = 0, kSharedOffRing = 1, kOwnLaunch = 2 };
+
 // Solves in chunks run one after another, the blocks of the shared launch side
 // by side: of the requests with a route in chunks, the i that would hold the
 // shared launch up longest keep it, for the i with the least total time.
 // (A dozen requests of 2e5 cells, k = 16, a_k = 64: in chunks 170 us each, in
-// the shared launch 310 for all.)
-void sdp_share_launch(const std::vector<Req*>& reqs, SdpRoute* route) {
+// the shared launch 310 for all.)  Windows that are too wide for the ring have
+// no say in it: they run beside.
+void sdp_share_launch(const std::vector<Req*>& reqs, const std::vector<SdpShare>& share, SdpRoute* route) {
   auto plain_us = [&](size_t b) {
     return sdp_plain_us(reqs[b]->n - reqs[b]->offs[0], reqs[b]->offs.back(), (int32_t)reqs[b]->offs.size());
   };
@@ -228,7 +235,7 @@ void sdp_share_launch(const std::vector<Req*>& reqs, SdpRoute* route) {
   for (size_t b = 0; b < reqs.size(); ++b) {
     if (route[b].chunks >= 2)
       by_time.emplace_back(plain_us(b), b);
-    else
+    else if (share[b] == kSharedRing)
       others = std::max(others, plain_us(b));
   }
   std::sort(by_time.rbegin(), by_time.rend());
@@ -245,32 +252,65 @@ void sdp_share_launch(const std::vector<Req*>& reqs, SdpRoute* route) {
   for (size_t i = keep; i < by_time.size(); ++i) route[by_time[i].second] = SdpRoute{};
 }
 
+// The routes and launches of a group's requests (host arithmetic only).
+std::vector<SdpShare> sdp_share(const std::vector<Req*>& reqs, int op, int sms, SdpRoute* route) {
+  std::vector<SdpShare> share(reqs.size());
+  for (size_t b = 0; b < reqs.size(); ++b) {
+    const Req* r = reqs[b];
+    int32_t threads = 0, ring_log2 = 0;
+    sdp_shape(r->offs[0], r->offs.back(), &threads, &ring_log2);
+    share[b] = ring_log2 > 0 ? kSharedRing : kSharedOffRing;
+    if (r->n > r->offs[0]) route[b] = sdp_route(r->n, r->offs.data(), (int)r->offs.size(), op, sms);
+  }
+  if (op == DP_OP_ADD_MOD32) sdp_share_launch(reqs, share, route);
+  // in launches of its own: a request in chunks, or with a tail long enough to
+  // fill from several SMs (one SM writes 2^18 cells in about 10 us)
+  for (size_t b = 0; b < reqs.size(); ++b)
+    if (route[b].chunks >= 2 || (route[b].tail_from > 0 && reqs[b]->n - route[b].tail_from > (1 << 18)))
+      share[b] = kOwnLaunch;
+  return share;
+}
+
+// Work of a group on the stream beside its own: begins after what the group's
+// stream holds so far, and the stream waits for it when the fork goes.
+struct Fork {
+  cudaStream_t main, side;
+  cudaEvent_t ev = nullptr;
+  Fork(cudaStream_t m, cudaStream_t s) : main(m), side(s) {}
+  cudaError_t begin() {
+    cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e == cudaSuccess && (e = cudaEventRecord(ev, main)) == cudaSuccess) e = cudaStreamWaitEvent(side, ev, 0);
+    return e;
+  }
+  cudaError_t join() {
+    if (!ev) return cudaSuccess;
+    cudaError_t e = cudaEventRecord(ev, side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(main, ev, 0);
+    cudaEventDestroy(ev);
+    ev = nullptr;
+    return e;
+  }
+  ~Fork() { join(); }
+};
+
 // A group of S-DP requests with one operator.  Requests long enough for the
 // chunked paths of sdp_solve (sdp_jump.cu for +, sdp_minjump.cu for min; the
 // same cost models decide) or with a long periodic tail run through those,
-// spread over the SMs; the others share one launch of the S-DP kernel, one block each.  Everything is
-// enqueued on the launch's stream, so one event covers the group.
+// spread over the SMs.  The others share a launch of the S-DP kernel, one
+// block each; those with a window too wide for the ring share another, beside
+// it, so that they cost the rest neither its ring nor its tails.  Everything
+// is ordered on the launch's stream, so one event covers the group.
 dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Launch* L) {
-  int threads = 32, kmax = 1, ring_log2 = 1;
   DevState* ds = nullptr;
   dp_status rc0 = current_dev(&ds);
   if (rc0 != DP_OK) return rc0;
   std::vector<SdpRoute> route(reqs.size());
-  std::vector<size_t> bat;  // requests of the shared launch
-  // a request in chunks, or with a tail long enough to fill from several SMs
-  // (one SM writes 2^18 cells in about 10 us)
-  auto own_launch = [&](size_t b) {
-    return route[b].chunks >= 2 || (route[b].tail_from > 0 && reqs[b]->n - route[b].tail_from > (1 << 18));
-  };
-  for (size_t b = 0; b < reqs.size(); ++b) {
-    const Req* r = reqs[b];
-    const int k = (int)r->offs.size();
-    if (r->n > r->offs[0]) route[b] = sdp_route(r->n, r->offs.data(), k, op, ds->sms);
-  }
-  if (op == DP_OP_ADD_MOD32) sdp_share_launch(reqs, route.data());
-  for (size_t b = 0; b < reqs.size(); ++b)
-    if (!own_launch(b)) bat.push_back(b);
-  bool ring_ok = true, same_k = true;
+  const std::vector<SdpShare> share = sdp_share(reqs, op, ds->sms, route.data());
+  std::vector<size_t> bat;  // requests of the shared launches: first those with a ring
+  for (SdpShare which : {kSharedRing, kSharedOffRing})
+    for (size_t b = 0; b < reqs.size(); ++b)
+      if (share[b] == which) bat.push_back(b);
+  const size_t nring = (size_t)std::count(share.begin(), share.end(), kSharedRing);
   std::vector<int64_t> st_off(reqs.size());
   int64_t cells = 0, noffs = 0;
   for (size_t b = 0; b < reqs.size(); ++b) {
@@ -278,22 +318,6 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
     st_off[b] = cells;
     cells = (int64_t)align_up((size_t)(cells + std::max<int64_t>(r->n, r->offs[0])), 64);
     noffs += (int64_t)r->offs.size();
-  }
-  for (size_t b : bat) {
-    const Req* r = reqs[b];
-    kmax = std::max(kmax, (int)r->offs.size());
-    same_k = same_k && r->offs.size() == reqs[bat[0]]->offs.size();
-    int th, lg;
-    sdp_shape(r->offs[0], r->offs.back(), &th, &lg);
-    threads = std::max(threads, th);
-  }
-  for (size_t b : bat) {
-    const Req* r = reqs[b];
-    const int W = std::min<int>(r->offs.back(), threads);
-    int lg = 0;
-    while ((1ll << lg) < (long long)r->offs[0] + W) ++lg;
-    if (lg > dpk::kSdpRingMaxLog2) ring_ok = false;
-    ring_log2 = std::max(ring_log2, lg);
   }
   size_t off = 0;
   auto take = [&](size_t b) { size_t o = off; off = align_up(off + std::max<size_t>(b, 16), 256); return o; };
@@ -335,7 +359,7 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
     insts[i].k = (int32_t)reqs[b]->offs.size();
     insts[i].a = reinterpret_cast<const int32_t*>(ws + o_offs) + a_at[b];
     insts[i].a_off = (int32_t)a_at[b];
-    insts[i].tail_from = ring_ok ? route[b].tail_from : 0;
+    insts[i].tail_from = route[b].tail_from;
     insts[i].g = route[b].g;
     bat_off[i] = st_off[b];
   }
@@ -352,22 +376,39 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
                        cudaSuccess)
       return fail_cuda(e, "serve: preset copy");
   }
-  if (!bat.empty()) {
+  // requests bat[i0 .. i1) in one launch
+  auto launch_shared = [&](size_t i0, size_t i1, cudaStream_t on) {
     dpk::SdpLaunchArgs args{};
-    args.insts = reinterpret_cast<const dpk::SdpInstDev*>(ws + o_insts);
-    args.one.k = kmax;
-    args.same_k = same_k;
-    args.ninst = (int32_t)bat.size();
+    args.same_k = 1;
+    args.threads = 32;
+    args.one.k = 1;
+    for (size_t i = i0; i < i1; ++i) {
+      const Req* r = reqs[bat[i]];
+      const int32_t k = (int32_t)r->offs.size();
+      int32_t threads = 0, ring_log2 = 0;
+      sdp_shape(r->offs[0], r->offs.back(), &threads, &ring_log2);
+      args.threads = std::max(args.threads, threads);
+      args.ring_log2 = std::max(args.ring_log2, ring_log2);
+      args.one.k = std::max(args.one.k, k);
+      args.same_k = args.same_k && k == (int32_t)reqs[bat[i0]]->offs.size();
+    }
+    args.insts = reinterpret_cast<const dpk::SdpInstDev*>(ws + o_insts) + i0;
+    args.ninst = (int32_t)(i1 - i0);
     args.op = op;
-    args.threads = threads;
-    args.ring_log2 = ring_ok ? ring_log2 : 0;
     args.st_all = st_all;
-    args.st_off = reinterpret_cast<const int64_t*>(ws + o_stoff);
+    args.st_off = reinterpret_cast<const int64_t*>(ws + o_stoff) + i0;
     args.status = d_status;
-    if ((e = dpk::launch_sdp(args, st)) != cudaSuccess) return fail_cuda(e, "serve: S-DP launch");
-  }
+    return dpk::launch_sdp(args, on);  // (nothing for an empty range)
+  };
+  const cudaStream_t side = S->sides[L->stream];
+  Fork fork(st, side);
+  const bool beside = nring < bat.size() && bat.size() - nring < reqs.size();
+  if (beside && (e = fork.begin()) != cudaSuccess) return fail_cuda(e, "serve: side stream");
+  if ((e = launch_shared(nring, bat.size(), beside ? side : st)) != cudaSuccess ||
+      (e = launch_shared(0, nring, st)) != cudaSuccess)
+    return fail_cuda(e, "serve: S-DP launch");
   for (size_t b = 0; b < reqs.size(); ++b) {
-    if (!own_launch(b)) continue;
+    if (share[b] != kOwnLaunch) continue;
     const Req* r = reqs[b];
     if (route[b].chunks < 2) {
       dpk::SdpLaunchArgs args;
@@ -390,6 +431,7 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
       if ((e = dpk::launch_sdp(args, st)) != cudaSuccess) return fail_cuda(e, "serve: S-DP launch");
     }
   }
+  if ((e = fork.join()) != cudaSuccess) return fail_cuda(e, "serve: side stream");
   if ((e = cudaMemcpyAsync(L->status_host, d_status, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess)
     return fail_cuda(e, "serve: status readback");
   cudaFreeAsync(ws, st);
@@ -512,18 +554,40 @@ dp_status serve_create(const dp_serve_config* cfg, void** srv) {
   auto* S = new Server();
   S->cfg = *cfg;
   S->t0 = std::chrono::steady_clock::now();
-  for (int i = 0; i < cfg->num_streams; ++i) {
+  for (int i = 0; i < 2 * cfg->num_streams; ++i) {
     cudaStream_t st;
     if ((e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking)) != cudaSuccess) {
       for (auto s : S->streams) cudaStreamDestroy(s);
+      for (auto s : S->sides) cudaStreamDestroy(s);
       delete S;
       return fail_cuda(e, "serve_create: stream");
     }
-    S->streams.push_back(st);
+    (i % 2 == 0 ? S->streams : S->sides).push_back(st);
   }
   S->th = std::thread(scheduler, S);
   *srv = S;
   return DP_OK;
+}
+
+// Test hook without a device: how the server would solve a group of (x) = op
+// requests on a device of `sms` SMs; out[b]: an SdpShare, and with bit 8 set a
+// request whose periodic tail is written.  offs: the requests' offsets, one
+// after the other.
+int32_t dp_test_serve_sdp_share(int32_t count, const int64_t* n, const int32_t* k, const int32_t* offs, int32_t op,
+                                int32_t sms, int32_t* out) {
+  if (count < 1 || !n || !k || !offs || !out) return -1;
+  std::vector<Req> req((size_t)count);
+  std::vector<Req*> reqs;
+  for (int32_t b = 0; b < count; offs += k[b], ++b) {
+    if (sdp_validate(n[b], offs, k[b], op) != DP_OK) return -1;
+    req[b].n = n[b];
+    req[b].offs.assign(offs, offs + k[b]);
+    reqs.push_back(&req[b]);
+  }
+  std::vector<SdpRoute> route(reqs.size());
+  const std::vector<SdpShare> share = sdp_share(reqs, op, sms, route.data());
+  for (int32_t b = 0; b < count; ++b) out[b] = share[b] | (route[b].tail_from > 0 ? 256 : 0);
+  return count;
 }
 
 dp_status serve_submit(void* srv, const dp_request* req, uint64_t* ticket) {
@@ -645,6 +709,10 @@ dp_status serve_destroy(void* srv) {
     delete r;
   }
   for (auto s : S->streams) {
+    cudaStreamSynchronize(s);
+    cudaStreamDestroy(s);
+  }
+  for (auto s : S->sides) {
     cudaStreamSynchronize(s);
     cudaStreamDestroy(s);
   }

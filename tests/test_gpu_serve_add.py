@@ -29,3 +29,26 @@ def test_groups(lengths):
         assert np.array_equal(got, oracle.sdp(p, n, a, "add")[:n])
         srv.release(t)
     srv.close()
+
+
+@pytest.mark.parametrize("op", ["min", "add"])
+@pytest.mark.parametrize("others", [[], [200000, 1 << 22], [200000] * 6 + [900, 1000]])
+def test_a_wide_window_among_others(op, others):
+    """A window too wide for the ring is solved beside the others of its group
+    (first, last, and alone in the group)."""
+    import paper_2008_01938_gb300 as dp
+    r = np.random.RandomState(len(others))
+    a = np.sort(np.r_[64, 1000, r.choice(np.arange(65, 1000), 14, replace=False)])[::-1].astype(np.int32)
+    wide = np.array([40000, 39000, 1024], np.int32)
+    requests = [(130001, wide)] + [(n, a) for n in others] + [(90000, wide), (40000, wide)]
+    presets = [r.randint(0, 1 << 32, q[0], dtype=np.uint64).astype(np.uint32) for _, q in requests]
+    srv = dp.Server()
+    tickets = [srv.submit_sdp(n, q, p, op=op) for (n, q), p in zip(requests, presets)]
+    for (n, q), p, t in zip(requests, presets, tickets):
+        while (res := srv.poll(t)) is None:
+            pass
+        assert res.status == 0
+        got = srv.tables(res).cpu().numpy().view(np.uint32)[:n]
+        assert np.array_equal(got, oracle.sdp(p, n, q, op)[:n])
+        srv.release(t)
+    srv.close()

@@ -52,6 +52,37 @@ def test_tail_is_found_where_it_matters():
     assert tail([8192, 8191], 1 << 26)[0] == 0  # fills in too slowly to be found
 
 
+SPREAD = list(range(1000, 63, -67)) + [64]  # 16 offsets, window on chip
+WIDE = [40000, 39000, 1024]                 # window too wide for the ring
+
+
+def share(requests, op):
+    """The server's decision for a group: (launch, whether the tail is written) per request."""
+    n = np.array([r[0] for r in requests], np.int64)
+    k = np.array([len(r[1]) for r in requests], np.int32)
+    offs = np.concatenate([np.asarray(r[1], np.int32) for r in requests])
+    out = np.zeros(n.size, np.int32)
+    ptr = lambda x: ctypes.c_void_p(x.ctypes.data)  # noqa: E731
+    assert native.load().dp_test_serve_sdp_share(n.size, ptr(n), ptr(k), ptr(offs), op, 152, ptr(out)) == n.size
+    return [(("ring", "off ring", "own")[x & 255], bool(x & 256)) for x in out]
+
+
+@pytest.mark.parametrize("op", [0, 1])
+@pytest.mark.parametrize("others", [[200000], [200000] * 12, [1 << 22, 200000, 90000, 500]])
+@pytest.mark.parametrize("wide", [300000, 1 << 22])
+def test_a_wide_window_leaves_a_served_group_its_routes(op, others, wide):
+    """A request whose window does not fit on chip goes off the ring by itself:
+    the others are solved as they would be without it."""
+    group = [(n, SPREAD) for n in others]
+    alone = share(group, op)
+    for at in (0, len(group)):
+        got = share(group[:at] + [(wide, WIDE)] + group[at:], op)
+        assert got.pop(at) == ("off ring", False)
+        assert got == alone
+    assert all(g[0] != "off ring" for g in alone)
+    assert all(g[1] for g, n in zip(alone, others) if n > 10000) if op == 0 else not any(g[1] for g in alone)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("a,n", CASES + [([8192, 7000, 5001, 3333, 1024], 5000003), ([1280, 768, 256], 1 << 20)])
 @pytest.mark.parametrize("shift", [0, 1])
