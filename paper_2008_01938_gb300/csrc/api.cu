@@ -65,6 +65,18 @@ struct ProfPair {
 std::vector<ProfPair> g_prof_ev;
 }  // namespace
 
+namespace {
+std::atomic<int32_t> g_refuse_scratch{0};  // workspace requests still to be refused
+}
+
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st) {
+  for (int32_t left = g_refuse_scratch.load(std::memory_order_relaxed); left > 0;)
+    if (g_refuse_scratch.compare_exchange_weak(left, left - 1)) return cudaErrorMemoryAllocation;
+  const cudaError_t e = cudaMallocAsync(p, bytes, st);
+  if (e == cudaErrorMemoryAllocation) cudaGetLastError();  // not sticky: whoever asks has another way
+  return e;
+}
+
 bool profiling() { return g_prof.load(std::memory_order_relaxed); }
 
 void profile_mark(int which, cudaStream_t st, bool after) {
@@ -437,8 +449,16 @@ SdpRoute sdp_route(int64_t n, const int32_t* a, int32_t k, int op, int sms) {
   sdp_shape(a[0], a[k - 1], &threads, &ring_log2);
   if (ring_log2 <= 0) r.tail_from = 0;  // the fill keeps the class minima where the ring would be
   r.chunks = sdp_min_jump_chunks(n, a, k, sms, r.tail_from);
-  if (r.chunks >= 2) r.tail_from = 0;
   return r;
+}
+
+dp_status sdp_in_chunks(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int op, SdpRoute* route,
+                        int32_t* status, cudaStream_t st) {
+  bool no_scratch = false;
+  const dp_status rc = op == DP_OP_MIN ? sdp_min_jump(ST, n, a, k, route->chunks, status, st, &no_scratch)
+                                       : sdp_add_jump(ST, n, a, k, route->chunks, status, st, &no_scratch);
+  if (no_scratch) route->chunks = 0;
+  return rc;
 }
 
 void sdp_single_args(dpk::SdpLaunchArgs* args, uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int op,
@@ -741,6 +761,11 @@ int32_t dp_test_mcm_device_queue(const int32_t* ns, int32_t m, int32_t i64, int3
   return test_queue(ns, m, i64, out, cap, true);
 }
 
+// Test hook: the next `count` workspace requests of the S-DP paths in chunks
+// are told that there is no memory.  Returns how many of the last call's are
+// still to come.
+int32_t dp_test_refuse_scratch(int32_t count) { return g_refuse_scratch.exchange(count); }
+
 // Test hooks for the (x) = + jump path: the number of chunks sdp_solve would
 // use, and the path itself with a given number of chunks.
 int32_t dp_test_sdp_jump_chunks(int64_t n, const int32_t* a, int32_t k) {
@@ -953,13 +978,9 @@ dp_status sdp_solve(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, dp_op 
   // beside its fill; the cost models decide
   SdpRoute route = sdp_route(n, a, k, op, ds->sms);
   int32_t* status = status_dev ? status_dev : ds->status;
-  if (route.chunks >= 2 && op == DP_OP_MIN)
-    return sdp_min_jump(ST, n, a, k, route.chunks, status, static_cast<cudaStream_t>(stream));
   if (route.chunks >= 2) {
-    bool no_scratch = false;
-    rc = sdp_add_jump(ST, n, a, k, route.chunks, status, static_cast<cudaStream_t>(stream), &no_scratch);
-    if (rc != DP_OK || !no_scratch) return rc;
-    route = SdpRoute{};
+    rc = sdp_in_chunks(ST, n, a, k, op, &route, status, static_cast<cudaStream_t>(stream));
+    if (rc != DP_OK || route.chunks >= 2) return rc;
   }
   dpk::SdpLaunchArgs args;
   sdp_single_args(&args, ST, n, a, k, op, route, ds->sms, status);

@@ -29,6 +29,10 @@ struct DevState {
 // Per-device state for the current device (created on first use).
 dp_status current_dev(DevState** out);
 
+// Stream-ordered workspace of an S-DP path that has another way without it
+// (dp_test_refuse_scratch makes it report that there is no memory).
+cudaError_t scratch_alloc(void** p, size_t bytes, cudaStream_t st);
+
 cudaError_t traceback_configure();  // kernel attributes of the current device (traceback.cu)
 
 long long spin_limit();     // bounded-wait budget in clock cycles
@@ -102,7 +106,8 @@ void sdp_shape(int32_t a1, int32_t ak, int* threads, int* ring_log2);
 // sdp_kernels.cuh).  0: not below n, or not found within a bounded search.
 int64_t sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g);
 // How one table is solved: in `chunks` >= 2 chunks from jumped windows, or by
-// the step kernel, with tail_from > 0 up to there and the rest filled.
+// the step kernel, with tail_from > 0 up to there and the rest filled (known
+// with chunks too, for when their workspace cannot be had).
 struct SdpRoute {
   int chunks = 0;
   int64_t tail_from = 0;
@@ -110,6 +115,10 @@ struct SdpRoute {
   double us = 0.0;  // (x) = + in chunks: the model's time
 };
 SdpRoute sdp_route(int64_t n, const int32_t* a, int32_t k, int op, int sms);
+// Solves a table whose route is in chunks; without memory for the workspace
+// it enqueues nothing and turns the route into the step kernel's.
+dp_status sdp_in_chunks(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int op, SdpRoute* route,
+                        int32_t* status, cudaStream_t st);
 // Fills the arguments of the step kernel's launch for one table (not for chunks >= 2).
 void sdp_single_args(dpk::SdpLaunchArgs* args, uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int op,
                      const SdpRoute& route, int sms, int32_t* status);
@@ -134,7 +143,8 @@ bool sdp_min_jump_eligible(int64_t n, const int32_t* a, int32_t k);
 int sdp_min_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms, int64_t tail_from);
 // The plan behind it (host arithmetic only): P, L, L0, squarings, chunks asked.
 int sdp_min_jump_plan(int64_t n, const int32_t* a, int32_t k, int sms, int64_t out[5]);
+// no_scratch as for sdp_add_jump.
 dp_status sdp_min_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int chunks, int32_t* status,
-                       cudaStream_t st);
+                       cudaStream_t st, bool* no_scratch = nullptr);
 
 }  // namespace dph

@@ -659,9 +659,8 @@ dp_status sdp_add_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
   const size_t o_ext = take((size_t)std::max(P1e - 1, 1) * sizeof(dpk::SdpInstDev));
   const size_t o_pre = take(2 * sizeof(dpk::SdpInstDev));
   uint8_t* ws = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&ws), off, st);
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&ws), off, st);
   if (e == cudaErrorMemoryAllocation && no_scratch) {
-    cudaGetLastError();
     *no_scratch = true;
     return DP_OK;
   }

@@ -493,7 +493,7 @@ int sdp_min_jump_chunks(int64_t n, const int32_t* a, int32_t k, int sms, int64_t
 }
 
 dp_status sdp_min_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int chunks, int32_t* status,
-                       cudaStream_t st) {
+                       cudaStream_t st, bool* no_scratch) {
   DevState* ds = nullptr;
   dp_status rc = current_dev(&ds);
   if (rc != DP_OK) return rc;
@@ -528,7 +528,11 @@ dp_status sdp_min_jump(uint32_t* ST, int64_t n, const int32_t* a, int32_t k, int
   const size_t o_insts = take((size_t)P * sizeof(dpk::SdpInstDev));
   const size_t o_pre = take(sizeof(dpk::SdpInstDev));
   uint8_t* ws = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&ws), off, st);
+  cudaError_t e = scratch_alloc(reinterpret_cast<void**>(&ws), off, st);
+  if (e == cudaErrorMemoryAllocation && no_scratch) {
+    *no_scratch = true;
+    return DP_OK;
+  }
   if (e != cudaSuccess) return fail_cuda(e, "sdp min jump: workspace");
   int32_t* d_offs = reinterpret_cast<int32_t*>(ws + o_offs);
   uint32_t* sets = reinterpret_cast<uint32_t*>(ws + o_sets);

@@ -410,26 +410,16 @@ dp_status launch_sdp_group(Server* S, const std::vector<Req*>& reqs, int op, Lau
   for (size_t b = 0; b < reqs.size(); ++b) {
     if (share[b] != kOwnLaunch) continue;
     const Req* r = reqs[b];
-    if (route[b].chunks < 2) {
-      dpk::SdpLaunchArgs args;
-      sdp_single_args(&args, st_all + st_off[b], r->n, r->offs.data(), (int)r->offs.size(), op, route[b], ds->sms,
-                      d_status);
-      if ((e = dpk::launch_sdp(args, st)) != cudaSuccess) return fail_cuda(e, "serve: S-DP launch");
-      continue;
+    if (route[b].chunks >= 2) {
+      const dp_status rc = sdp_in_chunks(st_all + st_off[b], r->n, r->offs.data(), (int32_t)r->offs.size(), op,
+                                         &route[b], d_status, st);
+      if (rc != DP_OK) return rc;
+      if (route[b].chunks >= 2) continue;
     }
-    bool no_scratch = false;
-    const dp_status rc = op == DP_OP_MIN
-                             ? sdp_min_jump(st_all + st_off[b], r->n, r->offs.data(), (int32_t)r->offs.size(), route[b].chunks,
-                                            d_status, st)
-                             : sdp_add_jump(st_all + st_off[b], r->n, r->offs.data(), (int32_t)r->offs.size(), route[b].chunks,
-                                            d_status, st, &no_scratch);
-    if (rc != DP_OK) return rc;
-    if (no_scratch) {
-      dpk::SdpLaunchArgs args;
-      sdp_single_args(&args, st_all + st_off[b], r->n, r->offs.data(), (int)r->offs.size(), op, SdpRoute{}, ds->sms,
-                      d_status);
-      if ((e = dpk::launch_sdp(args, st)) != cudaSuccess) return fail_cuda(e, "serve: S-DP launch");
-    }
+    dpk::SdpLaunchArgs args;
+    sdp_single_args(&args, st_all + st_off[b], r->n, r->offs.data(), (int)r->offs.size(), op, route[b], ds->sms,
+                    d_status);
+    if ((e = dpk::launch_sdp(args, st)) != cudaSuccess) return fail_cuda(e, "serve: S-DP launch");
   }
   if ((e = fork.join()) != cudaSuccess) return fail_cuda(e, "serve: side stream");
   if ((e = cudaMemcpyAsync(L->status_host, d_status, 4, cudaMemcpyDeviceToHost, st)) != cudaSuccess)

@@ -351,3 +351,69 @@ def test_batched_parity(dp, op):
         ref = oracle.sdp(x.preset, x.n, x.offsets, op)
         assert np.array_equal(got[st_off[i]:st_off[i] + x.n], ref), i
     plan.destroy()
+
+
+SPREAD = list(range(1000, 63, -67)) + [64]  # 16 offsets
+# (operator, n, offsets) that sdp_solve takes in chunks; the last one would
+# otherwise be written from cell 208965 on
+IN_CHUNKS = [("add", 200000, SPREAD), ("add", 1 << 20, [4099, 300, 64]), ("min", 1 << 20, [2048, 2047, 2046]),
+             ("min", 1 << 21, [5501, 37])]
+
+
+@pytest.mark.parametrize("op, n, a", IN_CHUNKS)
+def test_solved_without_a_workspace(dp, op, n, a):
+    """Where the workspace of the path in chunks cannot be had, the table is
+    solved by the step kernel (the host is told so: no memory is exhausted)."""
+    from paper_2008_01938_gb300 import native
+    lib = native.load()
+    preset = np.random.RandomState(n % 97).randint(0, 1 << 32, a[0], dtype=np.uint64).astype(np.uint32)
+    a = np.array(a, np.int32)
+    ref = oracle.sdp(preset, n, a, op)[:n]
+    lib.dp_test_refuse_scratch(1)
+    try:
+        got = _gpu(dp, preset, n, a, op)
+    finally:
+        left = lib.dp_test_refuse_scratch(0)
+    assert left == 0, "not solved in chunks"
+    assert np.array_equal(got, ref)
+    assert np.array_equal(_gpu(dp, preset, n, a, op), ref)  # and with it
+    # served, in a group of two
+    lib.dp_test_refuse_scratch(2)
+    try:
+        srv = dp.Server()
+        tickets = [srv.submit_sdp(m, a, preset, op=op) for m in (n, n - 1)]
+        for m, t in zip((n, n - 1), tickets):
+            while (res := srv.poll(t)) is None:
+                pass
+            assert res.status == 0
+            assert np.array_equal(srv.tables(res).cpu().numpy().view(np.uint32)[:m], ref[:m])
+            srv.release(t)
+        srv.close()
+    finally:
+        lib.dp_test_refuse_scratch(0)
+
+
+@pytest.mark.parametrize("op, n, a", IN_CHUNKS)
+def test_chunks_captured_in_a_graph(dp, op, n, a):
+    """A solve in chunks (workspace and overlapping launches included) replayed
+    from a graph on other presets."""
+    import torch
+    a = np.array(a, np.int32)
+    r = np.random.RandomState(3)
+    presets = [r.randint(0, 1 << 32, a[0], dtype=np.uint64).astype(np.uint32) for _ in range(3)]
+    t = torch.zeros(n, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        dp.sdp_solve(t, a, op=op)  # kernels loaded before the capture
+        stream.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            dp.sdp_solve(t, a, op=op)
+        for preset in presets:
+            t.zero_()
+            t[:a[0]] = torch.from_numpy(preset.view(np.int32)).cuda()
+            g.replay()
+            stream.synchronize()
+            got = t.cpu().numpy().view(np.uint32)
+            assert np.array_equal(got, oracle.sdp(preset, n, a, op)[:n])
+    dp.sync_status()
