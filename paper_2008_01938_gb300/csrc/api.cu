@@ -385,41 +385,102 @@ SdpSteps::SdpSteps(int32_t ak, int32_t k) : W(std::min<int32_t>(ak, 1024)) {
 
 double sdp_plain_us(int64_t cells, int32_t ak, int32_t k) { return SdpSteps(ak, k).us(cells); }
 
-int64_t sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g_out) {
-  int32_t g = a[0], gap = a[k - 1];
-  for (int j = 1; j < k; ++j) {
-    g = std::gcd(g, a[j]);
-    gap = std::max(gap, a[j - 1] - a[j]);
+namespace {
+// The sums of offsets / g as a bitset, 64 at a time, until a_k / g consecutive
+// ones: from the first of those (c) on, every number is a sum.  The search
+// costs up to kTailOps word operations (a word about k + 8 of them, measured
+// 1.2 to 2 per nanosecond), 30 us of host time; offsets that fill in slowly
+// pay all of it for nothing.  So a single solve spends at most kTailShare of
+// the step kernel's time on it.  (Over 12000 tables of 0.02 to 700 us, the
+// search exposed: shares of 1/8, 1/4, 1/2 and 1 give 0.542, 0.528, 0.527 and 0.532
+// of the time without a tail in the geometric mean, 1.12, 1.24, 1.44 and 1.76
+// at worst, 2.48 without a limit.)
+constexpr int64_t kTailOps = 1 << 15;
+constexpr double kTailOpsPerUs = 1200.0;
+constexpr double kTailShare = 0.5;
+
+// False where a_k / g consecutive sums of offsets / g cannot begin at c <= reach:
+//   * the sums of m offsets lie in [m a_k, m a_1], and as long as m (a_1 - a_k) <
+//     a_k - g there is a hole between these and the sums of m + 1;
+//   * modulo a_k the consecutive sums are all different, and without their a_k
+//     they are sums of the other k - 1 offsets, of which there are at most
+//     (x + a_1 + .. + a_{k-1})^(k-1) / ((k-1)! a_1 .. a_{k-1}) up to x (for k = 2
+//     that gives the first c exactly).
+// Of the searches that find nothing it spares half, those of k = 2 all (7.6 us
+// each before, 0.8 now; k = 4: 11.6 and 2.2).
+bool tail_within(const int32_t* a, int32_t k, int32_t g, int64_t reach) {
+  const int64_t lo = a[k - 1] / g, hi = a[0] / g;
+  if (lo < 2) return true;  // (k = 1 among them)
+  if ((lo - 2) / (hi - lo) * hi >= reach) return false;  // the last hole is above m hi, m = ceil((lo - 1) / (hi - lo)) - 1
+  if (k > 8) return true;
+  double x = (double)(reach + lo), count = 1.0;
+  for (int j = 0; j < k - 1; ++j) x += a[j] / g;
+  for (int j = 0; j < k - 1; ++j) count *= x / ((double)(j + 1) * (a[j] / g));
+  return count >= 0.999 * (double)lo;
+}
+
+// gcd of the offsets, widest gap below an offset (a_k: to 0), and the words of
+// the bitset to search (0: nothing would be found).
+struct TailSearch {
+  int32_t g, gap;
+  int64_t words = 0;
+  TailSearch(int64_t n, const int32_t* a, int32_t k, double budget_us) : g(a[0]), gap(a[k - 1]) {
+    for (int j = 1; j < k; ++j) {
+      g = std::gcd(g, a[j]);
+      gap = std::max(gap, a[j - 1] - a[j]);
+    }
+    const int64_t room = n - ((int64_t)a[0] + gap + g);  // largest useful g c
+    if (room < 0) return;
+    const double ops = std::min<double>((double)kTailOps, budget_us * kTailOpsPerUs);
+    const int64_t most = std::min<int64_t>(std::max<int64_t>((int64_t)ops / (k + 8), 1), room / g / 64 + 1);
+    if (tail_within(a, k, g, std::min<int64_t>(room / g, 64 * most))) words = most;
   }
-  // The sums of offsets / g as a bitset, 64 at a time, until offsets[k-1] / g
-  // consecutive ones: from the first of those (c) on, every number is a sum.
-  // The search stops at the table's end, and after kTailOps word operations
-  // (a word costs about k + 8; 40 us of host time in all), which offsets that
-  // fill in slowly reach first.
-  constexpr int64_t kTailOps = 1 << 15;
-  const int64_t room = n - ((int64_t)a[0] + gap + g);  // largest useful g c
-  if (room < 0) return 0;
-  const int64_t words = std::min<int64_t>(kTailOps / (k + 8), room / g / 64 + 1);
-  std::vector<uint64_t> sum((size_t)words + 1, 0);
+};
+}  // namespace
+
+double sdp_min_tail_budget_us(int64_t n, const int32_t* a, int32_t k) {
+  return kTailShare * sdp_plain_us(n - a[0], a[k - 1], k);
+}
+
+int64_t sdp_min_tail_ops(int64_t n, const int32_t* a, int32_t k, double budget_us) {
+  return TailSearch(n, a, k, budget_us).words * (k + 8);
+}
+
+int64_t sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g_out, double budget_us) {
+  const TailSearch search(n, a, k, budget_us);
+  const int32_t g = search.g, gap = search.gap;
+  const int64_t words = search.words;
+  if (words == 0) return 0;
+  // Word w collects the sums 64 w - b .. 64 w - b + 63 of the words before it,
+  // for each b = a_j / g: bits from word w - back on, shifted by r.  (Offsets
+  // beyond the last word add nothing.)
+  struct Term {
+    int32_t back, r;
+  };
+  std::vector<Term> term;
+  std::vector<int32_t> inside;
+  int64_t pad = 1;  // words before the first, all zero
+  for (int j = 0; j < k; ++j) {
+    const int64_t b = a[j] / g, back = (b + 63) / 64;
+    if (back > words) continue;
+    term.push_back(Term{(int32_t)back, (int32_t)(64 * back - b)});
+    if (b < 64) inside.push_back((int32_t)b);
+    pad = std::max(pad, back);
+  }
+  std::vector<uint64_t> sum((size_t)(pad + words + 1), 0);
   const int64_t need = a[k - 1] / g;
   int64_t run = 0, c = -1;
   for (int64_t w = 0; w < words && c < 0; ++w) {
     uint64_t x = w == 0 ? 1u : 0u;
-    for (int j = 0; j < k; ++j) {
-      const int64_t at = 64 * w - a[j] / g;  // sums at .. at + 63, of which those in earlier words are known
-      if (at <= -64) continue;
-      const int64_t q = at >> 6;
-      const int r = (int)(at & 63);
-      const uint64_t lo = q >= 0 ? sum[(size_t)q] : 0u, hi = q + 1 >= 0 && q + 1 < w ? sum[(size_t)q + 1] : 0u;
-      x |= r == 0 ? lo : (lo >> r) | (hi << (64 - r));
-    }
-    for (int j = k - 1; j >= 0 && a[j] / g < 64; --j)  // offsets that add up inside the word
-      for (int64_t d = a[j] / g; d < 64; d *= 2) x |= x << d;
-    sum[(size_t)w] = x;
+    const uint64_t* here = sum.data() + pad + w;
+    for (const Term& t : term) x |= here[-t.back] >> t.r | here[1 - t.back] << 1 << (63 - t.r);
+    for (const int32_t b : inside)  // offsets that add up inside the word
+      for (int32_t d = b; d < 64; d *= 2) x |= x << d;
+    sum[(size_t)(pad + w)] = x;
     if (x == ~(uint64_t)0) {
       run += 64;
       if (run >= need) c = 64 * w + 64 - run;
-    } else {
+    } else if (x != 0) {
       const int low = __builtin_ctzll(~x);  // ones that continue the run from the word below
       if (run + low >= need) c = 64 * w - run;
       for (int b = low, r = 0; need < 64 && b < 64 && c < 0; ++b) {  // runs inside the word
@@ -427,6 +488,8 @@ int64_t sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g_out) {
         if (r >= need) c = 64 * w + b + 1 - r;
       }
       run = __builtin_clzll(~x);  // ones at the top start the next run
+    } else {
+      run = 0;
     }
   }
   if (c < 0) return 0;
@@ -444,10 +507,10 @@ SdpRoute sdp_route(int64_t n, const int32_t* a, int32_t k, int op, int sms) {
     r.chunks = sdp_jump_chunks(n, a, k, sms, &r.us);
     return r;
   }
-  r.tail_from = sdp_min_tail(n, a, k, &r.g);
   int threads = 0, ring_log2 = 0;
   sdp_shape(a[0], a[k - 1], &threads, &ring_log2);
-  if (ring_log2 <= 0) r.tail_from = 0;  // the fill keeps the class minima where the ring would be
+  // (the fill keeps the class minima where the ring would be)
+  if (ring_log2 > 0) r.tail_from = sdp_min_tail(n, a, k, &r.g, sdp_min_tail_budget_us(n, a, k));
   r.chunks = sdp_min_jump_chunks(n, a, k, sms, r.tail_from);
   return r;
 }
@@ -789,6 +852,14 @@ int64_t dp_test_sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g)
   for (int j = 0; j < k; ++j)
     if (a[j] < 1 || (j > 0 && a[j] >= a[j - 1])) return -1;
   return n > a[0] ? sdp_min_tail(n, a, k, g) : 0;
+}
+
+// Test hook without a device: the word operations that sdp_solve's search for
+// the tail may take, and the modelled time of the step kernel in ns.
+int64_t dp_test_sdp_min_tail_ops(int64_t n, const int32_t* a, int32_t k, int64_t* plain_ns) {
+  if (!plain_ns || sdp_validate(n, a, k, DP_OP_MIN) != DP_OK) return -1;
+  *plain_ns = (int64_t)(1e3 * sdp_plain_us(n - a[0], a[k - 1], k));
+  return sdp_min_tail_ops(n, a, k, sdp_min_tail_budget_us(n, a, k));
 }
 
 // Test hook without a device: the min jump plan sdp_solve would take for

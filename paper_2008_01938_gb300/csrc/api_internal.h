@@ -103,8 +103,12 @@ struct SdpSteps {  // the same for several lengths
 void sdp_shape(int32_t a1, int32_t ak, int* threads, int* ring_log2);
 // (x) = min: the first cell from which the table repeats its last g cells, g
 // the gcd of the offsets (host arithmetic on the offsets only; see
-// sdp_kernels.cuh).  0: not below n, or not found within a bounded search.
-int64_t sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g);
+// sdp_kernels.cuh).  0: not below n, or not found within a bounded search, of
+// about budget_us of host time where given; the budget of a single solve, and
+// the word operations that a search may take.
+int64_t sdp_min_tail(int64_t n, const int32_t* a, int32_t k, int32_t* g, double budget_us = 1e9);
+double sdp_min_tail_budget_us(int64_t n, const int32_t* a, int32_t k);
+int64_t sdp_min_tail_ops(int64_t n, const int32_t* a, int32_t k, double budget_us);
 // How one table is solved: in `chunks` >= 2 chunks from jumped windows, or by
 // the step kernel, with tail_from > 0 up to there and the rest filled (known
 // with chunks too, for when their workspace cannot be had).

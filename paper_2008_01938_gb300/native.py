@@ -99,6 +99,7 @@ def load(path: str | None = None):
             "dp_test_sdp_jump": ([vp, i64, vp, i32, i32, vp, vp], ctypes.c_int),
             "dp_test_sdp_min_jump_chunks": ([i64, vp, i32], i32),
             "dp_test_sdp_min_tail": ([i64, vp, i32, ctypes.POINTER(i32)], i64),
+            "dp_test_sdp_min_tail_ops": ([i64, vp, i32, ctypes.POINTER(i64)], i64),
             "dp_test_sdp_min_jump_plan": ([i64, vp, i32, i32, vp], i32),
             "dp_test_sdp_min_jump": ([vp, i64, vp, i32, i32, vp, vp], ctypes.c_int),
             "dp_test_refuse_scratch": ([i32], i32),

@@ -2,6 +2,7 @@
 against the oracle's whole tables), and the tables the GPU writes there."""
 import ctypes
 import math
+import random
 
 import numpy as np
 import pytest
@@ -50,6 +51,59 @@ def test_tail_is_found_where_it_matters():
     assert tail([8192, 7000, 5001, 3333, 1024], 200003)[0] > 0
     assert tail([4096, 2048, 1024], 20000)[1] == 1024
     assert tail([8192, 8191], 1 << 26)[0] == 0  # fills in too slowly to be found
+
+
+def random_offsets(r):
+    hi = int(2 ** r.uniform(1, 8))
+    lo = max(1, int(hi * r.choice([0.05, 0.3, 0.7, 0.9])))
+    k = min(r.randint(1, 6), hi - lo + 1)
+    return sorted((x * r.choice([1, 2, 3]) for x in r.sample(range(lo, hi + 1), k)), reverse=True)
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_tail_is_given_up_only_where_there_is_none(seed):
+    """Against the sums themselves: the first of a_k / g consecutive ones says
+    where the tail starts, and a table that reaches past them has one."""
+    r = random.Random(seed)
+    for _ in range(400):
+        a = sorted(set(random_offsets(r)), reverse=True)
+        g = math.gcd(*a)
+        b = [x // g for x in a]
+        top = 65 * max(b) + 64
+        sums = 1
+        for x in b:
+            while (more := (sums | sums << x) & ((1 << top) - 1)) != sums:
+                sums = more
+        run = sums
+        for i in range(1, b[-1]):
+            run &= sums >> i
+        c = (run & -run).bit_length() - 1
+        if c < 0:
+            continue
+        gap = max(x - y for x, y in zip(a, a[1:] + [0]))
+        start = g * c + a[0] - 1 + gap + g  # the tail
+        for n in (start - 5, start):
+            assert tail(a, n)[0] == 0, (a, n)
+        for n in (start + a[-1] + 64 * g, 2 * start + a[-1] + 64 * g):  # (room for the whole run)
+            assert tail(a, n)[0] == start, (a, n)
+
+
+@pytest.mark.parametrize("n, a", [
+    (1 << 20, [8192, 8191]),                    # sums of m offsets stay apart: nothing to search for
+    (1 << 18, [4000, 3001]), (65536, [1200, 801]),
+    (55786, [7935 - 46 * i for i in range(32)]),  # a short table of many offsets
+    (76589, [23045 - 1239 * i for i in range(16)]), (97000, [9000, 8501, 8102, 7503]),
+    (1 << 26, [16000, 9000, 7001]),
+])
+def test_search_is_small_beside_the_solve(n, a):
+    """The host's search for a tail (1.2 word operations or more per ns) takes
+    at most half of the time that the steps take."""
+    a = np.asarray(a, np.int32)
+    plain = ctypes.c_int64()
+    ops = native.load().dp_test_sdp_min_tail_ops(n, ctypes.c_void_p(a.ctypes.data), int(a.size), ctypes.byref(plain))
+    assert 0 <= ops <= max(0.5 * 1.2 * plain.value, a.size + 8)
+    if a.size == 2:
+        assert ops == 0
 
 
 SPREAD = list(range(1000, 63, -67)) + [64]  # 16 offsets, window on chip
