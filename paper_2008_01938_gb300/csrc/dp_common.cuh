@@ -109,6 +109,23 @@ __device__ __forceinline__ void fence_proxy_async_global() {
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Launches a kernel whose blocks may start while the previous kernel of the
+// stream still runs; it waits for that one's end (grid_dependency_wait) before
+// it reads or writes anything.
+template <class... P, class... T>
+cudaError_t launch_early(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t st, T... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+}
+
 // ---------------------------------------------------------------------------
 // global flags
 // ---------------------------------------------------------------------------

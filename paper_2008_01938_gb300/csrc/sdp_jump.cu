@@ -384,23 +384,6 @@ __global__ void __launch_bounds__(256) jump_start_kernel(uint32_t* R1, const uin
   R1[A - 1 - t] = v;
 }
 
-// The launches of a product level are short: each is started while the one
-// before it runs, and waits for its end (griddepcontrol) before it reads or
-// writes anything.
-template <class... P, class... T>
-cudaError_t launch_early(void (*kernel)(P...), dim3 grid, int threads, cudaStream_t st, T... args) {
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
-}
-
 // Blocks that share the split range of a product of `batch` items with
 // `tblocks` output blocks each, over pieces of sb splits: one piece a block
 // until there are ten blocks per SM, then as evenly as can be.
@@ -411,6 +394,7 @@ int split_count(int64_t S, int sb, int64_t tblocks, int64_t batch, int sms) {
   return (int)((most + pieces - 1) / pieces);
 }
 
+// (The launches of a product level are short: hence launch_early.)
 cudaError_t conv(ToepArgs a, int64_t batch, int sms, cudaStream_t st) {
   constexpr int sb = kSBProduct;
   const int64_t all = (a.S + sb - 1) / sb;

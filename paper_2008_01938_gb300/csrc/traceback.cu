@@ -236,6 +236,7 @@ __global__ void __launch_bounds__(kThreads) traceback_kernel(const int16_t* __re
   extern __shared__ __align__(16) uint8_t raw[];
   Smem& sm = *reinterpret_cast<Smem*>(raw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  dpk::launch_dependents();  // the kernel for the small subtrees
   if (tid == 0) {
     sm.nfront[0] = sm.nfront[1] = sm.nlop[0] = sm.nlop[1] = sm.nsmall = 0;
     push(sm, 0, small, 0, n - 1, 0, 0);
@@ -317,6 +318,7 @@ __global__ void __launch_bounds__(32 * kTriWarps) traceback_small_kernel(const i
                                                                          int32_t* status) {
   __shared__ WarpTri tri[kTriWarps];
   const int warp = threadIdx.x >> 5;
+  dpk::grid_dependency_wait();  // the list
   const int total = *count;
   for (int x = blockIdx.x * kTriWarps + warp; x < total; x += gridDim.x * kTriWarps) {
     expand_small(s, n, small[x], tri[warp], steps, status, threadIdx.x & 31);
@@ -344,17 +346,21 @@ extern "C" dp_status mcm_traceback(const int16_t* s, int32_t n, int32_t* steps, 
   if (e != cudaSuccess) return dph::fail_cuda(e, "mcm_traceback: subtree list");
   int32_t* count = reinterpret_cast<int32_t*>(small + n / 2 + 1);
   int32_t* status = status_dev ? status_dev : ds->status;
-  // up to 512 matrices there are at most a few small subtrees for each of the
-  // block's warps, and a second launch costs more than it saves (n = 300: 25
-  // against 20 us); above, they are shared out over the SMs, about a warp each
-  // (2 n / kSmall in a random tree; n = 4000: 57 -> 26 us)
+  // Up to 512 matrices there are at most a few small subtrees for each of the
+  // block's warps, and a second launch costs more than it saves.  Above, they
+  // are shared out over the SMs, about a warp each (2 n / kSmall in a random
+  // tree; n = 4000: 57 -> 23 us), by blocks that are resident before the list is
+  // complete: launched after it, a balanced tree of 600 to 1000 took 14.3 us,
+  // 10.7 like this (a level at a time in one block: 11.3 to 12.4), a random one
+  // of 800 20.3 and 18.0 (19.1).
   const bool one = n <= 512;
   traceback_kernel<<<1, kThreads, sizeof(Smem), st>>>(s, n, steps, small, one ? nullptr : count, status);
-  if (!one) {
-    const int blocks = std::min(2 * ds->sms, n / (8 * kTriWarps) + 1);
-    traceback_small_kernel<<<blocks, 32 * kTriWarps, 0, st>>>(s, n, steps, small, count, status);
-  }
   e = cudaGetLastError();
+  if (!one && e == cudaSuccess) {
+    const int blocks = std::min(2 * ds->sms, n / (8 * kTriWarps) + 1);
+    e = dpk::launch_early(traceback_small_kernel, dim3((unsigned)blocks), 32 * kTriWarps, st, s, n, steps, small, count,
+                          status);
+  }
   cudaError_t e2 = cudaFreeAsync(small, st);
   if (e != cudaSuccess) return dph::fail_cuda(e, "mcm_traceback: launch");
   if (e2 != cudaSuccess) return dph::fail_cuda(e2, "mcm_traceback: release");

@@ -45,6 +45,34 @@ def test_chosen_trees(shape, n):
     assert np.array_equal(got.cpu().numpy(), ref)
 
 
+@pytest.mark.parametrize("n", [512, 513, 4500])
+def test_captured_in_a_graph(n):
+    """The second launch starts before the first has ended: replayed from a
+    graph on other trees, back to back."""
+    import torch
+    import paper_2008_01938_gb300 as dp
+    trees = [_tree(shape, n, n) for shape in ("balanced", "steps", "left", "random")]
+    s = torch.from_numpy(trees[0][0]).cuda()
+    steps = torch.empty((n - 1, 3), dtype=torch.int32, device="cuda")
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        dp.mcm_traceback(s, steps)  # kernels loaded before the capture
+        stream.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            dp.mcm_traceback(s, steps)
+        got = []
+        for tree, _ in trees:
+            s.copy_(torch.from_numpy(tree).cuda())
+            steps.fill_(-1)
+            g.replay()
+            got.append(steps.clone())
+        stream.synchronize()
+    dp.sync_status()
+    for x, (_, ref) in zip(got, trees):
+        assert np.array_equal(x.cpu().numpy(), ref)
+
+
 @pytest.mark.parametrize("n,at", [(20, (3, 9)), (600, (300, 599)), (3000, (0, 2999)), (3000, (1500, 2999))])
 def test_a_split_outside_its_subtree_is_reported(n, at):
     import torch
