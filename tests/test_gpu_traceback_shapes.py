@@ -73,15 +73,39 @@ def test_captured_in_a_graph(n):
         assert np.array_equal(x.cpu().numpy(), ref)
 
 
-@pytest.mark.parametrize("n,at", [(20, (3, 9)), (600, (300, 599)), (3000, (0, 2999)), (3000, (1500, 2999))])
-def test_a_split_outside_its_subtree_is_reported(n, at):
+def _bad(where, i, j):
+    return {"below": i - 1, "last": j, "above": j + 1}[where]
+
+
+# the nodes by their number of matrices, from the root down: the first ones (a
+# path begins after three lopsided ones), one in the middle, the smallest of
+# more than 32 matrices, the largest of at most 32, the smallest of all
+PLACES = ["root", 1, 2, 3, 4, 5, "middle", "last large", "first small", "leaf"]
+
+
+@pytest.mark.parametrize("shape", ["left", "right", "zigzag", "balanced", "steps", "random"])
+@pytest.mark.parametrize("n", [20, 600, 1300, 3000])
+def test_a_split_outside_its_subtree_is_reported(shape, n):
+    """One split of the tree set to i - 1, j or j + 1 at node (i, j): followed
+    by a thread, a warp's and the block's path (at its start, inside it and at
+    its end) and in a subtree expanded whole."""
     import torch
     import paper_2008_01938_gb300 as dp
-    s, ref = _tree("balanced", n, 1)
-    nodes = {(int(i), int(j)) for i, _, j in ref}
-    i, j = at if at in nodes else next(iter(sorted(nodes)))
-    s[i, j] = j
-    dp.mcm_traceback(torch.from_numpy(s).cuda())
-    with pytest.raises(dp.native.DpError) as e:
-        dp.sync_status()
-    assert e.value.code == dp.native.DP_EINVAL
+    s, ref = _tree(shape, n, n)
+    by_size = sorted(((int(j) - int(i) + 1, int(i), int(j)) for i, _, j in ref), reverse=True)
+    large = [x for x in by_size if x[0] > 32]
+    at = {"root": 0, "middle": len(large) // 2, "last large": len(large) - 1, "first small": len(large),
+          "leaf": len(by_size) - 1}
+    good = torch.from_numpy(s).cuda()
+    for rank in sorted({min(max(at.get(p, p), 0), len(by_size) - 1) for p in PLACES}):
+        _, i, j = by_size[rank]
+        for where in ("below", "last", "above"):
+            t = good.clone()
+            t[i, j] = _bad(where, i, j)
+            dp.mcm_traceback(t)
+            with pytest.raises(dp.native.DpError) as e:
+                dp.sync_status()
+            assert e.value.code == dp.native.DP_EINVAL, (i, j, where)
+    got = dp.mcm_traceback(good)
+    dp.sync_status()
+    assert np.array_equal(got.cpu().numpy(), ref)
