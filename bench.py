@@ -137,7 +137,7 @@ def measure_int32_peak(lib, native, stream):
     return rec
 
 
-def _int32_roofline(kernel_ms, evals, probe, clocks=None, name="mcm_main_kernel<int32>"):
+def _int32_roofline(kernel_ms, evals, probe, clocks=None, name="mcm_main_kernel (int32)"):
     achieved = INT_OPS_PER_EVAL * evals / (kernel_ms / 1e3) / 1e12
     lanes = probe["lanes_per_clk_sm"]["add2_both_pipes"]
     roof = {"bound": "alu", "achieved": round(achieved, 3), "peak": round(probe["peak_tops"], 3),
@@ -480,7 +480,7 @@ def bench_interval(dp, native, lib, dev, args):
                         "U[1,4] / U[0,4] seed 5, int32 weights, m and s",
             "split_evals_per_s": EVALS_4096 / (ms / 1e3), "ms_per_solve": ms, "main_kernel_ms": kernel_ms,
             "launches_per_solve": 3,
-            "roofline": _int32_roofline(kernel_ms, EVALS_4096, args.probe, name="mcm_main_kernel<int32, weighted>"),
+            "roofline": _int32_roofline(kernel_ms, EVALS_4096, args.probe, name="mcm_main_kernel (int32, weighted)"),
             "parity_sha256_ok": parity, "l2": "flushed between solves (outside the timed events)"}
 
 
@@ -582,9 +582,9 @@ def bench_batched(dp, native, lib, dev, args):
         rate = probe["bulk_loop_i64_split_evals_per_clk_sm"]
         peak = probe["sms"] * rate * probe["max_sm_clock_mhz"] * 1e6
         roof = {"bound": "alu", "achieved": total / t_graph, "peak": peak, "unit": "split-evals/s (int64)",
-                "frac": round(total / t_graph / peak, 4), "kernel": "mcm_main_kernel<int64> (graph replay)",
+                "frac": round(total / t_graph / peak, 4), "kernel": "mcm64_kernel (graph replay)",
                 "peak_basis": (f"measured: {probe['sms']} SMs x {rate:.2f} int64 split evaluations/clk/SM "
-                               f"(the int64 solver's bulk loop on a staged panel, 2 blocks/SM) x "
+                               f"(the int64 solver's segment loop on a staged panel, 2 blocks/SM) x "
                                f"{probe['max_sm_clock_mhz']:.0f} MHz")}
     return {"workload": "10,000 chains, n log-uniform [8,512], dims U[1,1000] seed 3, int64 costs",
             "roofline": roof,

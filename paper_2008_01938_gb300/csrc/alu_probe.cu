@@ -27,11 +27,13 @@
 //      merge into 64-bit keys); reported as split evaluations per clock per
 //      SM.  This is the
 //      ceiling of the solver's inner loop when nothing waits.
+//   6  the segment loop of the int64 solver, likewise
 #include <cuda_runtime.h>
 
 #include <cstdint>
 
 #include "api_internal.h"
+#include "mcm_tile.cuh"
 
 namespace {
 
@@ -98,7 +100,7 @@ __global__ void __launch_bounds__(kProbeThreads, kBulkBlocksPerSm)
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      P[r][c] = ((seed >> (2 * r + c)) & 1023u) | 1u;  // eight different multipliers, as in a tile
+      P[r][c] = (((seed >> (2 * r + c)) + 37u * tg) & 1023u) | 1u;  // eight multipliers of the thread's own, as in a tile
       best[r][c] = ~0ull;
     }
   __syncthreads();
@@ -147,13 +149,13 @@ __global__ void __launch_bounds__(kProbeThreads, kBulkBlocksPerSm)
   if (x == 0x123456789ull) atomicAdd(&out->sink, 1ull);
 }
 
-// The int64 solver's bulk loop (seg_i64): 64-bit packed (value, k) entries
-// on a shared-memory panel, a 64-bit multiply-add of the weight and a 64-bit
-// minimum per split, 4 x 2 cells per thread, two resident blocks per SM as
-// in the int64 solver.
+// The int64 solver's segment loop (mcm64.cu): 64-bit packed (value, k)
+// entries on a shared-memory panel, a 64-bit multiply-add of the weight and
+// fold64's minimum per split, 4 x 2 cells per thread, two resident blocks per
+// SM as in the int64 solver.
 constexpr int kBulk64BlocksPerSm = 2;
 __global__ void __launch_bounds__(kProbeThreads, kBulk64BlocksPerSm)
-    bulk64_rate_kernel(ProbeOut* out, uint32_t seed, int trips) {
+    bulk64_rate_kernel(ProbeOut* out, uint32_t seed, int trips, uint32_t one) {
   constexpr int T = 32;
   __shared__ __align__(16) unsigned long long A[T * T], B[T * T];
   __shared__ uint32_t PK[T];
@@ -161,7 +163,7 @@ __global__ void __launch_bounds__(kProbeThreads, kBulk64BlocksPerSm)
     A[x] = ((unsigned long long)((seed * (x + 7u)) & 0x7FFFFFu) << 16) | (unsigned)(x & 1023);
     B[x] = ((unsigned long long)((seed * (x + 3u)) & 0x3FFFFFu) << 16);
   }
-  if (threadIdx.x < T) PK[threadIdx.x] = (threadIdx.x % 31u) + 1u;
+  if (threadIdx.x < T) PK[threadIdx.x] = ((threadIdx.x % 31u) + 1u) << 16;
   const int tg = threadIdx.x & 127, ty = tg >> 4, tx = tg & 15;
   uint32_t P[4][2];
   unsigned long long best[4][2];
@@ -169,7 +171,7 @@ __global__ void __launch_bounds__(kProbeThreads, kBulk64BlocksPerSm)
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
-      P[r][c] = (((seed >> (2 * r + c)) & 1023u) | 1u) << 16;
+      P[r][c] = (((seed >> (2 * r + c)) + 37u * tg) & 1023u) | 1u;
       best[r][c] = ~0ull;
     }
   __syncthreads();
@@ -187,13 +189,11 @@ __global__ void __launch_bounds__(kProbeThreads, kBulk64BlocksPerSm)
 #pragma unroll
       for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const unsigned long long cand = (unsigned long long)P[r][c] * pk + av[r] + bv[c];
-          best[r][c] = best[r][c] < cand ? best[r][c] : cand;
-        }
+        for (int c = 0; c < 2; ++c)
+          dpk::fold64(best[r][c], (unsigned long long)P[r][c] * pk + av[r] + bv[c], one);
     }
     // a different panel word each trip, so nothing is loop-invariant
-    if (threadIdx.x == 0) PK[it & 31] += 1u;
+    if (threadIdx.x == 0) PK[it & 31] += 1u << 16;
     __syncthreads();
   }
   const long long t1 = clock64();
@@ -252,7 +252,7 @@ extern "C" dp_status dp_measure_int32_rates(double* out, int32_t nout, void* str
         case 3: int32_rate_kernel<3><<<grid, kProbeThreads, 0, st>>>(d, 0x2545F491u, trips); break;
         case 4: int32_rate_kernel<4><<<grid, kProbeThreads, 0, st>>>(d, 0x2545F491u, trips); break;
         case 5: bulk_rate_kernel<<<grid, kProbeThreads, 0, st>>>(d, 0x2545F491u, trips); break;
-        default: bulk64_rate_kernel<<<grid, kProbeThreads, 0, st>>>(d, 0x2545F491u, trips); break;
+        default: bulk64_rate_kernel<<<grid, kProbeThreads, 0, st>>>(d, 0x2545F491u, trips, 1u); break;
       }
       cudaEventRecord(e1, st);
       if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaEventSynchronize(e1)) != cudaSuccess) {

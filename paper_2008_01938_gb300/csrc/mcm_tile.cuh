@@ -57,12 +57,12 @@ __device__ __forceinline__ void tile_ldp(const uint32_t* p, uint32_t (&v)[8]) {
   v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
 }
 
-// m = min(m, c).  A 64-bit minimum is a
-// compare and a select in two halves each, all on the ALU pipe, which bounds
-// these kernels.  Written as predicated multiply-adds by `one` (1), which the
-// compiler cannot turn back into selects, the halves move on the otherwise
-// idle FMA pipe: 9.65 -> 12.4 split evaluations per clock and SM in a loop of
-// 2 x 2 cells per thread, 13.2 with 4 x 2.
+// m = min(m, c).  A 64-bit minimum is a compare and a select in two halves
+// each, all on the ALU pipe, which bounds these kernels.  Written as
+// predicated multiply-adds by `one` (1), which the compiler cannot turn back
+// into selects, the halves move on the less loaded FMA pipe: the segment loop
+// of 4 x 2 cells per thread 9.74 -> 10.64 split evaluations per clock and SM
+// (alu_probe.cu), batches of chains 4077 -> 3617 us.
 __device__ __forceinline__ void fold64(U64& m, U64 c, uint32_t one) {
   uint32_t ml = (uint32_t)m, mh = (uint32_t)(m >> 32);
   asm("{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
