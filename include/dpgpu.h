@@ -260,13 +260,15 @@ dp_status mcm_plan_destroy(void *plan);
  * table is cut into chunks that run side by side, each starting from a
  * window obtained by products modulo the recurrence's characteristic
  * polynomial.  That path enqueues a few dozen launches and takes a
- * workspace of up to some 30 MB from the stream-ordered allocator (released on the
- * same stream).  Its result is bit-identical.
+ * workspace from the stream-ordered allocator (released on the same stream):
+ * up to 26 MB for a_1 <= 8192, up to 65 MB for the widest windows.  Where that
+ * cannot be had, the table is solved step by step.  The result is
+ * bit-identical either way.
  * With DP_OP_MIN every cell from some position on is the minimum of its
  * residue class of the preset, modulo the gcd of the offsets.  Where the
  * offsets (read on the host) say that this position is near enough, one
  * launch computes the cells before it and writes the others; otherwise long
- * tables are cut into chunks as above. */
+ * tables are cut into chunks as above (with a workspace of a few MB). */
 dp_status sdp_solve(uint32_t *ST, int64_t n, const int32_t *a, int32_t k, dp_op op,
                     int32_t *status_dev, void *stream);
 
@@ -294,7 +296,9 @@ dp_status sdp_plan_destroy(void *plan);
 /* ------------------------------------------------------------------------- */
 
 typedef struct {
-  int64_t hbm_cap_bytes;     /* admission cap on device tables held by the server */
+  int64_t hbm_cap_bytes;     /* admission cap on device tables held by the server and MCM
+                              * workspaces (the workspace of an S-DP solve in chunks, see
+                              * sdp_solve, comes on top, at most one per stream) */
   int32_t max_inflight;      /* maximum requests admitted but not released */
   int32_t num_streams;       /* launch streams used in rotation (>= 1) */
   int32_t max_batch;         /* maximum requests grouped into one launch */

@@ -68,8 +68,10 @@ __global__ void __launch_bounds__(256) ntt_table_kernel(uint32_t* tables) {
   tables[(size_t)(pi * 2 + inverse) * N + at] = below(r, c.p);
 }
 
-// Shared-memory place of word i: a word of padding every 16 keeps the strides
-// of every pass (4096, 256, 16 and 1) free of bank conflicts.
+// Shared-memory place of word i: a word of padding every 16 keeps the passes
+// of strides 16 and 1 free of bank conflicts.  In those of strides 4096 and 256
+// a warp touches 32 neighbouring words, of which the first and the last then
+// share a bank: two wavefronts for what could be one.
 __device__ __forceinline__ int place(int i) { return i + (i >> 4); }
 constexpr int kSmemWords = N + N / 16;
 // Twiddles of the levels up to distance 2048 follow the words in shared memory

@@ -6,9 +6,9 @@
 // Directly that is A^2 multiply-adds each; as cyclic convolutions of length N =
 // 2^14 >= 2A - 1 of the reversed u with z (the outputs wanted, at A - 1 + t, are
 // the ones no wrapped term reaches) it is a transform per row, a point-wise
-// product and an inverse transform per pair, modulo three primes of 30 bits.
+// product and an inverse transform per pair, modulo three primes of 30, 28 and 29 bits.
 // The exact integer sums are below A 2^64 <= 2^77, less than the primes' product
-// 2^85, so Garner's form of the Chinese remainder theorem gives them modulo
+// (above 2^86), so Garner's form of the Chinese remainder theorem gives them modulo
 // 2^32 exactly.  (D. E. Knuth, The Art of Computer Programming 2, 4.3.2 and
 // 4.3.3; products by constants as in V. Shoup's NTL.)
 #pragma once

@@ -130,6 +130,9 @@ int64_t mcm_footprint(int64_t n, int cost) {
   return n * n * (es + 2) + n * n * es * 2 + n * n * 4 + (1 << 20);
 }
 
+// (The workspace of a solve in chunks, which the launch of a group decides on,
+// is outside the cap: it is held while the solve runs, one per stream, and
+// where it cannot be had the table is solved step by step.)
 int64_t sdp_footprint(int64_t n) { return n * 4 + (1 << 16); }
 
 // ---- launch builders (called by the scheduler thread with the lock released) ----
